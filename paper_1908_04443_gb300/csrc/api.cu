@@ -1097,7 +1097,7 @@ struct lbm_batch {
     std::string err;
     double* h_stage = nullptr;         // pinned: per instance the reduction sums and the error word
     double* d_stage = nullptr;         // the same on the device, filled by the reductions, copied at once
-    RedGrid* d_redgrids = nullptr;     // the instances' reduction table (one reduction launch for all)
+    char* d_obstab = nullptr;          // the instances' fields and reduction tables (one launch each for all)
 };
 
 namespace {
@@ -1160,7 +1160,7 @@ void batch_free(lbm_batch* b) {
     if (b->h_stage) cudaFreeHost(b->h_stage);
     b->h_stage = nullptr;
     dfree(b->d_stage, b->stream);
-    dfree(b->d_redgrids, b->stream);
+    dfree(b->d_obstab, b->stream);
     for (lbm_handle* h : b->inst) {
         h->batch_member = false;
         lbm_destroy(h);
@@ -1661,18 +1661,36 @@ lbm_status lbm_batch_observables_fields(lbm_batch* b, lbm_obs* out_n, double* co
     if (!b->h_stage)
         CKB(b, cudaHostAlloc(reinterpret_cast<void**>(&b->h_stage), sizeof(double) * W * n, cudaHostAllocDefault));
     if (!b->d_stage) CKB(b, dmalloc(&b->d_stage, sizeof(double) * W * n, b->stream));
-    if (!b->d_redgrids) CKB(b, dmalloc(&b->d_redgrids, sizeof(RedGrid) * n, b->stream));
-    // every instance's fields pass on the batch's stream, then the reductions of all instances in one
-    // pair of launches, each instance's sums and error word into its slot of one device array, one
-    // copy of the array, then one synchronisation
-    std::vector<RedGrid> tab(n);
-    int total = 0;
+    const size_t tab_bytes = (sizeof(FieldGrid) + sizeof(RedGrid)) * n;
+    if (!b->d_obstab) CKB(b, dmalloc(&b->d_obstab, tab_bytes, b->stream));
+    // the fields pass of all instances in one launch on the batch's stream, then the reductions of all
+    // instances in one pair of launches, each instance's sums and error word into its slot of one device
+    // array, one copy of the array, then one synchronisation
+    std::vector<char> tabs(tab_bytes);
+    FieldGrid* ftab = reinterpret_cast<FieldGrid*>(tabs.data());
+    RedGrid* tab = reinterpret_cast<RedGrid*>(tabs.data() + sizeof(FieldGrid) * n);
+    int total = 0, ftotal = 0;
     for (size_t i = 0; i < n; ++i) {
         lbm_handle* h = b->inst[i];
         lbm_status st = ensure_obs_buffers(h);
         if (st != LBM_OK) return bfail(b, st, "instance " + std::to_string(i) + ": " + h->err);
-        CKB(b, launch_fields(h->lat, h->prec, h->f[h->cur], h->dp, h->d_rho, h->d_u, h->stream));
-        h->launches += 1;
+        FieldGrid& f = ftab[i];
+        f.fin = h->f[h->cur];
+        f.rho = h->d_rho;
+        f.u = h->d_u;
+        f.err = h->d_err;
+        f.type = h->d_type;
+        f.tile_solid = h->d_tile_solid;
+        f.wall_id = h->d_wall_id;
+        f.kappa_w = h->dp.kappa_w;
+        f.kappa = h->dp.kappa;
+        f.nx = h->cfg.nx;
+        f.ny = h->cfg.ny;
+        f.fp = h->dp.fp;
+        f.fs = int(h->dp.fs);
+        f.tile0 = ftotal;
+        f.tx = h->tiles[0];
+        ftotal += h->tiles[0] * h->tiles[1];
         RedGrid& r = tab[i];
         r.rho = h->d_rho;
         r.u = h->d_u;
@@ -1690,9 +1708,12 @@ lbm_status lbm_batch_observables_fields(lbm_batch* b, lbm_obs* out_n, double* co
         total += r.nblk;
     }
     // (from pageable memory: staged before the call returns)
-    CKB(b, cudaMemcpyAsync(b->d_redgrids, tab.data(), sizeof(RedGrid) * n, cudaMemcpyHostToDevice, b->stream));
-    CKB(b, launch_reduce_grids(b->inst[0]->D, b->d_redgrids, int(n), total, b->stream));
-    b->inst[0]->launches += 2;
+    CKB(b, cudaMemcpyAsync(b->d_obstab, tabs.data(), tab_bytes, cudaMemcpyHostToDevice, b->stream));
+    CKB(b, launch_fields_grids(b->prec, reinterpret_cast<const FieldGrid*>(b->d_obstab), int(n), ftotal, b->phys,
+                               b->stream));
+    CKB(b, launch_reduce_grids(b->inst[0]->D, reinterpret_cast<const RedGrid*>(b->d_obstab + sizeof(FieldGrid) * n),
+                               int(n), total, b->stream));
+    b->inst[0]->launches += 3;
     for (size_t i = 0; i < n; ++i) {
         lbm_handle* h = b->inst[i];
         if (rho_hosts && rho_hosts[i])

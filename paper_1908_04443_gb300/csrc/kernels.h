@@ -96,6 +96,20 @@ cudaError_t launch_step(int lat, int prec, const void* fin, void* fout, const De
 // buffers; either may be null.
 cudaError_t launch_fields(int lat, int prec, const void* fin, const DevParams& p, double* rho, double* u,
                           cudaStream_t s);
+// The fields of several D2Q9 grids of one physics in one launch: grid k owns the tiles
+// [g[k].tile0, g[k].tile0 + its tile count) of the launch (step_tile_shape tiles, x fastest).
+struct FieldGrid {
+    const void* fin;           // stored state
+    double *rho, *u;           // N and 2 N doubles
+    unsigned* err;             // the grid's error word
+    const uint8_t *type, *tile_solid;
+    const int* wall_id;
+    const double* kappa_w;     // per wall node or null
+    double kappa;
+    int nx, ny, fp, fs, tile0, tx;   // tx: tiles per row
+};
+cudaError_t launch_fields_grids(int prec, const FieldGrid* grids, int ngrids, int total_tiles, const DevParams& phys,
+                                cudaStream_t s);
 // f* such that the next pull yields f^eq(rho0, u0) (rho0: N doubles, u0: d*N doubles or null).
 cudaError_t launch_init(int lat, int prec, void* fout, const DevParams& p, const double* rho0, const double* u0,
                         cudaStream_t s);

@@ -479,6 +479,38 @@ __global__ void __launch_bounds__(TileShape<L, S>::X* TileShape<L, S>::Y* TileSh
                                                                rho_out, u_out, sm);
 }
 
+// The fields pass of several grids (a batch's observables) in one launch.  A launch per grid leaves
+// most of the chip idle: a grid of 600 x 400 is 950 tiles, 1.6 waves of 4 CTAs per SM, and its tail and
+// start-up are most of its 8.6 us.  24 such grids: 206 us one by one, 113 us together.
+template <class S>
+__global__ void __launch_bounds__(TileShape<D2Q9, S>::X* TileShape<D2Q9, S>::Y, TileShape<D2Q9, S>::MINB)
+    fields_grids(const FieldGrid* __restrict__ tab, int n, Phys<S> ph) {
+    using TS = TileShape<D2Q9, S>;
+    __shared__ TileSmem<D2Q9, S, TS::X, TS::Y, 1> sm;
+    const int k = grid_of_tile(tab, n);
+    const FieldGrid& q = tab[k];
+    Geo g;
+    g.nx = q.nx;
+    g.ny = q.ny;
+    g.nz = 1;
+    g.N = q.nx * q.ny;
+    g.fp = q.fp;
+    g.fs = q.fs;
+    g.type = q.type;
+    g.tile_solid = nullptr;
+    g.wall_id = q.wall_id;
+    g.kappa_w = q.kappa_w;
+    g.kappa = q.kappa;
+    const int tile = int(blockIdx.x) - q.tile0, ty = tile / q.tx, tx = tile - ty * q.tx;
+    const S* fin = static_cast<const S*>(q.fin);
+    if (q.tile_solid[tile])
+        tile_body_w<D2Q9, S, S, TS::X, TS::Y, 1, 1, true>(fin, nullptr, g, ph, tx * TS::X, ty * TS::Y, 0, true, q.err,
+                                                          q.rho, q.u, sm);
+    else
+        tile_body_w<D2Q9, S, S, TS::X, TS::Y, 1, 1, false>(fin, nullptr, g, ph, tx * TS::X, ty * TS::Y, 0, false,
+                                                           q.err, q.rho, q.u, sm);
+}
+
 // Adjoint local part (D2Q9): the forward tile machinery recomputes rho, psi and rho_w of the state
 // pulled from f*_k, then each node writes the reverse of its collision and its psi data.
 template <class S>
@@ -738,6 +770,21 @@ cudaError_t launch_step(int lat, int prec, const void* fin, void* fout, const De
 cudaError_t launch_fields(int lat, int prec, const void* fin, const DevParams& p, double* rho, double* u,
                           cudaStream_t s) {
     return dispatch<1>(lat, prec, fin, nullptr, p, rho, u, s);
+}
+
+template <class S>
+static cudaError_t fields_grids_t(const FieldGrid* grids, int ngrids, int total_tiles, const DevParams& p,
+                                  cudaStream_t s) {
+    using TS = TileShape<D2Q9, S>;
+    fields_grids<S><<<total_tiles, dim3(TS::X, TS::Y, 1), 0, s>>>(grids, ngrids, make_phys<S>(p));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fields_grids(int prec, const FieldGrid* grids, int ngrids, int total_tiles, const DevParams& p,
+                                cudaStream_t s) {
+    if (ngrids < 1 || total_tiles < 1) return cudaSuccess;
+    return prec == PREC_FP64 ? fields_grids_t<double>(grids, ngrids, total_tiles, p, s)
+                             : fields_grids_t<float>(grids, ngrids, total_tiles, p, s);
 }
 
 template <class L, class S>

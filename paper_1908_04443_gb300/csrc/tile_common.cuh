@@ -205,6 +205,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, unsign
     return false;
 }
 
+// The grid whose tiles hold this CTA's: the last with tile0 <= blockIdx.x (tile0 ascends from 0).  Every
+// warp counts them, 32 table entries per load.
+__device__ __forceinline__ int grid_of_tile(const FieldGrid* tab, int n) {
+    const int lane = (threadIdx.x + blockDim.x * threadIdx.y) & 31;
+    int k = -1;
+    for (int base = 0; base < n; base += 32)
+        k += __popc(__ballot_sync(0xffffffffu, base + lane < n && tab[base + lane].tile0 <= int(blockIdx.x)));
+    return k;
+}
+
 __device__ __forceinline__ int wrap_full(int v, int n) {
     v %= n;
     return v < 0 ? v + n : v;
