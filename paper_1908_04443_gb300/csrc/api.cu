@@ -502,6 +502,30 @@ lbm_status validate_config(const lbm_config& c, const double* kappa_per_wall) {
     return LBM_OK;
 }
 
+int device_sms() {
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
+// Solid flags of a w x th tiling of a D2Q9 grid from those of its step_tile_shape tiles: a tile is
+// flagged where any of those that it overlaps is (their cells + 3-node halos cover its own).
+std::vector<uint8_t> merged_flags(const lbm_handle* h, int w, int th) {
+    const int nx = h->cfg.nx, ny = h->cfg.ny, bw = h->int_tile[0], bh = h->int_tile[1];
+    const int tx = (nx + w - 1) / w, ty = (ny + th - 1) / th;
+    std::vector<uint8_t> out((size_t)tx * ty, 0);
+    for (int y = 0; y < ty; ++y)
+        for (int x = 0; x < tx; ++x) {
+            const int x1 = std::min((x + 1) * w, nx) - 1, y1 = std::min((y + 1) * th, ny) - 1;
+            uint8_t any = 0;
+            for (int j = y * th / bh; j <= y1 / bh; ++j)
+                for (int i = x * w / bw; i <= x1 / bw; ++i) any |= h->tile_solid[(size_t)j * h->tiles[0] + i];
+            out[(size_t)y * tx + x] = any;
+        }
+    return out;
+}
+
 // The mask scan for a validated configuration: the step kernels' tile shape and, for D2Q9 in FP32,
 // the pair kernel's.
 void scan_for(const lbm_config& c, const uint8_t* solid_mask, int threads, MaskScan* out) {
@@ -598,8 +622,16 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
     CKI(guarded_malloc(&h->f[0], h->fbytes, h->stream), "cudaMalloc f");
     CKI(guarded_malloc(&h->f[1], h->fbytes, h->stream), "cudaMalloc f");
     CKI(dmalloc(&h->d_type, N, h->stream), "cudaMalloc type");
-    CKI(dmalloc(&h->d_tile_solid, h->tile_solid.size(), h->stream), "cudaMalloc tile flags");
-    CKI(cudaMemcpyAsync(h->d_tile_solid, h->tile_solid.data(), h->tile_solid.size(), cudaMemcpyHostToDevice, h->stream),
+    // (D2Q9 FP64: followed by the flags of the grid's FP64 tiles)
+    std::vector<uint8_t> flags = h->tile_solid;
+    int fw = 0, fh = 0;
+    if (h->D == 2 && h->prec == LBM_FP64) {
+        d2q9_fp64_tile(&nx, &ny, 1, device_sms(), &fw, &fh);
+        const std::vector<uint8_t> own = merged_flags(h, fw, fh);
+        flags.insert(flags.end(), own.begin(), own.end());
+    }
+    CKI(dmalloc(&h->d_tile_solid, flags.size(), h->stream), "cudaMalloc tile flags");
+    CKI(cudaMemcpyAsync(h->d_tile_solid, flags.data(), flags.size(), cudaMemcpyHostToDevice, h->stream),
         "copy tile flags");
     CKI(dmalloc(&h->d_wall_id, sizeof(int) * N, h->stream), "cudaMalloc wall_id");
     CKI(dmalloc(&h->d_err, sizeof(unsigned), h->stream), "cudaMalloc err");
@@ -687,6 +719,9 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
     p.wall_id = h->d_wall_id;
     p.type = h->d_type;
     p.tile_solid = h->d_tile_solid;
+    p.tile_w = fw;
+    p.tile_h = fh;
+    if (fw > 0) p.pair_solid = h->d_tile_solid + h->tile_solid.size();
     p.err = h->d_err;
     // D3Q19 FP32 step kernel and the tensor maps of the TMA-staged z-march
     p.step3 = c.step_kernel == LBM_KERNEL_PAIR ? 1 : (c.step_kernel == LBM_KERNEL_TILE ? 2 : 0);
@@ -738,9 +773,7 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
     if (h->D == 2) {
         h->mask.assign(solid_mask, solid_mask + N);
         if (c.step_kernel == LBM_KERNEL_YMARCH) {
-            int dev = 0, sms = 1;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            const int sms = device_sms();
             YGrid grid{nx, ny, h->mask.data(), BatchItem{}};
             grid.proto.f[0] = h->f[0];
             grid.proto.f[1] = h->f[1];
@@ -1021,7 +1054,7 @@ int32_t lbm_step_kernel_used(const lbm_handle* h) {
         return h->dp.step3 == 0 && h->dp.ztmap ? LBM_KERNEL_ZTMA : LBM_KERNEL_PAIR;
     }
     if (h->ymarch) return LBM_KERNEL_YMARCH;
-    return h->dp.pair_solid ? LBM_KERNEL_PAIR : LBM_KERNEL_TILE;
+    return h->prec == LBM_FP32_DEV && h->dp.pair_solid ? LBM_KERNEL_PAIR : LBM_KERNEL_TILE;
 }
 
 void lbm_destroy(lbm_handle* h) {
@@ -1074,6 +1107,7 @@ struct BatchGroup {
     int* d_begin = nullptr;            // y-march: per-CTA ranges of d_items
     unsigned* d_sched = nullptr;       // pair kernel: tile-claim counters (zero between launches)
     int n_items = 0, ctas = 1;
+    int tw = 0, th = 0;                // FP64 tile kernel: the tile shape of its items
     cudaStream_t side = nullptr;       // its branch of the captured steps (batches of several groups)
     cudaEvent_t done = nullptr;
 };
@@ -1196,13 +1230,24 @@ cudaError_t group_build(lbm_batch* b, BatchGroup& g) {
         begin = std::move(plan.begin);
         g.ctas = plan.ctas;
     } else {
-        const bool pair = g.kind == LBM_KERNEL_PAIR;
+        const bool pair = g.kind == LBM_KERNEL_PAIR, fp64 = b->prec == LBM_FP64;
         int tx, ty, tz;
         step_tile_shape(b->lat, b->prec, &tx, &ty, &tz);
         if (pair) pair_tile_shape(&tx, &ty);
+        if (fp64) {   // one shape for the group's grids together
+            std::vector<int> gx, gy;
+            for (int i : g.members) {
+                gx.push_back(b->inst[i]->cfg.nx);
+                gy.push_back(b->inst[i]->cfg.ny);
+            }
+            d2q9_fp64_tile(gx.data(), gy.data(), int(gx.size()), b->sms, &tx, &ty);
+            g.tw = tx;
+            g.th = ty;
+        }
         for (int i : g.members) {
             lbm_handle* h = b->inst[i];
             const int nx = h->cfg.nx, ny = h->cfg.ny;
+            const std::vector<uint8_t> own = fp64 ? merged_flags(h, tx, ty) : std::vector<uint8_t>();
             for (int y = 0; y < ny; y += ty)
                 for (int x = 0; x < nx; x += tx) {
                     const size_t t = (size_t)(y / ty) * ((nx + tx - 1) / tx) + x / tx;
@@ -1215,7 +1260,7 @@ cudaError_t group_build(lbm_batch* b, BatchGroup& g) {
                     it.x0 = x;
                     it.y0 = y;
                     it.y1 = std::min(y + ty, ny);
-                    it.solid = int(pair ? h->pair_solid[t] : h->tile_solid[t]);
+                    it.solid = int(pair ? h->pair_solid[t] : (fp64 ? own[t] : h->tile_solid[t]));
                     it.inst = i;
                     it.f[0] = h->f[0];
                     it.f[1] = h->f[1];
@@ -1228,7 +1273,7 @@ cudaError_t group_build(lbm_batch* b, BatchGroup& g) {
                     items.push_back(it);
                 }
         }
-        const int max_per_sm = pair ? pair_ctas_per_sm() : batched_ctas_per_sm(b->lat, b->prec);
+        const int max_per_sm = pair ? pair_ctas_per_sm() : batched_ctas_per_sm();
         const int per_sm = g.ctas_per_sm > 0 && g.ctas_per_sm < max_per_sm ? g.ctas_per_sm : max_per_sm;
         const long long cap = (long long)b->sms * per_sm;
         g.ctas = int((long long)items.size() < cap ? (long long)items.size() : cap);
@@ -1249,7 +1294,8 @@ cudaError_t group_build(lbm_batch* b, BatchGroup& g) {
 cudaError_t group_launch(lbm_batch* b, const BatchGroup& g, cudaStream_t s, int parity) {
     if (g.kind == LBM_KERNEL_YMARCH) return launch_ymarch(b->prec, parity, b->phys, g.d_items, g.d_begin, g.ctas, s);
     if (g.kind == LBM_KERNEL_PAIR) return launch_pair_batched(parity, b->phys, g.d_items, g.n_items, g.ctas, g.d_sched, s);
-    return launch_step_batched(b->lat, b->prec, parity, b->phys, b->d_insts, g.d_items, g.n_items, g.ctas, s);
+    if (b->prec == LBM_FP64) return launch_d2q9_fp64_batched(parity, b->phys, g.d_items, g.n_items, g.tw, g.th, s);
+    return launch_step_batched(parity, b->phys, b->d_insts, g.d_items, g.n_items, g.ctas, s);
 }
 
 // One time step of every group: in sequence on s, or (fork) as parallel branches joined back into s
@@ -1680,7 +1726,8 @@ lbm_status lbm_batch_observables_fields(lbm_batch* b, lbm_obs* out_n, double* co
         f.u = h->d_u;
         f.err = h->d_err;
         f.type = h->d_type;
-        f.tile_solid = h->d_tile_solid;
+        const bool fp64 = b->prec == LBM_FP64;
+        f.tile_solid = fp64 ? h->dp.pair_solid : h->d_tile_solid;
         f.wall_id = h->d_wall_id;
         f.kappa_w = h->dp.kappa_w;
         f.kappa = h->dp.kappa;
@@ -1689,8 +1736,10 @@ lbm_status lbm_batch_observables_fields(lbm_batch* b, lbm_obs* out_n, double* co
         f.fp = h->dp.fp;
         f.fs = int(h->dp.fs);
         f.tile0 = ftotal;
-        f.tx = h->tiles[0];
-        ftotal += h->tiles[0] * h->tiles[1];
+        f.tw = fp64 ? h->dp.tile_w : h->int_tile[0];
+        f.th = fp64 ? h->dp.tile_h : h->int_tile[1];
+        f.tx = (f.nx + f.tw - 1) / f.tw;
+        ftotal += f.tx * ((f.ny + f.th - 1) / f.th);
         RedGrid& r = tab[i];
         r.rho = h->d_rho;
         r.u = h->d_u;

@@ -32,7 +32,10 @@ struct DevParams {
     const int* wall_id;          // per node: index into kappa_w (valid at wall nodes)
     const uint8_t* type;         // per node: T_SOLID | T_WALL | T_NEARWALL | T_BULK
     const uint8_t* tile_solid;   // per tile of the step kernel's grid: a solid node within the tile + 3-node halo
-    const uint8_t* pair_solid;   // the same per tile of the FP32 pair kernel; null: FP32 steps use the tile kernel
+    // the same per tile of the FP32 pair kernel (null: FP32 steps use the tile kernel) or, in FP64, of the
+    // grid's FP64 tiles (tile_w x tile_h nodes)
+    const uint8_t* pair_solid;
+    int tile_w, tile_h;
     // D3Q19 FP32 step kernel: 0 the TMA-staged z-march, 1 the z-pair march, 2 the scalar z-march
     int step3;
     const void* ztmap;           // TMA tensor maps of the two 3D FP32 distribution buffers (device, 2 x 128 B)
@@ -97,7 +100,8 @@ cudaError_t launch_step(int lat, int prec, const void* fin, void* fout, const De
 cudaError_t launch_fields(int lat, int prec, const void* fin, const DevParams& p, double* rho, double* u,
                           cudaStream_t s);
 // The fields of several D2Q9 grids of one physics in one launch: grid k owns the tiles
-// [g[k].tile0, g[k].tile0 + its tile count) of the launch (step_tile_shape tiles, x fastest).
+// [g[k].tile0, g[k].tile0 + its tile count) of the launch (x fastest): step_tile_shape tiles in FP32, the
+// grid's own FP64 tiles in FP64.
 struct FieldGrid {
     const void* fin;           // stored state
     double *rho, *u;           // N and 2 N doubles
@@ -107,6 +111,7 @@ struct FieldGrid {
     const double* kappa_w;     // per wall node or null
     double kappa;
     int nx, ny, fp, fs, tile0, tx;   // tx: tiles per row
+    int tw, th;                      // FP64: the grid's tile shape
 };
 cudaError_t launch_fields_grids(int prec, const FieldGrid* grids, int ngrids, int total_tiles, const DevParams& phys,
                                 cudaStream_t s);
@@ -117,10 +122,10 @@ cudaError_t launch_init(int lat, int prec, void* fout, const DevParams& p, const
 cudaError_t launch_get_state(int lat, int prec, const void* fin, const DevParams& p, double* fpost, cudaStream_t s);
 // Stored state from post-streaming doubles [q][N].
 cudaError_t launch_set_state(int lat, int prec, void* fout, const DevParams& p, const double* fpost, cudaStream_t s);
-// Batched step: a persistent grid of `ctas` CTAs walks the work list (instance, tile) of every
+// Batched D2Q9 FP32 step with the tile kernel: a persistent grid of `ctas` CTAs walks the work list (instance, tile) of every
 // instance of the batch; each instance reads f[parity] and writes f[parity ^ 1].
-cudaError_t launch_step_batched(int lat, int prec, int parity, const DevParams& phys, const BatchInstance* insts,
-                                const BatchItem* items, int n_items, int ctas, cudaStream_t s);
+cudaError_t launch_step_batched(int parity, const DevParams& phys, const BatchInstance* insts, const BatchItem* items,
+                                int n_items, int ctas, cudaStream_t s);
 // D2Q9 FP32 step with two nodes per thread (packed FP32x2 arithmetic) on 32 x 16 tiles: one
 // grid (tile flags p.pair_solid) or a persistent grid of `ctas` CTAs walking (instance, tile) items,
 // claimed dynamically through `sched` (two device counters, zero before the first launch; the
@@ -129,6 +134,16 @@ cudaError_t launch_pair_step(const void* fin, void* fout, const DevParams& p, cu
 cudaError_t launch_pair_batched(int parity, const DevParams& phys, const BatchItem* items, int n_items, int ctas,
                                 unsigned* sched, cudaStream_t s);
 void pair_tile_shape(int* tx, int* ty);
+// D2Q9 FP64: the step (mode 0, into fout) or the fields (mode 1, into rho and u) of one grid on tiles of
+// p.tile_w x p.tile_h nodes with the flags p.pair_solid; the step of a batch's (instance, tile) items; the
+// fields of several grids; and the tile shape for `ngrids` grids on `sms` SMs.
+cudaError_t launch_d2q9_fp64(int mode, const void* fin, void* fout, const DevParams& p, double* rho, double* u,
+                             cudaStream_t s);
+cudaError_t launch_d2q9_fp64_batched(int parity, const DevParams& phys, const BatchItem* items, int n_items, int tw,
+                                     int th, cudaStream_t s);
+cudaError_t launch_d2q9_fp64_fields(const FieldGrid* grids, int ngrids, int total_tiles, const DevParams& phys,
+                                    cudaStream_t s);
+void d2q9_fp64_tile(const int* nx, const int* ny, int ngrids, int sms, int* tw, int* th);
 // Measured FP64 fused multiply-add rate of the device (GFLOP/s, best of three timed launches of
 // independent FMA chains after one warm-up); synchronises the stream.
 cudaError_t probe_fp64_rate(cudaStream_t s, double* gflops);
@@ -167,7 +182,7 @@ void ztma_box_dims(int* bx, int* by);
 std::vector<ZItem> ztma_work_list(const uint8_t* mask, int nx, int ny, int nz);
 // Tile shape (x, y, z) of the step kernels and the resident CTAs per SM of the batched kernel.
 void step_tile_shape(int lat, int prec, int* tx, int* ty, int* tz);
-int batched_ctas_per_sm(int lat, int prec);
+int batched_ctas_per_sm();
 // Node-type flags from the solid mask: T_SOLID, T_WALL (solid with a fluid lattice neighbour),
 // T_NEARWALL (within Euclidean distance 3 of a solid node) and T_BULK (fluid with every lattice
 // neighbour fluid).

@@ -481,11 +481,11 @@ __global__ void __launch_bounds__(TileShape<L, S>::X* TileShape<L, S>::Y* TileSh
 
 // The fields pass of several grids (a batch's observables) in one launch.  A launch per grid leaves
 // most of the chip idle: a grid of 600 x 400 is 950 tiles, 1.6 waves of 4 CTAs per SM, and its tail and
-// start-up are most of its 8.6 us.  24 such grids: 206 us one by one, 113 us together.
-template <class S>
-__global__ void __launch_bounds__(TileShape<D2Q9, S>::X* TileShape<D2Q9, S>::Y, TileShape<D2Q9, S>::MINB)
-    fields_grids(const FieldGrid* __restrict__ tab, int n, Phys<S> ph) {
-    using TS = TileShape<D2Q9, S>;
+// start-up are most of its 8.6 us.  24 such grids: 206 us one by one, 59 us together.
+__global__ void __launch_bounds__(TileShape<D2Q9, float>::X* TileShape<D2Q9, float>::Y, TileShape<D2Q9, float>::MINB)
+    fields_grids(const FieldGrid* __restrict__ tab, int n, Phys<float> ph) {
+    using S = float;
+    using TS = TileShape<D2Q9, float>;
     __shared__ TileSmem<D2Q9, S, TS::X, TS::Y, 1> sm;
     const int k = grid_of_tile(tab, n);
     const FieldGrid& q = tab[k];
@@ -756,7 +756,7 @@ template <int MODE>
 static cudaError_t dispatch(int lat, int prec, const void* fin, void* fout, const DevParams& p, double* rho, double* u,
                             cudaStream_t s) {
     if (lat == LAT_D2Q9) {
-        if (prec == PREC_FP64) return launch_tile<D2Q9, double, MODE>(fin, fout, p, rho, u, s);
+        if (prec == PREC_FP64) return launch_d2q9_fp64(MODE, fin, fout, p, rho, u, s);
         return launch_tile<D2Q9, float, MODE>(fin, fout, p, rho, u, s);
     }
     return launch_step3d(prec, MODE, fin, fout, geo_of(p), p, rho, u, s);
@@ -772,37 +772,21 @@ cudaError_t launch_fields(int lat, int prec, const void* fin, const DevParams& p
     return dispatch<1>(lat, prec, fin, nullptr, p, rho, u, s);
 }
 
-template <class S>
-static cudaError_t fields_grids_t(const FieldGrid* grids, int ngrids, int total_tiles, const DevParams& p,
-                                  cudaStream_t s) {
-    using TS = TileShape<D2Q9, S>;
-    fields_grids<S><<<total_tiles, dim3(TS::X, TS::Y, 1), 0, s>>>(grids, ngrids, make_phys<S>(p));
-    return cudaGetLastError();
-}
-
 cudaError_t launch_fields_grids(int prec, const FieldGrid* grids, int ngrids, int total_tiles, const DevParams& p,
                                 cudaStream_t s) {
+    if (prec == PREC_FP64) return launch_d2q9_fp64_fields(grids, ngrids, total_tiles, p, s);
     if (ngrids < 1 || total_tiles < 1) return cudaSuccess;
-    return prec == PREC_FP64 ? fields_grids_t<double>(grids, ngrids, total_tiles, p, s)
-                             : fields_grids_t<float>(grids, ngrids, total_tiles, p, s);
-}
-
-template <class L, class S>
-static cudaError_t batched_l(int parity, const DevParams& p, const BatchInstance* insts, const BatchItem* items,
-                             int n_items, int ctas, cudaStream_t s) {
-    using TS = TileShape<L, S>;
-    dim3 block(TS::X, TS::Y, TS::Z);
-    fused_step_batched<L, S, S><<<ctas, block, 0, s>>>(parity, insts, items, n_items, make_phys<S>(p), p.err);
+    using TS = TileShape<D2Q9, float>;
+    fields_grids<<<total_tiles, dim3(TS::X, TS::Y, 1), 0, s>>>(grids, ngrids, make_phys<float>(p));
     return cudaGetLastError();
 }
 
-cudaError_t launch_step_batched(int lat, int prec, int parity, const DevParams& p, const BatchInstance* insts,
-                                const BatchItem* items, int n_items, int ctas, cudaStream_t s) {
-    if (lat == LAT_D2Q9) {
-        if (prec == PREC_FP64) return batched_l<D2Q9, double>(parity, p, insts, items, n_items, ctas, s);
-        return batched_l<D2Q9, float>(parity, p, insts, items, n_items, ctas, s);
-    }
-    return cudaErrorInvalidValue;   // batches are D2Q9
+cudaError_t launch_step_batched(int parity, const DevParams& p, const BatchInstance* insts, const BatchItem* items,
+                                int n_items, int ctas, cudaStream_t s) {
+    using TS = TileShape<D2Q9, float>;
+    fused_step_batched<D2Q9, float, float><<<ctas, dim3(TS::X, TS::Y, TS::Z), 0, s>>>(parity, insts, items, n_items,
+                                                                                      make_phys<float>(p), p.err);
+    return cudaGetLastError();
 }
 
 template <class S>
@@ -838,19 +822,13 @@ void step_tile_shape(int lat, int prec, int* tx, int* ty, int* tz) {
     }
 }
 
-template <class L, class S>
-static int occ() {
-    using TS = TileShape<L, S>;
+int batched_ctas_per_sm() {
+    using TS = TileShape<D2Q9, float>;
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fused_step_batched<L, S, S>, TS::X * TS::Y * TS::Z, 0) !=
-        cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fused_step_batched<D2Q9, float, float>,
+                                                      TS::X * TS::Y * TS::Z, 0) != cudaSuccess)
         n = 1;
     return n < 1 ? 1 : n;
-}
-
-int batched_ctas_per_sm(int lat, int prec) {
-    (void)lat;
-    return prec == PREC_FP64 ? occ<D2Q9, double>() : occ<D2Q9, float>();
 }
 
 static unsigned grid_for(long long n) {

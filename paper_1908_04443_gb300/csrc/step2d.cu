@@ -16,7 +16,9 @@
 // node types 8.  Persistent CTAs walk a host-planned list of runs (the planner balances the rows
 // per CTA).
 #include <cmath>
+#include <type_traits>
 
+#include "fp64.cuh"
 #include "kernels.h"
 #include "lattice.cuh"
 #include "tile_common.cuh"
@@ -41,6 +43,10 @@ struct YSmem {
     C psi[8][TW];
     uint8_t type[8][TW + 8];  // cell hx at index hx + 1 (x = x0 + index - 3)
 };
+
+// psi as the tile kernel of the same precision computes it (the two kernels agree bit for bit)
+__device__ __forceinline__ float psi_y(float rho, const Phys<float>& e, unsigned* err) { return psi_checked(rho, e, err); }
+__device__ __forceinline__ double psi_y(double rho, const Phys<double>& e, unsigned* err) { return psi64(rho, e, err); }
 
 // One run: columns x0 .. x0 + TW - 5 (those below nx), rows yb .. ye - 1.
 template <class S, bool SOLID>
@@ -112,12 +118,20 @@ __device__ __forceinline__ void ymarch_run(const S* __restrict__ fin, S* __restr
         if constexpr (SOLID) t = sm.type[yl & 7][ti];
         if (active && !(t & T_SOLID)) {
             const S* fr = &sm.f[yl & 3][0][hx];
-            C drho = C(0);
+            C rho;
+            if constexpr (std::is_same_v<C, double>) {
+                C v[Q];
 #pragma unroll
-            for (int a = 0; a < Q; ++a) drho += C(fr[a * TW]);
-            const C rho = ph.rho_ref + drho;
+                for (int a = 0; a < Q; ++a) v[a] = fr[a * TW];
+                rho = density64(v);
+            } else {
+                C drho = C(0);
+#pragma unroll
+                for (int a = 0; a < Q; ++a) drho += C(fr[a * TW]);
+                rho = ph.rho_ref + drho;
+            }
             if constexpr (SOLID) sm.rho[yl & 3][hx] = rho;
-            sm.psi[yl & 7][hx] = psi_checked(rho, ph, err);
+            sm.psi[yl & 7][hx] = psi_y(rho, ph, err);
         } else if (active) {
             sm.psi[yl & 7][hx] = C(0);   // a solid cell: wall cells get their psi in phase B (not with SF)
         }
@@ -164,7 +178,7 @@ __device__ __forceinline__ void ymarch_run(const S* __restrict__ fin, S* __restr
                             rw = rw < ph.rho_g ? ph.rho_g : rw;
                         }
                     }
-                    sm.psi[yw & 7][hx] = psi_checked(rw, ph, err);
+                    sm.psi[yw & 7][hx] = psi_y(rw, ph, err);
                 }
                 __syncthreads();
             }
@@ -181,6 +195,32 @@ __device__ __forceinline__ void ymarch_run(const S* __restrict__ fin, S* __restr
 #pragma unroll
             for (int a = 0; a < Q; ++a) f[a] = C(fr[a * TW]);
             const C psi_c = sm.psi[yc & 7][hx];
+            if constexpr (std::is_same_v<C, double>) {
+                auto diff = [&](int ex, int ey) {
+                    return dsub(sm.psi[(yc + ey) & 7][hx + ex], sm.psi[(yc - ey) & 7][hx - ex]);
+                };
+                const bool sf = SOLID && ph.wall_kind == 2 && !(sm.type[yc & 7][ti] & T_BULK);
+                C ax = C(0), ay = C(0);
+                if (sf) {
+#pragma unroll
+                    for (int a = 1; a < Q; ++a) {
+                        const int ex = L::ex(a), ey = L::ey(a);
+                        if (sm.type[(yc + ey) & 7][ti + ex] & T_SOLID) {
+                            if (ex) ax += C(L::wf(a) * ex);
+                            if (ey) ay += C(L::wf(a) * ey);
+                        }
+                    }
+                }
+                const C rho = density64(f);
+                if (!(rho > C(0))) atomicOr(err, ERR_RHO);
+                C ux, uy;
+                node2d64<true>(f, rho, diff(1, 0), diff(0, 1), diff(1, 1), diff(-1, 1), psi_c, sf, ax, ay, ph, ux, uy);
+                const int fi = yc * fp + gx;
+#pragma unroll
+                for (int a = 0; a < Q; ++a) fout[a * fs + fi] = f[a];
+                load_types(yl + 3);
+                continue;
+            }
             // sum_a w_a psi(x + e_a) e_a, taken over opposite pairs: w_a e_a (psi(x + e_a) - psi(x - e_a))
             C sx = C(0), sy = C(0);
 #pragma unroll

@@ -130,19 +130,6 @@ struct PairSmem {
     int nwall;
 };
 
-// The grid of a single-grid launch (kernel parameters); a batch passes its work record (shared
-// memory) with the same member names.  Members are read where they are used, so that nothing of
-// the grid needs a register across the tile's barriers.
-struct PairGrid {
-    int nx, ny, N;
-    int fp, fs;   // distribution row pitch and direction stride
-    const uint8_t* type;
-    const int* wall_id;
-    const double* kappa_w;
-    double kappa;
-    const void* f[2];
-};
-
 // One 32 x 16 tile with first node (x0, y0), reading g.f[parity] and writing g.f[parity ^ 1].
 // SOLID = false: no solid node within the tile + 3-node halo.  WRAP as in the scalar tile kernel:
 // 0 no periodic wrap, 1 a single wrap, 2 full modulo.
@@ -666,18 +653,7 @@ int pair_ctas_per_sm() {
 }
 
 cudaError_t launch_pair_step(const void* fin, void* fout, const DevParams& p, cudaStream_t s) {
-    PairGrid g;
-    g.nx = p.nx;
-    g.ny = p.ny;
-    g.N = int(p.N);
-    g.fp = p.fp;
-    g.fs = int(p.fs);
-    g.type = p.type;
-    g.wall_id = p.wall_id;
-    g.kappa_w = p.kappa_w;
-    g.kappa = p.kappa;
-    g.f[0] = fin;
-    g.f[1] = fout;
+    const PairGrid g = pair_grid(fin, fout, p);
     dim3 grid((p.nx + PTX - 1) / PTX, (p.ny + PNY - 1) / PNY, 1);
     pair_step<<<grid, dim3(PTX, PTY, 1), 0, s>>>(g, p.pair_solid, make_phys<float>(p), make_pair_rates(p), p.err);
     return cudaGetLastError();

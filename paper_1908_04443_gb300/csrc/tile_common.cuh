@@ -9,6 +9,41 @@
 
 namespace lbmwet {
 
+// Constants of the FP64 kernels (fp64.cuh), folded on the host; the other precisions have none.
+template <class C>
+struct Fold {};
+template <>
+struct Fold<double> {
+    double kRT, ka, kaphi, k3;     // 2/G times R T, a, a phi(T), 1/3
+    double g1, g2;                 // -G times the D2Q9 weights of Eq. 5 (|e|^2 = 1 and 2)
+    // a_k = (m*_k - m_k) / |row_k|^2 of the D2Q9 collision (the names of PairRates in step2p.cu)
+    double ke1, ke2, ke3, kp1, kp2, kp3, kq1, kq2, kn1, kn2, kh8;
+    bool body;                     // a body force is set
+};
+using Fold64 = Fold<double>;
+inline void make_fold(Fold<float>*, const DevParams&) {}
+inline void make_fold(Fold<double>* k, const DevParams& p) {
+    k->kRT = p.two_over_G * p.RT;
+    k->ka = p.two_over_G * p.a;
+    k->kaphi = p.two_over_G * p.aphi;
+    k->k3 = p.two_over_G / 3.0;
+    k->g1 = -p.G / 3.0;
+    k->g2 = -p.G / 12.0;
+    const double he = 1.0 - 0.5 * p.s_e, hp = 1.0 - 0.5 * p.s_eps, hq = 1.0 - 0.5 * p.s_q, hn = 1.0 - 0.5 * p.s_nu;
+    k->ke1 = -p.s_e / 36.0;
+    k->ke2 = 6.0 * he / 36.0;
+    k->ke3 = he * p.c_e / 36.0;
+    k->kp1 = -p.s_eps / 36.0;
+    k->kp2 = -6.0 * hp / 36.0;
+    k->kp3 = -hp * p.c_eps / 36.0;
+    k->kq1 = -p.s_q / 12.0;
+    k->kq2 = -hq / 12.0;
+    k->kn1 = -p.s_nu / 4.0;
+    k->kn2 = 2.0 * hn / 4.0;
+    k->kh8 = hn / 4.0;
+    k->body = p.fx != 0.0 || p.fy != 0.0 || p.fz != 0.0;
+}
+
 // physics constants in compute precision
 template <class C>
 struct Phys {
@@ -17,6 +52,7 @@ struct Phys {
     C rho_l, rho_g, rho_ref, fx, fy, fz;
     C wall_param;   // VD: the constant virtual density; SF: the adhesion parameter G_w of Eq. 8
     Rates<C> r;
+    Fold<C> fold;
 };
 
 template <class C>
@@ -46,6 +82,7 @@ Phys<C> make_phys(const DevParams& p) {
     h.r.s_m = C(p.s_m);
     h.r.c_e = C(p.c_e);
     h.r.c_eps = C(p.c_eps);
+    make_fold(&h.fold, p);
     return h;
 }
 
@@ -59,6 +96,34 @@ struct Geo {
     const double* kappa_w;   // per wall node or null
     double kappa;
 };
+
+// The grid of a single-grid launch (kernel parameters); a batch passes its work record (shared
+// memory) with the same member names.  Members are read where they are used, so that nothing of
+// the grid needs a register across the tile's barriers.
+struct PairGrid {
+    int nx, ny, N;
+    int fp, fs;   // distribution row pitch and direction stride
+    const uint8_t* type;
+    const int* wall_id;
+    const double* kappa_w;
+    double kappa;
+    const void* f[2];
+};
+inline PairGrid pair_grid(const void* fin, const void* fout, const DevParams& p) {
+    PairGrid g;
+    g.nx = p.nx;
+    g.ny = p.ny;
+    g.N = int(p.N);
+    g.fp = p.fp;
+    g.fs = int(p.fs);
+    g.type = p.type;
+    g.wall_id = p.wall_id;
+    g.kappa_w = p.kappa_w;
+    g.kappa = p.kappa;
+    g.f[0] = fin;
+    g.f[1] = fout;
+    return g;
+}
 
 // Division in compute precision: FP64 keeps IEEE division (parity with the FP64 oracle); the FP32
 // path uses the fast hardware approximation (relative error of a few ulp, below the rounding of the
