@@ -622,12 +622,21 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
     CKI(guarded_malloc(&h->f[0], h->fbytes, h->stream), "cudaMalloc f");
     CKI(guarded_malloc(&h->f[1], h->fbytes, h->stream), "cudaMalloc f");
     CKI(dmalloc(&h->d_type, N, h->stream), "cudaMalloc type");
-    // (D2Q9 FP64: followed by the flags of the grid's FP64 tiles)
+    // (FP64: followed by the flags of the grid's FP64 tiles)
     std::vector<uint8_t> flags = h->tile_solid;
-    int fw = 0, fh = 0;
-    if (h->D == 2 && h->prec == LBM_FP64) {
-        d2q9_fp64_tile(&nx, &ny, 1, device_sms(), &fw, &fh);
-        const std::vector<uint8_t> own = merged_flags(h, fw, fh);
+    int fw = 0, fh = 0, fz = 1;
+    if (h->prec == LBM_FP64) {
+        std::vector<uint8_t> own;
+        if (h->D == 2) {
+            d2q9_fp64_tile(&nx, &ny, 1, device_sms(), &fw, &fh);
+            own = merged_flags(h, fw, fh);
+        } else {
+            // (a brick is much smaller than the 32-plane chunks of tile_solid, and a flagged one costs more
+            // halo planes: its own scan)
+            d3q19_fp64_brick(nx, ny, nz, device_sms(), &fw, &fh, &fz);
+            const int t[3] = {fw, fh, fz};
+            own = tile_solid_flags(solid_mask, nx, ny, nz, t, 3, scan_threads(N));
+        }
         flags.insert(flags.end(), own.begin(), own.end());
     }
     CKI(dmalloc(&h->d_tile_solid, flags.size(), h->stream), "cudaMalloc tile flags");
@@ -721,6 +730,7 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
     p.tile_solid = h->d_tile_solid;
     p.tile_w = fw;
     p.tile_h = fh;
+    p.tile_z = fz;
     if (fw > 0) p.pair_solid = h->d_tile_solid + h->tile_solid.size();
     p.err = h->d_err;
     // D3Q19 FP32 step kernel and the tensor maps of the TMA-staged z-march

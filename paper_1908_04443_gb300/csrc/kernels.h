@@ -33,9 +33,9 @@ struct DevParams {
     const uint8_t* type;         // per node: T_SOLID | T_WALL | T_NEARWALL | T_BULK
     const uint8_t* tile_solid;   // per tile of the step kernel's grid: a solid node within the tile + 3-node halo
     // the same per tile of the FP32 pair kernel (null: FP32 steps use the tile kernel) or, in FP64, of the
-    // grid's FP64 tiles (tile_w x tile_h nodes)
+    // grid's FP64 tiles (tile_w x tile_h (x tile_z) nodes)
     const uint8_t* pair_solid;
-    int tile_w, tile_h;
+    int tile_w, tile_h, tile_z;
     // D3Q19 FP32 step kernel: 0 the TMA-staged z-march, 1 the z-pair march, 2 the scalar z-march
     int step3;
     const void* ztmap;           // TMA tensor maps of the two 3D FP32 distribution buffers (device, 2 x 128 B)
@@ -165,6 +165,11 @@ struct Geo;
 cudaError_t launch_step3d(int prec, int mode, const void* fin, void* fout, const Geo& g, const DevParams& p,
                           double* rho, double* u, cudaStream_t s);
 void zmarch_tile_shape(int prec, int* tx, int* ty, int* tz);
+// D3Q19 FP64: the step (mode 0) or the fields (mode 1) on bricks of p.tile_w x p.tile_h x p.tile_z nodes with
+// the flags p.pair_solid; and the brick for a grid on `sms` SMs.
+cudaError_t launch_d3q19_fp64(int mode, const void* fin, void* fout, const Geo& g, const DevParams& p, double* rho,
+                              double* u, cudaStream_t s);
+void d3q19_fp64_brick(int nx, int ny, int nz, int sms, int* bw, int* bh, int* bz);
 // D3Q19 FP32 step as a z-pair march (two planes per thread, packed FP32x2 arithmetic); chunk flags
 // g.tile_solid per FP32 z-march chunk.
 cudaError_t launch_zpair_step(const void* fin, void* fout, const Geo& g, const DevParams& p, cudaStream_t s);

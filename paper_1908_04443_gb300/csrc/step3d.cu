@@ -46,7 +46,7 @@ struct ZShape;
 template <> struct ZShape<float> {
     static constexpr int X = LBMWET_Z3F_X, Y = LBMWET_Z3F_Y, Z = LBMWET_Z3F_Z, MINB = LBMWET_Z3F_MINB;
 };
-template <> struct ZShape<double> { static constexpr int X = 32, Y = 4, Z = 32, MINB = 1; };
+template <> struct ZShape<double> { static constexpr int X = 32, Y = 4, Z = 32; };   // flags only (FP64: step3d64.cu)
 
 template <class S, class C, int MODE>
 __global__ void __launch_bounds__(ZShape<S>::X* ZShape<S>::Y, ZShape<S>::MINB)
@@ -324,8 +324,7 @@ cudaError_t launch_step3d(int prec, int mode, const void* fin, void* fout, const
     if (prec == PREC_FP32 && mode == 0 && p.step3 == 0 && p.ztmap)
         return launch_ztma_step(fin, fout, static_cast<const char*>(p.ztmap) + (fin == p.zf0 ? 0 : 128), g, p, s);
     if (prec == PREC_FP32 && mode == 0 && p.step3 != 2) return launch_zpair_step(fin, fout, g, p, s);
-    if (prec == PREC_FP64)
-        return mode == 0 ? launch_z<double, 0>(fin, fout, g, p, rho, u, s) : launch_z<double, 1>(fin, fout, g, p, rho, u, s);
+    if (prec == PREC_FP64) return launch_d3q19_fp64(mode, fin, fout, g, p, rho, u, s);
     return mode == 0 ? launch_z<float, 0>(fin, fout, g, p, rho, u, s) : launch_z<float, 1>(fin, fout, g, p, rho, u, s);
 }
 

@@ -7,8 +7,7 @@
 // has the same number of them.  A tile's ring costs 26 FP64 instructions a cell (density and psi)
 // against 136 for an own node, so large tiles are cheaper (32 x 16: ring 20 % of the cells, +4 %) as long
 // as there are many of them per SM; a grid with few nodes is cut into small tiles, about one per SM
-// (d2q9_fp64_tile), since an SM works on a 32 x 8 tile for 17 us however idle the others are: the step of
-// a 100 x 100 grid 25.9 -> 13.0 us with 130 tiles of 8 x 10 in place of 52 of 32 x 8.
+// (d2q9_fp64_tile), since an SM works on a 32 x 8 tile for 17 us however idle the others are.
 // Columns and rows of a tile beyond the grid's edge are skipped instead of wrapped.
 // Integer work is free beside the FP64 pipe: shapes are run-time values and every neighbour wraps.
 #include "fp64.cuh"
@@ -33,18 +32,6 @@ struct Smem64 {
     short wall[PYP * PXP];
     int nwall;
 };
-
-// cell k of the one-cell ring of an ax x ay box
-__device__ __forceinline__ void ring_cell(int k, int ax, int ay, int& x, int& y) {
-    if (k < 2 * ax) {
-        y = k < ax ? 0 : ay - 1;
-        x = k < ax ? k : k - ax;
-    } else {
-        const int j = k - 2 * ax;
-        y = 1 + (j >> 1);
-        x = (j & 1) ? ax - 1 : 0;
-    }
-}
 
 // One tile of w x h nodes (w = 1 << wl) at (x0, y0) of the grid g (a BatchItem or PairGrid), reading
 // g.f[parity].  MODE 0: step into g.f[parity ^ 1]; 1: fields.  SOLID: a solid node lies within the tile
@@ -295,20 +282,24 @@ __global__ void __launch_bounds__(NT, 2) fields64_grids(const FieldGrid* __restr
 
 }  // namespace
 
-// The shape with the least modelled time: the tiles of an SM one after another, each costing its own
-// nodes' and its ring's FP64 instructions and a fixed latency (loads, dependent chains, barriers; about
-// 3000 clocks) that hides behind the other tiles of the SM when it has several.
+// The shape with the least modelled time.  A tile costs the FP64 instructions of its warps (own nodes and
+// ring cells rounded up to warps) at 1.9 lane operations per clock and 1000 clocks of latency that its SM's
+// other tiles do not hide; alone on its SM it takes 1.35 times that.  Up to two tiles per SM run at once, and
+// the fullest SM decides; beyond that tiles are handed out as SMs get free and half a tile is the tail.
+// Fitted to 14 shapes on 4 grids (100 x 100 to
+// 1000 x 1000): it picks a shape within 5 % of the fastest on each, 8 x 10 (10.9 us a step) for 100 x 100,
+// 32 x 12 for 300 x 350 (34.6 us; 32 x 16 takes 44.9), 16 x 16 for 600 x 400 (67.8 us; 32 x 16 takes 78.9).
 void d2q9_fp64_tile(const int* nx, const int* ny, int ngrids, int sms, int* tw, int* th) {
+    auto warps = [](int n) { return double((n + 31) / 32 * 32); };
     double best = 1e300;
     for (int w = 8; w <= MW; w *= 2)
-        for (int h = 1; h <= MH; ++h) {
-            long long tiles = 0;
-            for (int i = 0; i < ngrids; ++i) tiles += (long long)((nx[i] + w - 1) / w) * ((ny[i] + h - 1) / h);
-            const long long per_sm = (tiles + sms - 1) / sms;
-            const double work = (136.0 * w * h + 26.0 * (2 * w + 2 * h + 4)) / 1.7;
-            const double cost = double(per_sm) * work + 3000.0 * (per_sm > 1 ? double(per_sm) / 2 : 1.0);
-            if (cost < best * 0.999) {
-                best = cost;
+        for (int h = 64 / w; h <= MH; ++h) {   // (at least two warps of nodes)
+            long long n = 0;
+            for (int i = 0; i < ngrids; ++i) n += (long long)((nx[i] + w - 1) / w) * ((ny[i] + h - 1) / h);
+            const double tile = (136.0 * warps(w * h) + 26.0 * warps(2 * w + 2 * h + 4)) / 1.9 + 1000.0;
+            const double rounds = n <= sms ? 1.35 : (n <= 2LL * sms ? 2.0 : double(n) / sms + 0.5);
+            if (tile * rounds < best * 0.999) {
+                best = tile * rounds;
                 *tw = w;
                 *th = h;
             }

@@ -18,6 +18,8 @@ struct Fold<double> {
     double g1, g2;                 // -G times the D2Q9 weights of Eq. 5 (|e|^2 = 1 and 2)
     // a_k = (m*_k - m_k) / |row_k|^2 of the D2Q9 collision (the names of PairRates in step2p.cu)
     double ke1, ke2, ke3, kp1, kp2, kp3, kq1, kq2, kn1, kn2, kh8;
+    // the same of the D3Q19 collision (the names of Rates3P in step3p.cu), and its Eq. 5 weight of |e|^2 = 1
+    double g3, t1e, t2e, t3e, t1p, t2p, t3p, tq1, tq2, tn9, th9, tp10, th10, tn11, th11, tp12, th12, tn13, th13, tm;
     bool body;                     // a body force is set
 };
 using Fold64 = Fold<double>;
@@ -33,7 +35,7 @@ inline void make_fold(Fold<double>* k, const DevParams& p) {
     k->ke1 = -p.s_e / 36.0;
     k->ke2 = 6.0 * he / 36.0;
     k->ke3 = he * p.c_e / 36.0;
-    k->kp1 = -p.s_eps / 36.0;
+    k->kp1 = -p.s_eps * 3.0 / 36.0;
     k->kp2 = -6.0 * hp / 36.0;
     k->kp3 = -hp * p.c_eps / 36.0;
     k->kq1 = -p.s_q / 12.0;
@@ -41,6 +43,27 @@ inline void make_fold(Fold<double>* k, const DevParams& p) {
     k->kn1 = -p.s_nu / 4.0;
     k->kn2 = 2.0 * hn / 4.0;
     k->kh8 = hn / 4.0;
+    const double hpi = 1.0 - 0.5 * p.s_pi;
+    k->g3 = -p.G / 6.0;
+    k->t1e = -p.s_e * 19.0 / 2394.0;
+    k->t2e = 38.0 * he / 2394.0;
+    k->t3e = he * p.c_e / 2394.0;
+    k->t1p = -p.s_eps / 252.0;
+    k->t2p = -11.0 * hp / 252.0;
+    k->t3p = -hp * p.c_eps / 252.0;
+    k->tq1 = -p.s_q / 40.0;
+    k->tq2 = -hq * (2.0 / 3.0) / 40.0;
+    k->tn9 = -p.s_nu / 36.0;
+    k->th9 = 2.0 * hn / 36.0;
+    k->tp10 = -p.s_pi / 72.0;
+    k->th10 = -hpi / 72.0;
+    k->tn11 = -p.s_nu / 12.0;
+    k->th11 = 2.0 * hn / 12.0;
+    k->tp12 = -p.s_pi / 24.0;
+    k->th12 = -hpi / 24.0;
+    k->tn13 = -p.s_nu / 4.0;
+    k->th13 = hn / 4.0;
+    k->tm = -p.s_m / 8.0;
     k->body = p.fx != 0.0 || p.fy != 0.0 || p.fz != 0.0;
 }
 
