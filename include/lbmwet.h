@@ -85,7 +85,7 @@ typedef enum { LBM_BODY_NONE = 0, LBM_BODY_BALL = 1, LBM_BODY_PLANE = 2 } lbm_bo
 
 /* Step kernel (no counterpart in the paper: a choice of work decomposition).
  * D2Q9:
- *   TILE: one CTA per 32 x 8 tile with its halo ring, one node per thread.  YMARCH: persistent
+ *   TILE: one CTA per tile with its halo ring (32 x 8 nodes in FP32, sized for the grid in FP64).  YMARCH: persistent
  *   CTAs walking runs of rows of column blocks (124 own columns plus a 2-cell halo on each side),
  *   planned on the host so that every CTA pulls about the same number of rows; bit-identical to
  *   TILE.  PAIR (FP32 only): 32 x 16 tiles, two nodes per thread computed together with packed
@@ -95,14 +95,15 @@ typedef enum { LBM_BODY_NONE = 0, LBM_BODY_BALL = 1, LBM_BODY_PLANE = 2 } lbm_bo
  *   has chosen one.  A y-march handle that records a trajectory for the adjoint steps with TILE
  *   from lbm_record on.
  * D3Q19 (every kernel marches z-planes through 32-plane chunks of x-y columns):
- *   ZTMA (FP32 only): 32 x 8 columns cut along z into the work items of lbm_d3q19_work_list, one
- *   CTA per item; the lead plane's 19 pull boxes are staged in shared memory by TMA, two planes in
- *   flight, two cells per thread in packed FP32x2 arithmetic; items on planes near a solid also
- *   stage node types and do the bounce-back and virtual-density work; columns cut by the grid's
- *   edge (ragged) run the z-pair march.  PAIR (FP32 only): the z-pair march, 32 x 4 columns, two planes
- *   per thread.  TILE: the scalar z-march (the only D3Q19 kernel in FP64).  AUTO: ZTMA in FP32
- *   (PAIR where the rows are not a multiple of 16 bytes), TILE in FP64.  The FP32 kernels agree up
- *   to FP32 rounding. */
+ *   ZTMA (FP32 only): 32 x 8 columns cut along z into work items, one CTA per item (those of
+ *   lbm_d3q19_work_list, except that columns cut by the grid's edge are moved inside it and that small
+ *   grids are cut into shorter items); the lead plane's 19 pull boxes are staged in shared memory by
+ *   TMA, two planes in flight; items on planes near a solid also stage node types and do the bounce-back
+ *   and virtual-density work; grids below 40 x 16 x 4 nodes run the z-pair march.  PAIR (FP32 only): the
+ *   z-pair march, 32 x 4 columns, two planes per thread.  TILE: the scalar z-march; in FP64 (the only
+ *   D3Q19 kernel there) bricks sized for the grid.  AUTO: ZTMA in FP32 (PAIR on grids below 40 x 16 x 4
+ *   whose rows are not a multiple of 16 bytes), TILE in FP64.  The FP32 kernels agree up to FP32
+ *   rounding. */
 typedef enum { LBM_KERNEL_AUTO = 0, LBM_KERNEL_TILE = 1, LBM_KERNEL_YMARCH = 2, LBM_KERNEL_PAIR = 3,
                LBM_KERNEL_ZTMA = 4 } lbm_step_kernel;
 
@@ -292,7 +293,8 @@ lbm_status lbm_grid_shape(const lbm_handle* h, int32_t* shape4);
 int64_t lbm_kernel_launches(const lbm_handle* h);
 
 /* The work list of the TMA-staged D3Q19 z-march (LBM_KERNEL_ZTMA) for a solid mask: host code only
- * (no device, no handle), the list lbm_init builds for an FP32 D3Q19 handle on that kernel.  One
+ * (no device, no handle), the list lbm_init builds for an FP32 D3Q19 handle on that kernel where every
+ * column is full and the grid fills the GPU (else see lbm_step_kernel).  One
  * time step (Eqs. 1-7 with the Eq. 16-17 walls) is split into items, one CTA each: item i is the 5
  * int32 values items[5i .. 5i+4] = {bx, by, z0, z1, solid}: the column of cells x in [32 bx,
  * 32 bx + 32), y in [8 by, 8 by + 8) (clipped to the grid), planes z0 <= z < z1, and solid = 1 where

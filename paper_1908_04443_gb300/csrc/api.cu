@@ -122,14 +122,14 @@ bool encode_pair_map(CUtensorMap* m, void* f, int nx, int ny, int fp, long long 
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// TMA tensor map of one FP32 D3Q19 distribution buffer f[a][z][y][x] seen as a 3D tensor
+// TMA tensor map of one FP32 D3Q19 distribution buffer f[a][z][y][x] (row pitch fp) seen as a 3D tensor
 // (x, y, a * nz + z): the box of the TMA-staged z-march (one direction on one plane, bx x by).
 // False where TMA cannot address the buffer (rows not a multiple of 16 bytes).
-bool encode_z_map(CUtensorMap* m, void* f, int nx, int ny, int nz, int bx, int by) {
+bool encode_z_map(CUtensorMap* m, void* f, int nx, int ny, int nz, int fp, int bx, int by) {
     PFN_cuTensorMapEncodeTiled_v12000 enc = tmap_encoder();
-    if (!enc || nx % 4 != 0) return false;
+    if (!enc || fp % 4 != 0) return false;
     const cuuint64_t dims[3] = {cuuint64_t(nx), cuuint64_t(ny), cuuint64_t(19) * cuuint64_t(nz)};
-    const cuuint64_t strides[2] = {cuuint64_t(nx) * 4, cuuint64_t(nx) * cuuint64_t(ny) * 4};
+    const cuuint64_t strides[2] = {cuuint64_t(fp) * 4, cuuint64_t(fp) * cuuint64_t(ny) * 4};
     const cuuint32_t box[3] = {cuuint32_t(bx), cuuint32_t(by), 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, f, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -351,6 +351,19 @@ lbm_status enqueue_steps(lbm_handle* h, int64_t n) {
         }
     }
     return LBM_OK;
+}
+
+// A checkpoint holds the distributions as stored, except that the rows of 3D grids are unpadded.
+size_t checkpoint_bytes(const lbm_handle* h) {
+    return h->D == 3 ? h->fbytes / (size_t)h->dp.fp * (size_t)h->dp.nx : h->fbytes;
+}
+cudaError_t checkpoint_copy(lbm_handle* h, void* dst, const void* src, bool to_host) {
+    const cudaMemcpyKind kind = to_host ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice;
+    if (h->D == 2 || h->dp.fp == h->dp.nx) return cudaMemcpyAsync(dst, src, checkpoint_bytes(h), kind, h->stream);
+    const size_t es = h->prec == LBM_FP64 ? sizeof(double) : sizeof(float);
+    const size_t row = es * (size_t)h->dp.nx, pitch = es * (size_t)h->dp.fp;
+    return cudaMemcpy2DAsync(dst, to_host ? row : pitch, src, to_host ? pitch : row, row, h->fbytes / pitch, kind,
+                             h->stream);
 }
 
 // lbm_obs from the NRED sums of the observables reduction (mass, density extremes, max |u|^2,
@@ -606,8 +619,9 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
     const size_t ssize = c.precision == LBM_FP64 ? sizeof(double) : sizeof(float);
     // distributions: 2D rows padded to a multiple of 32 nodes (128-byte rows in FP32: TMA needs
     // 16-byte row strides, and a row that starts a cache line keeps a warp's 32 consecutive nodes in
-    // one line)
-    const int fpitch = h->D == 2 ? (nx + 31) / 32 * 32 : nx;
+    // one line); 3D FP32 rows to a multiple of 4 nodes, so that every width has tensor maps
+    const int pad = h->D == 2 ? 32 : (c.precision == LBM_FP32_DEV ? 4 : 1);
+    const int fpitch = (nx + pad - 1) / pad * pad;
     const long long fstride = (long long)fpitch * ny * nz;
     h->fbytes = ssize * h->Q * (size_t)fstride;
     auto oom = [&](cudaError_t e, const char* what) {
@@ -737,15 +751,16 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
     p.step3 = c.step_kernel == LBM_KERNEL_PAIR ? 1 : (c.step_kernel == LBM_KERNEL_TILE ? 2 : 0);
     p.ztmap = nullptr;
     p.zf0 = h->f[0];
-    if (h->D == 3 && c.precision == LBM_FP32_DEV && p.step3 == 0) {
+    if (h->D == 3 && c.precision == LBM_FP32_DEV && p.step3 == 0 && ztma_marches(nx, ny, nz)) {
         int bx, by;
         ztma_box_dims(&bx, &by);
         CUtensorMap maps[2];
-        if (encode_z_map(&maps[0], h->f[0], nx, ny, nz, bx, by) && encode_z_map(&maps[1], h->f[1], nx, ny, nz, bx, by)) {
+        if (encode_z_map(&maps[0], h->f[0], nx, ny, nz, fpitch, bx, by) &&
+            encode_z_map(&maps[1], h->f[1], nx, ny, nz, fpitch, bx, by)) {
             CKI(dmalloc(&h->d_zmaps, sizeof(maps), h->stream), "cudaMalloc tensor maps");
             // (from pageable memory: staged before the call returns, so `maps` may go out of scope)
             CKI(cudaMemcpyAsync(h->d_zmaps, maps, sizeof(maps), cudaMemcpyHostToDevice, h->stream), "copy tensor maps");
-            const std::vector<ZItem> items = ztma_work_list(solid_mask, nx, ny, nz);
+            const std::vector<ZItem> items = ztma_items(solid_mask, nx, ny, nz, 2 * device_sms());   // (2 CTAs per SM)
             CKI(dmalloc(&h->d_zitems, sizeof(ZItem) * items.size(), h->stream), "cudaMalloc work list");
             CKI(cudaMemcpyAsync(h->d_zitems, items.data(), sizeof(ZItem) * items.size(), cudaMemcpyHostToDevice,
                                 h->stream), "copy work list");
@@ -1008,25 +1023,26 @@ lbm_status lbm_set_state(lbm_handle* h, const double* f_host, int64_t step) {
 
 lbm_status lbm_save_state(lbm_handle* h, void* host_buf, size_t* bytes) {
     if (!h || !bytes) return LBM_ERR_ARG;
-    const size_t need = h->fbytes + sizeof(int64_t);
+    const size_t body = checkpoint_bytes(h), need = body + sizeof(int64_t);
     if (!host_buf) {
         *bytes = need;
         return LBM_OK;
     }
     if (*bytes < need) return fail(h, LBM_ERR_ARG, "checkpoint buffer too small");
-    CK(h, cudaMemcpyAsync(host_buf, h->f[h->cur], h->fbytes, cudaMemcpyDeviceToHost, h->stream));
+    CK(h, checkpoint_copy(h, host_buf, h->f[h->cur], true));
     CK(h, cudaStreamSynchronize(h->stream));
-    std::memcpy(static_cast<char*>(host_buf) + h->fbytes, &h->step, sizeof(int64_t));
+    std::memcpy(static_cast<char*>(host_buf) + body, &h->step, sizeof(int64_t));
     *bytes = need;
     return LBM_OK;
 }
 
 lbm_status lbm_load_state(lbm_handle* h, const void* host_buf, size_t bytes) {
     if (!h || !host_buf) return LBM_ERR_ARG;
-    if (bytes != h->fbytes + sizeof(int64_t)) return fail(h, LBM_ERR_ARG, "checkpoint size mismatch");
-    CK(h, cudaMemcpyAsync(h->f[h->cur], host_buf, h->fbytes, cudaMemcpyHostToDevice, h->stream));
+    const size_t body = checkpoint_bytes(h);
+    if (bytes != body + sizeof(int64_t)) return fail(h, LBM_ERR_ARG, "checkpoint size mismatch");
+    CK(h, checkpoint_copy(h, h->f[h->cur], host_buf, false));
     CK(h, cudaStreamSynchronize(h->stream));
-    std::memcpy(&h->step, static_cast<const char*>(host_buf) + h->fbytes, sizeof(int64_t));
+    std::memcpy(&h->step, static_cast<const char*>(host_buf) + body, sizeof(int64_t));
     return LBM_OK;
 }
 
@@ -1061,7 +1077,8 @@ int32_t lbm_step_kernel_used(const lbm_handle* h) {
     if (!h) return LBM_KERNEL_AUTO;
     if (h->D == 3) {
         if (h->prec == LBM_FP64 || h->dp.step3 == 2) return LBM_KERNEL_TILE;
-        return h->dp.step3 == 0 && h->dp.ztmap ? LBM_KERNEL_ZTMA : LBM_KERNEL_PAIR;
+        // (a grid smaller than the march's columns and boxes runs the z-pair march under the same name)
+        return h->dp.step3 == 0 && (h->dp.ztmap || h->cfg.nx % 4 == 0) ? LBM_KERNEL_ZTMA : LBM_KERNEL_PAIR;
     }
     if (h->ymarch) return LBM_KERNEL_YMARCH;
     return h->prec == LBM_FP32_DEV && h->dp.pair_solid ? LBM_KERNEL_PAIR : LBM_KERNEL_TILE;

@@ -185,6 +185,14 @@ void ztma_box_dims(int* bx, int* by);
 // (a first or last piece shorter than 8 planes joins its neighbour); the other columns as the z-pair
 // march's 32-plane chunks; ordered by first plane, then column.
 std::vector<ZItem> ztma_work_list(const uint8_t* mask, int nx, int ny, int nz);
+// The items a handle's launch runs, for `slots` resident CTAs: every column on the march (the last ones moved
+// inside the grid), and shorter pieces where the grid would not fill the chip.  Only for grids that the march
+// covers (ztma_marches).
+std::vector<ZItem> ztma_items(const uint8_t* mask, int nx, int ny, int nz, int slots);
+bool ztma_marches(int nx, int ny, int nz);
+// The fields pass on the same items.
+cudaError_t launch_ztma_fields(const void* fin, const void* tmap, const Geo& g, const DevParams& p, double* rho,
+                               double* u, cudaStream_t s);
 // Tile shape (x, y, z) of the step kernels and the resident CTAs per SM of the batched kernel.
 void step_tile_shape(int lat, int prec, int* tx, int* ty, int* tz);
 int batched_ctas_per_sm();

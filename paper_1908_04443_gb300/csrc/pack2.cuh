@@ -23,6 +23,41 @@ __device__ __forceinline__ V2 operator-(V2 a, V2 b) { return fma2(-1.0f, b, a); 
 __device__ __forceinline__ V2 operator-(V2 a) { return -1.0f * a; }
 __device__ __forceinline__ V2 div2(V2 a, V2 b) { return mk(__fdividef(a.v.x, b.v.x), __fdividef(a.v.y, b.v.y)); }
 
+// One FP32 value with the pair's operations, each rounded as a lane of the pair is.
+struct V1 {
+    float v;
+};
+__device__ __forceinline__ V1 operator+(V1 a, V1 b) { return {__fadd_rn(a.v, b.v)}; }
+__device__ __forceinline__ V1 operator*(V1 a, V1 b) { return {__fmul_rn(a.v, b.v)}; }
+__device__ __forceinline__ V1 operator*(float s, V1 b) { return {__fmul_rn(s, b.v)}; }
+__device__ __forceinline__ V1 fma2(V1 a, V1 b, V1 c) { return {__fmaf_rn(a.v, b.v, c.v)}; }
+__device__ __forceinline__ V1 fma2(float s, V1 b, V1 c) { return {__fmaf_rn(s, b.v, c.v)}; }
+__device__ __forceinline__ V1 operator-(V1 a, V1 b) { return {__fsub_rn(a.v, b.v)}; }
+__device__ __forceinline__ V1 operator-(V1 a) { return {-a.v}; }
+__device__ __forceinline__ V1 div2(V1 a, V1 b) { return {__fdividef(a.v, b.v)}; }
+
+// psi of one value, as psi2 below computes a lane; a non-positive argument flags ERR_PSI
+__device__ __forceinline__ V1 psi1(V1 rho, const Phys<float>& e, unsigned* err) {
+    const V1 one = {1.0f};
+    V1 p;
+    if (e.eos_kind == 1) {
+        const V1 eta = e.b4 * rho;
+        const V1 om = one - eta;
+        const V1 poly = fma2(eta * eta, one - eta, one + eta);
+        p = div2((e.RT * rho) * poly, (om * om) * om) - e.a * (rho * rho);
+    } else {
+        const V1 br = e.b * rho;
+        const V1 den2 = fma2(br, V1{2.0f} - br, one);
+        p = div2(e.RT * rho, one - br) - div2(e.aphi * (rho * rho), den2);
+    }
+    const V1 arg = e.two_over_G * fma2(-1.0f / 3.0f, rho, p);
+    if (!(arg.v > 0.0f)) {
+        atomicOr(err, ERR_PSI);
+        return {0.0f};
+    }
+    return {arg.v * rsqrtf(arg.v)};
+}
+
 // psi of a pair (Eq. 6 with the C-S or PR pressure); a non-positive argument flags ERR_PSI on
 // the lanes in `check` and gives psi 0
 __device__ __forceinline__ V2 psi2(V2 rho, const Phys<float>& e, bool check_a, bool check_b, unsigned* err) {

@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(ZShape<S>::X* ZShape<S>::Y, ZShape<S>::MINB)
     const int tile = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
     const bool solid = g.tile_solid ? g.tile_solid[tile] != 0 : true;
     const int nxy = nx * ny;
+    const int fp = g.fp, fs = g.fs, fxy = fp * ny;   // distributions: row pitch, direction and plane stride
 
     auto load_types = [&](int z) {
         if (!solid) return;
@@ -85,13 +86,13 @@ __global__ void __launch_bounds__(ZShape<S>::X* ZShape<S>::Y, ZShape<S>::MINB)
     // pull of node (gx, gy, gz) of plane z whose type-plane cell is ti
     auto pull = [&](C (&f)[Q], int gx, int gy, int gz, int z, int ti, uint8_t self) {
         const int cx[3] = {wrap1(gx - 1, nx), gx, wrap1(gx + 1, nx)};
-        const int ry[3] = {wrap1(gy - 1, ny) * nx, gy * nx, wrap1(gy + 1, ny) * nx};
-        const int pz[3] = {wrap1(gz - 1, nz) * nxy, gz * nxy, wrap1(gz + 1, nz) * nxy};
+        const int ry[3] = {wrap1(gy - 1, ny) * fp, gy * fp, wrap1(gy + 1, ny) * fp};
+        const int pz[3] = {wrap1(gz - 1, nz) * fxy, gz * fxy, wrap1(gz + 1, nz) * fxy};
         const int gi = pz[1] + ry[1] + cx[1];
         if (self & T_BULK) {
 #pragma unroll
             for (int a = 0; a < Q; ++a)
-                f[a] = C(fin[a * N + pz[1 - L::ez(a)] + ry[1 - L::ey(a)] + cx[1 - L::ex(a)]]);
+                f[a] = C(fin[a * fs + pz[1 - L::ez(a)] + ry[1 - L::ey(a)] + cx[1 - L::ex(a)]]);
         } else {
             const uint8_t* tm = sm.type[ring(z - 1, 5)];
             const uint8_t* t0 = sm.type[ring(z, 5)];
@@ -102,7 +103,7 @@ __global__ void __launch_bounds__(ZShape<S>::X* ZShape<S>::Y, ZShape<S>::MINB)
                 const int ex = L::ex(a), ey = L::ey(a), ez = L::ez(a);
                 const uint8_t* tz = ez > 0 ? tm : (ez < 0 ? tp : t0);   // upstream plane is z - ez
                 const bool bb = (tz[ti - ex - ey * YX] & T_SOLID) != 0;
-                f[a] = C(fin[bb ? L::opp(a) * N + gi : a * N + pz[1 - ez] + ry[1 - ey] + cx[1 - ex]]);
+                f[a] = C(fin[bb ? L::opp(a) * fs + gi : a * fs + pz[1 - ez] + ry[1 - ey] + cx[1 - ex]]);
             }
         }
     };
@@ -272,7 +273,7 @@ __global__ void __launch_bounds__(ZShape<S>::X* ZShape<S>::Y, ZShape<S>::MINB)
                     const C X = cdiv(Fmx * Fmx + Fmy * Fmy + Fmz * Fmz, psi_c * psi_c);
                     collide_d3q19<C>(f, drho, rho, ux, uy, uz, Fx, Fy, Fz, X, ph.r);
 #pragma unroll
-                    for (int a = 0; a < Q; ++a) fout[a * N + gi] = S(f[a]);
+                    for (int a = 0; a < Q; ++a) fout[a * fs + zc * fxy + (y0 + ly) * fp + x0 + lx] = S(f[a]);
                 }
             }
         }
@@ -321,8 +322,10 @@ void zmarch_tile_shape(int prec, int* tx, int* ty, int* tz) {
 
 cudaError_t launch_step3d(int prec, int mode, const void* fin, void* fout, const Geo& g, const DevParams& p,
                           double* rho, double* u, cudaStream_t s) {
-    if (prec == PREC_FP32 && mode == 0 && p.step3 == 0 && p.ztmap)
-        return launch_ztma_step(fin, fout, static_cast<const char*>(p.ztmap) + (fin == p.zf0 ? 0 : 128), g, p, s);
+    if (prec == PREC_FP32 && p.ztmap) {
+        const void* map = static_cast<const char*>(p.ztmap) + (fin == p.zf0 ? 0 : 128);
+        return mode == 0 ? launch_ztma_step(fin, fout, map, g, p, s) : launch_ztma_fields(fin, map, g, p, rho, u, s);
+    }
     if (prec == PREC_FP32 && mode == 0 && p.step3 != 2) return launch_zpair_step(fin, fout, g, p, s);
     if (prec == PREC_FP64) return launch_d3q19_fp64(mode, fin, fout, g, p, rho, u, s);
     return mode == 0 ? launch_z<float, 0>(fin, fout, g, p, rho, u, s) : launch_z<float, 1>(fin, fout, g, p, rho, u, s);

@@ -83,92 +83,93 @@ Rates3P make_rates3p(const DevParams& p) {
 }
 
 // MRT collision (d'Humieres D3Q19, source of Eq. 7 as in collide_d3q19) of a pair; f += M^-1 (m* - m)
-__device__ __forceinline__ void collide3p(V2 (&f)[19], V2 drho, V2 rho, V2 ux, V2 uy, V2 uz, V2 Fx, V2 Fy, V2 Fz, V2 X,
+template <class V>   // V2 (a pair) or V1
+__device__ __forceinline__ void collide3p(V (&f)[19], V drho, V rho, V ux, V uy, V uz, V Fx, V Fy, V Fz, V X,
                                           const Rates3P& k) {
     // moments of the non-conserved rows
-    const V2 ax = f[1] + f[2], ay = f[3] + f[4], az = f[5] + f[6];
-    const V2 d12 = f[1] - f[2], d34 = f[3] - f[4], d56 = f[5] - f[6];
-    const V2 p78 = f[7] + f[8], p910 = f[9] + f[10], p1112 = f[11] + f[12], p1314 = f[13] + f[14];
-    const V2 p1516 = f[15] + f[16], p1718 = f[17] + f[18];
-    const V2 q78 = f[7] - f[8], q910 = f[9] - f[10], q1112 = f[11] - f[12], q1314 = f[13] - f[14];
-    const V2 q1516 = f[15] - f[16], q1718 = f[17] - f[18];
-    const V2 exy = p78 + p910, exz = p1112 + p1314, eyz = p1516 + p1718;
-    const V2 s16 = (ax + ay) + az, s718 = (exy + exz) + eyz;
-    const V2 m1 = fma2(-30.0f, f[0], fma2(8.0f, s718, -11.0f * s16));
-    const V2 m2 = fma2(12.0f, f[0], fma2(-4.0f, s16, s718));
-    const V2 m4 = fma2(-4.0f, d12, (q78 + q910) + (q1112 + q1314));
-    const V2 m6 = fma2(-4.0f, d34, (q78 - q910) + (q1516 + q1718));
-    const V2 m8 = fma2(-4.0f, d56, (q1112 - q1314) + (q1516 - q1718));
-    const V2 exyz = exy + exz;
-    const V2 ayz = ay + az;
-    const V2 m9 = fma2(2.0f, ax, fma2(-2.0f, eyz, exyz - ayz));
-    const V2 m10 = fma2(-4.0f, ax, fma2(2.0f, ayz, fma2(-2.0f, eyz, exyz)));
-    const V2 m11 = (ay - az) + (exy - exz);
-    const V2 m12 = fma2(2.0f, az - ay, exy - exz);
-    const V2 m13 = p78 - p910, m14 = p1516 - p1718, m15 = p1112 - p1314;
-    const V2 m16 = (q78 + q910) - (q1112 + q1314);
-    const V2 m17 = (q910 - q78) + (q1516 + q1718);
-    const V2 m18 = (q1112 - q1314) - (q1516 - q1718);
+    const V ax = f[1] + f[2], ay = f[3] + f[4], az = f[5] + f[6];
+    const V d12 = f[1] - f[2], d34 = f[3] - f[4], d56 = f[5] - f[6];
+    const V p78 = f[7] + f[8], p910 = f[9] + f[10], p1112 = f[11] + f[12], p1314 = f[13] + f[14];
+    const V p1516 = f[15] + f[16], p1718 = f[17] + f[18];
+    const V q78 = f[7] - f[8], q910 = f[9] - f[10], q1112 = f[11] - f[12], q1314 = f[13] - f[14];
+    const V q1516 = f[15] - f[16], q1718 = f[17] - f[18];
+    const V exy = p78 + p910, exz = p1112 + p1314, eyz = p1516 + p1718;
+    const V s16 = (ax + ay) + az, s718 = (exy + exz) + eyz;
+    const V m1 = fma2(-30.0f, f[0], fma2(8.0f, s718, -11.0f * s16));
+    const V m2 = fma2(12.0f, f[0], fma2(-4.0f, s16, s718));
+    const V m4 = fma2(-4.0f, d12, (q78 + q910) + (q1112 + q1314));
+    const V m6 = fma2(-4.0f, d34, (q78 - q910) + (q1516 + q1718));
+    const V m8 = fma2(-4.0f, d56, (q1112 - q1314) + (q1516 - q1718));
+    const V exyz = exy + exz;
+    const V ayz = ay + az;
+    const V m9 = fma2(2.0f, ax, fma2(-2.0f, eyz, exyz - ayz));
+    const V m10 = fma2(-4.0f, ax, fma2(2.0f, ayz, fma2(-2.0f, eyz, exyz)));
+    const V m11 = (ay - az) + (exy - exz);
+    const V m12 = fma2(2.0f, az - ay, exy - exz);
+    const V m13 = p78 - p910, m14 = p1516 - p1718, m15 = p1112 - p1314;
+    const V m16 = (q78 + q910) - (q1112 + q1314);
+    const V m17 = (q910 - q78) + (q1516 + q1718);
+    const V m18 = (q1112 - q1314) - (q1516 - q1718);
     // equilibria (deviation form) and sources
-    const V2 uxx = ux * ux, uyy = uy * uy, uzz = uz * uz;
-    const V2 u2 = (uxx + uyy) + uzz;
-    const V2 rhou2 = rho * u2;
-    const V2 uF = fma2(ux, Fx, fma2(uy, Fy, uz * Fz));
-    const V2 e_eq = fma2(19.0f, rhou2, -11.0f * drho);
-    const V2 eps_eq = fma2(-5.5f, rhou2, 3.0f * drho);
-    const V2 a1 = fma2(k.k3e, X, fma2(k.k2e, uF, k.k1e * (m1 - e_eq)));
-    const V2 a2 = fma2(k.k3p, X, fma2(k.k2p, uF, k.k1p * (m2 - eps_eq)));
-    const V2 a4 = fma2(k.kq2, Fx, k.kq1 * fma2(2.0f / 3.0f, rho * ux, m4));
-    const V2 a6 = fma2(k.kq2, Fy, k.kq1 * fma2(2.0f / 3.0f, rho * uy, m6));
-    const V2 a8 = fma2(k.kq2, Fz, k.kq1 * fma2(2.0f / 3.0f, rho * uz, m8));
-    const V2 p3xx = rho * fma2(3.0f, uxx, -u2);
-    const V2 uyFy = uy * Fy, uzFz = uz * Fz;
-    const V2 S3xx = 2.0f * fma2(2.0f * ux, Fx, -(uyFy + uzFz));
-    const V2 a9 = fma2(k.kh9, S3xx, k.kn9 * (m9 - p3xx));
-    const V2 a10 = fma2(k.kh10, S3xx, k.kp10 * fma2(0.5f, p3xx, m10));
-    const V2 pww = rho * (uyy - uzz);
-    const V2 Sww = 2.0f * (uyFy - uzFz);
-    const V2 a11 = fma2(k.kh11, Sww, k.kn11 * (m11 - pww));
-    const V2 a12 = fma2(k.kh12, Sww, k.kp12 * fma2(0.5f, pww, m12));
-    const V2 a13 = fma2(k.kh13, fma2(ux, Fy, uy * Fx), k.kn13 * (m13 - rho * (ux * uy)));
-    const V2 a14 = fma2(k.kh13, fma2(uy, Fz, uz * Fy), k.kn13 * (m14 - rho * (uy * uz)));
-    const V2 a15 = fma2(k.kh13, fma2(ux, Fz, uz * Fx), k.kn13 * (m15 - rho * (ux * uz)));
-    const V2 a16 = k.km * m16, a17 = k.km * m17, a18 = k.km * m18;
-    const V2 a3 = 0.1f * Fx, a5 = 0.1f * Fy, a7 = 0.1f * Fz;
+    const V uxx = ux * ux, uyy = uy * uy, uzz = uz * uz;
+    const V u2 = (uxx + uyy) + uzz;
+    const V rhou2 = rho * u2;
+    const V uF = fma2(ux, Fx, fma2(uy, Fy, uz * Fz));
+    const V e_eq = fma2(19.0f, rhou2, -11.0f * drho);
+    const V eps_eq = fma2(-5.5f, rhou2, 3.0f * drho);
+    const V a1 = fma2(k.k3e, X, fma2(k.k2e, uF, k.k1e * (m1 - e_eq)));
+    const V a2 = fma2(k.k3p, X, fma2(k.k2p, uF, k.k1p * (m2 - eps_eq)));
+    const V a4 = fma2(k.kq2, Fx, k.kq1 * fma2(2.0f / 3.0f, rho * ux, m4));
+    const V a6 = fma2(k.kq2, Fy, k.kq1 * fma2(2.0f / 3.0f, rho * uy, m6));
+    const V a8 = fma2(k.kq2, Fz, k.kq1 * fma2(2.0f / 3.0f, rho * uz, m8));
+    const V p3xx = rho * fma2(3.0f, uxx, -u2);
+    const V uyFy = uy * Fy, uzFz = uz * Fz;
+    const V S3xx = 2.0f * fma2(2.0f * ux, Fx, -(uyFy + uzFz));
+    const V a9 = fma2(k.kh9, S3xx, k.kn9 * (m9 - p3xx));
+    const V a10 = fma2(k.kh10, S3xx, k.kp10 * fma2(0.5f, p3xx, m10));
+    const V pww = rho * (uyy - uzz);
+    const V Sww = 2.0f * (uyFy - uzFz);
+    const V a11 = fma2(k.kh11, Sww, k.kn11 * (m11 - pww));
+    const V a12 = fma2(k.kh12, Sww, k.kp12 * fma2(0.5f, pww, m12));
+    const V a13 = fma2(k.kh13, fma2(ux, Fy, uy * Fx), k.kn13 * (m13 - rho * (ux * uy)));
+    const V a14 = fma2(k.kh13, fma2(uy, Fz, uz * Fy), k.kn13 * (m14 - rho * (uy * uz)));
+    const V a15 = fma2(k.kh13, fma2(ux, Fz, uz * Fx), k.kn13 * (m15 - rho * (ux * uz)));
+    const V a16 = k.km * m16, a17 = k.km * m17, a18 = k.km * m18;
+    const V a3 = 0.1f * Fx, a5 = 0.1f * Fy, a7 = 0.1f * Fz;
     // f += M^T diag(1/|row|^2) (m* - m), columns of M per velocity
     f[0] = fma2(-30.0f, a1, fma2(12.0f, a2, f[0]));
-    const V2 axis = fma2(-11.0f, a1, -4.0f * a2);
-    const V2 a910 = fma2(-2.0f, a10, a9);                       // a9 - 2 a10
-    const V2 axx = fma2(2.0f, a910, axis);                      // axis + 2 a9 - 4 a10
-    const V2 r34 = fma2(-4.0f, a4, a3), r56 = fma2(-4.0f, a6, a5), r78 = fma2(-4.0f, a8, a7);
+    const V axis = fma2(-11.0f, a1, -4.0f * a2);
+    const V a910 = fma2(-2.0f, a10, a9);                       // a9 - 2 a10
+    const V axx = fma2(2.0f, a910, axis);                      // axis + 2 a9 - 4 a10
+    const V r34 = fma2(-4.0f, a4, a3), r56 = fma2(-4.0f, a6, a5), r78 = fma2(-4.0f, a8, a7);
     f[1] = f[1] + (axx + r34);
     f[2] = f[2] + (axx - r34);
-    const V2 a1112 = fma2(-2.0f, a12, a11);                     // a11 - 2 a12
-    const V2 ayy = (axis - a910) + a1112;
-    const V2 azz = (axis - a910) - a1112;
+    const V a1112 = fma2(-2.0f, a12, a11);                     // a11 - 2 a12
+    const V ayy = (axis - a910) + a1112;
+    const V azz = (axis - a910) - a1112;
     f[3] = f[3] + (ayy + r56);
     f[4] = f[4] + (ayy - r56);
     f[5] = f[5] + (azz + r78);
     f[6] = f[6] + (azz - r78);
-    const V2 edge = fma2(8.0f, a1, a2);
-    const V2 b910 = a9 + a10, b1112 = a11 + a12;
-    const V2 exy0 = (edge + b910) + b1112, exz0 = (edge + b910) - b1112;
-    const V2 eyz0 = fma2(-2.0f, b910, edge);
-    const V2 t34 = a3 + a4, t56 = a5 + a6, t78 = a7 + a8;
-    const V2 g1 = t34 + t56, g2 = t34 - t56;
-    const V2 h1 = a16 - a17, h2 = a16 + a17;
+    const V edge = fma2(8.0f, a1, a2);
+    const V b910 = a9 + a10, b1112 = a11 + a12;
+    const V exy0 = (edge + b910) + b1112, exz0 = (edge + b910) - b1112;
+    const V eyz0 = fma2(-2.0f, b910, edge);
+    const V t34 = a3 + a4, t56 = a5 + a6, t78 = a7 + a8;
+    const V g1 = t34 + t56, g2 = t34 - t56;
+    const V h1 = a16 - a17, h2 = a16 + a17;
     f[7] = f[7] + ((exy0 + a13) + (g1 + h1));
     f[8] = f[8] + ((exy0 + a13) - (g1 + h1));
     f[9] = f[9] + ((exy0 - a13) + (g2 + h2));
     f[10] = f[10] + ((exy0 - a13) - (g2 + h2));
-    const V2 g3 = t34 + t78, g4 = t34 - t78;
-    const V2 h3 = a18 - a16, h4 = a16 + a18;
+    const V g3 = t34 + t78, g4 = t34 - t78;
+    const V h3 = a18 - a16, h4 = a16 + a18;
     f[11] = f[11] + ((exz0 + a15) + (g3 + h3));
     f[12] = f[12] + ((exz0 + a15) - (g3 + h3));
     f[13] = f[13] + ((exz0 - a15) + (g4 - h4));
     f[14] = f[14] + ((exz0 - a15) - (g4 - h4));
-    const V2 g5 = t56 + t78, g6 = t56 - t78;
-    const V2 h5 = a17 - a18, h6 = a17 + a18;
+    const V g5 = t56 + t78, g6 = t56 - t78;
+    const V h5 = a17 - a18, h6 = a17 + a18;
     f[15] = f[15] + ((eyz0 + a14) + (g5 + h5));
     f[16] = f[16] + ((eyz0 + a14) - (g5 + h5));
     f[17] = f[17] + ((eyz0 - a14) + (g6 + h6));
@@ -198,7 +199,8 @@ __device__ __forceinline__ void zpair_chunk(const float* __restrict__ fin, float
     constexpr int Q = 19, TX = ZTX, TY = ZTY, NT = TX * TY;
     using Sm = ZPSmem<TX, TY>;
     constexpr int YX = Sm::YX, YY = Sm::YY, RX = Sm::RX, RY = Sm::RY, PX = Sm::PX, PY = Sm::PY;
-    const int nx = g.nx, ny = g.ny, nz = g.nz, N = g.N, nxy = nx * ny;
+    const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
+    const int fp = g.fp, fxy = fp * ny;   // distributions: row pitch and plane stride
     const int ze = min(zb + ZCH, nz);
     const int lx = threadIdx.x, ly = threadIdx.y, tid = ly * TX + lx;
     const bool small = nx < TX + 8 || ny < TY + 8 || nz < 8;
@@ -220,12 +222,12 @@ __device__ __forceinline__ void zpair_chunk(const float* __restrict__ fin, float
     // sources of node (gx, gy, gz) of plane z (type cell ti): sink(a, pointer)
     auto pull_src = [&](auto&& sink, int gx, int gy, int gz, int z, int ti, uint8_t self) {
         const int cx[3] = {wrap1(gx - 1, nx), gx, wrap1(gx + 1, nx)};
-        const int ry[3] = {wrap1(gy - 1, ny) * nx, gy * nx, wrap1(gy + 1, ny) * nx};
-        const int pz[3] = {wrap1(gz - 1, nz) * nxy, gz * nxy, wrap1(gz + 1, nz) * nxy};
+        const int ry[3] = {wrap1(gy - 1, ny) * fp, gy * fp, wrap1(gy + 1, ny) * fp};
+        const int pz[3] = {wrap1(gz - 1, nz) * fxy, gz * fxy, wrap1(gz + 1, nz) * fxy};
         if (!SOLID || (self & T_BULK)) {
 #pragma unroll
             for (int a = 0; a < Q; ++a)
-                sink(a, fin + (a * N + pz[1 - L::ez(a)] + ry[1 - L::ey(a)] + cx[1 - L::ex(a)]));
+                sink(a, fin + (a * g.fs + pz[1 - L::ez(a)] + ry[1 - L::ey(a)] + cx[1 - L::ex(a)]));
         } else {
             const uint8_t* tm = sm.type[(z - 1) & 7];
             const uint8_t* t0 = sm.type[z & 7];
@@ -235,7 +237,7 @@ __device__ __forceinline__ void zpair_chunk(const float* __restrict__ fin, float
                 const int ex = L::ex(a), ey = L::ey(a), ez = L::ez(a);
                 const uint8_t* tz = ez > 0 ? tm : (ez < 0 ? tp : t0);   // upstream plane is z - ez
                 const bool bb = (tz[ti - ex - ey * YX] & T_SOLID) != 0;
-                sink(a, fin + (bb ? L::opp(a) * N + pz[1] + ry[1] + cx[1] : a * N + pz[1 - ez] + ry[1 - ey] + cx[1 - ex]));
+                sink(a, fin + (bb ? L::opp(a) * g.fs + pz[1] + ry[1] + cx[1] : a * g.fs + pz[1 - ez] + ry[1 - ey] + cx[1 - ex]));
             }
         }
     };
@@ -442,11 +444,11 @@ __device__ __forceinline__ void zpair_chunk(const float* __restrict__ fin, float
                 const V2 ux = fma2(0.5f, Fx, jx) * inv, uy = fma2(0.5f, Fy, jy) * inv, uz = fma2(0.5f, Fz, jz) * inv;
                 const V2 X = div2(fma2(Fmx, Fmx, fma2(Fmy, Fmy, Fmz * Fmz)), psi_c * psi_c);
                 collide3p(f, drho, rho, ux, uy, uz, Fx, Fy, Fz, X, kr);
-                const int gi = zc * nxy + (y0 + ly) * nx + x0 + lx;
+                const int gi = zc * fxy + (y0 + ly) * fp + x0 + lx;
 #pragma unroll
                 for (int a = 0; a < Q; ++a) {
-                    if (fl0) fout[a * N + gi] = f[a].v.x;
-                    if (fl1) fout[a * N + gi + nxy] = f[a].v.y;
+                    if (fl0) fout[a * g.fs + gi] = f[a].v.x;
+                    if (fl1) fout[a * g.fs + gi + fxy] = f[a].v.y;
                 }
             }
         }
@@ -475,9 +477,10 @@ __global__ void __launch_bounds__(ZTX* ZTY, LBMWET_ZP_MINB)
 
 
 // ---------------------------------------------------------------------------------------------
-// TMA-staged z-march (the default FP32 D3Q19 step).  A CTA of 32 x 4 threads owns a 32 x 8 column
-// of a 32-plane chunk; thread (lx, ly) carries the cells (x0 + lx, y0 + ly) and (x0 + lx, y0 + ly + 4)
-// as the two lanes of its FP32x2 values.  The chunk marches plane by plane through shared memory:
+// TMA-staged z-march (the default FP32 D3Q19 step, and its fields pass).  A CTA of 32 x 8 threads owns a
+// 32 x 8 column, one cell per thread, over the planes of a work item, and marches plane by plane through
+// shared memory.  (128 threads with two cells each in packed FP32x2 arithmetic take the same time on 256^3,
+// 532 against 536 us, and longer where items are few: 64^3 42.7 against 39.8, 128^3 124 against 108.)
 //   * every lead plane zl is staged by TMA: for each direction a, the box of f*_a on plane zl - ez(a)
 //     over x0 - 4 .. x0 + 35 (x starts on a 16-byte boundary) and y0 - 2 .. y0 + 9 (y0 - 3 .. y0 + 10
 //     in chunks holding solids, whose walls need densities two nodes out), so that the pull (Eq. 3)
@@ -497,10 +500,11 @@ __global__ void __launch_bounds__(ZTX* ZTY, LBMWET_ZP_MINB)
 //   * phase C collides plane zl - 1 (zl - 2 in chunks holding solids) once its psi neighbours are
 //     final: F_m (Eq. 5; plus Eq. 8 with the solid-fluid interaction scheme), u (Eq. 4), the MRT
 //     collision with the consistency source (Eqs. 2, 7), coalesced stores.
-// Ragged edge columns and small grids take the z-pair march on the column's two 32 x 4 halves.
+// Grids smaller than a box (ztma_marches) take the z-pair march.
 // ---------------------------------------------------------------------------------------------
 constexpr int TTX = 32, TTY = 8, TCH = ZCH;
 static_assert(TTX == ZTX && TTY == 2 * ZTY, "a TMA column is two z-pair columns");
+constexpr int TNT = TTX * TTY;                // threads: one per cell
 constexpr int TBX = TTX + 8;                  // box columns: x0 - 4 .. x0 + 35
 constexpr int TBY = TTY + 4;                  // box rows: y0 - 2 .. y0 + 9
 constexpr int TBSLOT = TBY * TBX;             // floats per direction and stage, chunks without solids (480)
@@ -542,7 +546,7 @@ struct ZTSmem {
     };
     uint64_t bar[2];
 };
-constexpr size_t ZT_SMEM = sizeof(ZTSmem) > sizeof(ZPSmem<ZTX, ZTY>) ? sizeof(ZTSmem) : sizeof(ZPSmem<ZTX, ZTY>);
+constexpr size_t ZT_SMEM = sizeof(ZTSmem);
 
 // Polls of an mbarrier before a wait gives up (about one second at ~3.8 us per unsuccessful poll).
 constexpr unsigned ZT_POLL_LIMIT = 1u << 18;
@@ -606,63 +610,83 @@ struct OutBand {
     }
 };
 
+// Where the fields pass (MODE 1) writes a node's density and velocity; either may be null.
+struct ZTOut {
+    double* rho;
+    double* u;
+    int N;
+    __device__ __forceinline__ void node(int g, float r, float ux, float uy, float uz) const {
+        if (rho) rho[g] = double(r);
+        if (u) {
+            u[g] = double(ux);
+            u[N + g] = double(uy);
+            u[2 * N + g] = double(uz);
+        }
+    }
+};
+
 // A chunk without solids within 3 nodes: no walls, no bounce-back; lag 1 between the lead plane
 // and the collided plane.
+template <int MODE>
 __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, float* __restrict__ fout,
                                                 const void* tmap, const Geo& g, const Phys<float>& ph,
-                                                const Rates3P& kr, int x0, int y0, int zb, int ze, unsigned* err,
-                                                ZTBulk& S, uint64_t* bar) {
+                                                const Rates3P& kr, int x0, int y0, int xs, int ys, int zb, int ze,
+                                                unsigned* err, ZTBulk& S, uint64_t* bar, const ZTOut& out) {
     using L = D3Q19;
     constexpr int Q = 19;
-    const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
+    const int nx = g.nx, ny = g.ny, nz = g.nz, fp = g.fp, fxy = fp * ny;   // (fp: row pitch of the distributions)
     const long long fs = g.fs;
     const int lx = threadIdx.x, ly = threadIdx.y, tid = ly * TTX + lx;
     const int zlo = zb - 1, zhi = ze;   // lead planes zlo .. zhi, collided planes zb .. ze - 1
     const int nlead = zhi - zlo + 1;
 
-    // out-of-range cells of the used window (rows 0 .. 11, columns 2 .. 37): at most
-    // 2 * 36 + 2 * 10 = 92 < 128, one per thread, prefetched one plane ahead
+    // out-of-range cells of the used window (rows 0 .. 11, columns 2 .. 37): at most 2 rows and 5 columns,
+    // 2 * 36 + 5 * 10 = 122 < 128, one per thread, prefetched one plane ahead
     const OutBand ob_(x0 - 4, y0 - 2, nx, ny, 0, TBY, 2, TBX - 2);
     const bool edge = ob_.cells > 0;
     int fr = 0, fcl = 0, fsrc = 0;
     const bool fixer = tid < ob_.cells;
     if (fixer) {
         ob_.cell(tid, 2, fr, fcl);
-        fsrc = wrap_full(y0 - 2 + fr, ny) * nx + wrap_full(x0 - 4 + fcl, nx);
+        fsrc = wrap_full(y0 - 2 + fr, ny) * fp + wrap_full(x0 - 4 + fcl, nx);
     }
     float fix[Q];
-    auto issue = [&](int zl, int s) {   // thread 0: the 19 boxes of lead plane zl into stage s
+    // lane 0 of every warp: its share of the 19 boxes of lead plane zl into stage s (one thread issuing them
+    // all held its warp, and the barrier behind it, for 19 instructions)
+    auto issue = [&](int zl, int s) {
         fence_proxy_async();
-        mbar_expect_tx(&bar[s], TBYTES_BULK);
-#pragma unroll
-        for (int a = 0; a < Q; ++a) tma_box3(S.stage[s][a], tmap, x0 - 4, y0 - 2, a * nz + wrap1(zl - L::ez(a), nz), &bar[s]);
+        if (ly == 0) mbar_expect_tx(&bar[s], TBYTES_BULK);
+        for (int a = ly; a < Q; a += TTY)
+            tma_box3(S.stage[s][a], tmap, x0 - 4, y0 - 2, a * nz + wrap1(zl - ez_rt(a), nz), &bar[s]);
     };
 
-    if (tid == 0) {
+    if (lx == 0) {
         issue(zlo, 0);
         issue(zlo + 1, 1);
     }
     if (edge && fixer) {
 #pragma unroll
-        for (int a = 0; a < Q; ++a) fix[a] = fin[a * fs + (long long)wrap1(zlo - L::ez(a), nz) * nxy + fsrc];
+        for (int a = 0; a < Q; ++a) fix[a] = fin[a * fs + (long long)wrap1(zlo - L::ez(a), nz) * fxy + fsrc];
     }
 
     // own cells in box and psi-window coordinates
     const int ob = (ly + 2) * TBX + lx + 4;
     const int pc = (ly + 1) * TPX + lx + 1;
-    // this thread's halo-ring cell (threads 0 .. 83)
+    // the nodes this item writes (a column moved inside the grid shares some with its neighbours)
+    const bool wr = x0 + lx >= xs && x0 + lx < nx && y0 + ly >= ys;
+    // this thread's halo-ring cell (the last 84 threads; the first ones patch the edges)
     int rb = 0, rp = 0;
-    const bool ringer = tid < TRING;
+    const bool ringer = TNT - 1 - tid < TRING;
     if (ringer) {
         int px, py, pz;
-        Shell<TPX, TPY, 1, 2>::cell(tid, px, py, pz);
+        Shell<TPX, TPY, 1, 2>::cell(TNT - 1 - tid, px, py, pz);
         rb = (py + 1) * TBX + px + 3;
         rp = py * TPX + px;
     }
 
-    V2 fprev[Q];
+    V1 fprev[Q];
 #pragma unroll
-    for (int a = 0; a < Q; ++a) fprev[a] = bc(0.0f);
+    for (int a = 0; a < Q; ++a) fprev[a].v = 0.0f;
 
 #pragma unroll 1
     for (int i = 0; i < nlead; ++i) {
@@ -678,77 +702,73 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
             if (fixer && zl + 1 <= zhi) {
 #pragma unroll
                 for (int a = 0; a < Q; ++a)
-                    fix[a] = fin[a * fs + (long long)wrap1(zl + 1 - L::ez(a), nz) * nxy + fsrc];
+                    fix[a] = fin[a * fs + (long long)wrap1(zl + 1 - L::ez(a), nz) * fxy + fsrc];
             }
             __syncthreads();
         }
         // A. rho and psi of lead plane zl: the column (own values kept) and its halo ring
-        V2 fcur[Q];
+        V1 fcur[Q];
 #pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            const int off = a * TBSLOT - L::ey(a) * TBX - L::ex(a);
-            fcur[a] = mk(st[ob + off], st[ob + 4 * TBX + off]);
-        }
+        for (int a = 0; a < Q; ++a) fcur[a].v = st[ob + a * TBSLOT - L::ey(a) * TBX - L::ex(a)];
         {
-            V2 d = fcur[0];
+            V1 d = fcur[0];
 #pragma unroll
             for (int a = 1; a < Q; ++a) d = d + fcur[a];
-            const V2 ps = psi2(bc(ph.rho_ref) + d, ph, true, true, err);
-            float* pp = S.psi[zl & 3];
-            pp[pc] = ps.v.x;
-            pp[pc + 4 * TPX] = ps.v.y;
+            S.psi[zl & 3][pc] = psi1(V1{ph.rho_ref} + d, ph, err).v;
         }
         if (ringer) {
-            float d = 0.0f;
+            V1 d = {st[rb]};
 #pragma unroll
-            for (int a = 0; a < Q; ++a) d += st[rb + a * TBSLOT - L::ey(a) * TBX - L::ex(a)];
-            S.psi[zl & 3][rp] = psi_checked(ph.rho_ref + d, ph, err);
+            for (int a = 1; a < Q; ++a) d = d + V1{st[rb + a * TBSLOT - L::ey(a) * TBX - L::ex(a)]};
+            S.psi[zl & 3][rp] = psi1(V1{ph.rho_ref} + d, ph, err).v;
         }
         __syncthreads();
-        if (tid == 0 && zl + 2 <= zhi) issue(zl + 2, s);
+        if (lx == 0 && zl + 2 <= zhi) issue(zl + 2, s);
 
         // C. collide plane zc = zl - 1
         const int zc = zl - 1;
         if (zc >= zb) {
-            V2(&f)[Q] = fprev;
+            V1(&f)[Q] = fprev;
             auto psi_at = [&](int dz, int off) {
-                const float* pp = S.psi[(zc + dz) & 3];
-                return mk(pp[pc + off], pp[pc + 4 * TPX + off]);
+                return V1{S.psi[(zc + dz) & 3][pc + off]};
             };
-            const V2 psi_c = psi_at(0, 0);
-            V2 sx = bc(0.0f), sy = bc(0.0f), sz = bc(0.0f);
+            const V1 psi_c = psi_at(0, 0);
+            V1 sx = {0.0f}, sy = {0.0f}, sz = {0.0f};
 #pragma unroll
             for (int a = 1; a < Q; ++a) {
                 if (L::opp(a) < a) continue;
                 const int ex = L::ex(a), ey = L::ey(a), ez = L::ez(a);
                 const int off = ex + ey * TPX;
-                const V2 wd = float(L::wf(a)) * (psi_at(ez, off) - psi_at(-ez, -off));
+                const V1 wd = float(L::wf(a)) * (psi_at(ez, off) - psi_at(-ez, -off));
                 if (ex) sx = ex > 0 ? sx + wd : sx - wd;
                 if (ey) sy = ey > 0 ? sy + wd : sy - wd;
                 if (ez) sz = ez > 0 ? sz + wd : sz - wd;
             }
             // Eq. 5
-            const V2 gpsi = (-ph.G) * psi_c;
-            const V2 Fmx = gpsi * sx, Fmy = gpsi * sy, Fmz = gpsi * sz;
-            const V2 Fx = Fmx + bc(ph.fx), Fy = Fmy + bc(ph.fy), Fz = Fmz + bc(ph.fz);
-            V2 drho = f[0];
+            const V1 gpsi = (-ph.G) * psi_c;
+            const V1 Fmx = gpsi * sx, Fmy = gpsi * sy, Fmz = gpsi * sz;
+            const V1 Fx = Fmx + V1{ph.fx}, Fy = Fmy + V1{ph.fy}, Fz = Fmz + V1{ph.fz};
+            V1 drho = f[0];
 #pragma unroll
             for (int a = 1; a < Q; ++a) drho = drho + f[a];
-            const V2 jx = ((f[1] - f[2]) + (f[7] - f[8])) + ((f[9] - f[10]) + (f[11] - f[12])) + (f[13] - f[14]);
-            const V2 jy = ((f[3] - f[4]) + (f[7] - f[8])) + ((f[10] - f[9]) + (f[15] - f[16])) + (f[17] - f[18]);
-            const V2 jz = ((f[5] - f[6]) + (f[11] - f[12])) + ((f[14] - f[13]) + (f[15] - f[16])) + (f[18] - f[17]);
-            const V2 rho = bc(ph.rho_ref) + drho;
-            if (!(rho.v.x > 0.0f) || !(rho.v.y > 0.0f)) atomicOr(err, ERR_RHO);
+            const V1 jx = ((f[1] - f[2]) + (f[7] - f[8])) + ((f[9] - f[10]) + (f[11] - f[12])) + (f[13] - f[14]);
+            const V1 jy = ((f[3] - f[4]) + (f[7] - f[8])) + ((f[10] - f[9]) + (f[15] - f[16])) + (f[17] - f[18]);
+            const V1 jz = ((f[5] - f[6]) + (f[11] - f[12])) + ((f[14] - f[13]) + (f[15] - f[16])) + (f[18] - f[17]);
+            const V1 rho = V1{ph.rho_ref} + drho;
+            if (!(rho.v > 0.0f)) atomicOr(err, ERR_RHO);
             // Eq. 4: rho u = sum e f + F/2
-            const V2 inv = div2(bc(1.0f), rho);
-            const V2 ux = fma2(0.5f, Fx, jx) * inv, uy = fma2(0.5f, Fy, jy) * inv, uz = fma2(0.5f, Fz, jz) * inv;
-            const V2 X = div2(fma2(Fmx, Fmx, fma2(Fmy, Fmy, Fmz * Fmz)), psi_c * psi_c);
-            collide3p(f, drho, rho, ux, uy, uz, Fx, Fy, Fz, X, kr);
-            float* o = fout + (long long)zc * nxy + (y0 + ly) * nx + x0 + lx;
+            const V1 inv = div2(V1{1.0f}, rho);
+            const V1 ux = fma2(0.5f, Fx, jx) * inv, uy = fma2(0.5f, Fy, jy) * inv, uz = fma2(0.5f, Fz, jz) * inv;
+            if constexpr (MODE == 1) {
+                if (wr) out.node((zc * ny + y0 + ly) * nx + x0 + lx, rho.v, ux.v, uy.v, uz.v);
+            } else {
+                const V1 X = div2(fma2(Fmx, Fmx, fma2(Fmy, Fmy, Fmz * Fmz)), psi_c * psi_c);
+                collide3p(f, drho, rho, ux, uy, uz, Fx, Fy, Fz, X, kr);
+                float* o = fout + (long long)zc * fxy + (y0 + ly) * fp + x0 + lx;
+                if (wr) {
 #pragma unroll
-            for (int a = 0; a < Q; ++a) {
-                o[a * fs] = f[a].v.x;
-                o[a * fs + 4 * nx] = f[a].v.y;
+                    for (int a = 0; a < Q; ++a) o[a * fs] = f[a].v;
+                }
             }
         }
 #pragma unroll
@@ -759,14 +779,14 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
 // A chunk holding solids within 3 nodes: node types of planes zl - 3 .. zl + 2 in a ring, bounce-back
 // links, a 2-node density ring for the wall cells' Eq. 17, lag 2 between lead and collided plane.
 // Coordinates (rb, c) are those of the box: row rb is grid row y0 - 2 + rb, column c is x0 - 4 + c.
-template <bool SF>
+template <bool SF, int MODE>
 __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, float* __restrict__ fout,
                                                  const void* tmap, const Geo& g, const Phys<float>& ph,
-                                                 const Rates3P& kr, int x0, int y0, int zb, int ze, unsigned* err,
-                                                 ZTSolid& S, uint64_t* bar) {
+                                                 const Rates3P& kr, int x0, int y0, int xs, int ys, int zb, int ze,
+                                                 unsigned* err, ZTSolid& S, uint64_t* bar, const ZTOut& out) {
     using L = D3Q19;
-    constexpr int Q = 19, NT = TTX * ZTY;
-    const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
+    constexpr int Q = 19, NT = TNT;
+    const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny, fp = g.fp, fxy = fp * ny;
     const long long fs = g.fs;
     const int lx = threadIdx.x, ly = threadIdx.y, tid = ly * TTX + lx;
     const int zlo = zb - 2, zhi = ze + 1;   // lead planes; collided planes zb .. ze - 1
@@ -783,24 +803,39 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
     auto xrow_src = [&](int z, int k) {
         const int row = k / 190, rem = k - row * 190, d = rem / 38, col = 1 + rem % 38;
         const int a = int(((row ? XROW_DN : XROW_UP) >> (5 * d)) & 31u);
-        return fin[a * fs + (long long)wz(z - ez_rt(a)) * nxy + wrap1(row ? y0 + 10 : y0 - 3, ny) * nx +
+        return fin[a * fs + (long long)wz(z - ez_rt(a)) * fxy + wrap1(row ? y0 + 10 : y0 - 3, ny) * fp +
                    wrap1(x0 - 4 + col, nx)];
     };
     auto xrow_dst = [&](int z, int k) -> float& {
         const int row = k / 190, rem = k - row * 190, d = rem / 38, col = 1 + rem % 38;
         return S.xrow[z & 1][row][d][col];
     };
-    // out-of-range cells of the used window (rows 0 .. 11, columns 1 .. 38), written after each
-    // wait from plain loads (chunks holding solids rarely touch the grid's edges)
+    // out-of-range cells of the used window (rows 0 .. 11, columns 1 .. 38): at most 2 rows and 6 columns, 136
+    // cells; a thread's first cell is loaded before each wait, the few beyond NT after it, all directions of
+    // a cell together (one at a time, the loads' latencies added up to 9 us a plane)
     const OutBand band(x0 - 4, y0 - 2, nx, ny, 0, TBY, 1, TBX - 1);
     const bool edge = band.cells > 0;
-    auto issue = [&](int zl, int s) {   // thread 0: the 19 boxes of lead plane zl into stage s
-        fence_proxy_async();
-        mbar_expect_tx(&bar[s], TBYTES_BULK);
+    auto band_load = [&](int k, int zl, float (&v)[Q]) {
+        int rb, c;
+        band.cell(k, 1, rb, c);
+        const float* p = fin + (long long)wrap1(y0 - 2 + rb, ny) * fp + wrap1(x0 - 4 + c, nx);
+        const int pz[3] = {wz(zl - 1) * fxy, wz(zl) * fxy, wz(zl + 1) * fxy};
 #pragma unroll
-        for (int a = 0; a < Q; ++a) tma_box3(S.stage[s][a], tmap, x0 - 4, y0 - 2, a * nz + wz(zl - L::ez(a)), &bar[s]);
+        for (int a = 0; a < Q; ++a) v[a] = p[a * fs + pz[1 - L::ez(a)]];
     };
-    if (tid == 0) {
+    auto band_store = [&](int k, float* st, const float (&v)[Q]) {
+        int rb, c;
+        band.cell(k, 1, rb, c);
+#pragma unroll
+        for (int a = 0; a < Q; ++a) st[a * TBSLOT + rb * TBX + c] = v[a];
+    };
+    auto issue = [&](int zl, int s) {   // lane 0 of every warp, as in bulk
+        fence_proxy_async();
+        if (ly == 0) mbar_expect_tx(&bar[s], TBYTES_BULK);
+        for (int a = ly; a < Q; a += TTY)
+            tma_box3(S.stage[s][a], tmap, x0 - 4, y0 - 2, a * nz + wz(zl - ez_rt(a)), &bar[s]);
+    };
+    if (lx == 0) {
         issue(zlo, 0);
         issue(zlo + 1, 1);
     }
@@ -811,7 +846,7 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
 
     // post-collision value f*_{opp(a)} of box cell (rb, c) on plane z (bounce-back source)
     auto bb_src = [&](int a, int z, int rb, int c) {
-        return fin[L::opp(a) * fs + (long long)wz(z) * nxy + wrap1(y0 - 2 + rb, ny) * nx + wrap1(x0 - 4 + c, nx)];
+        return fin[L::opp(a) * fs + (long long)wz(z) * fxy + wrap1(y0 - 2 + rb, ny) * fp + wrap1(x0 - 4 + c, nx)];
     };
     // pull of a fluid cell (rb, c) of plane zl with its type t; RING2: the cell may lie on box row 0
     // or 11, whose pulls reach the rows beyond the box
@@ -848,34 +883,35 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
     const int pc = (ly + 1) * TPX + lx + 1;   // own cell in the psi window
     const int rc = (ly + 2) * TRX + lx + 2;   // own cell in the density window
     const int tcl = (ly + 3) * TYX + lx + 3;  // own cell in the type window
-    V2 f1[Q], f2[Q];                          // own values of planes zl - 1 and zl - 2
+    V1 f1[Q], f2[Q];                          // own values of planes zl - 1 and zl - 2
 #pragma unroll
-    for (int a = 0; a < Q; ++a) f1[a] = f2[a] = bc(0.0f);
-    uint8_t tnext[5];                         // types of plane zl + 2 (this thread's cells)
-    float xnext[3];                           // the rows beyond the box of plane zl + 1
+    for (int a = 0; a < Q; ++a) f1[a].v = f2[a].v = 0.0f;
+    constexpr int TN = (TTYPES + NT - 1) / NT, XN = (380 + NT - 1) / NT;
+    uint8_t tnext[TN];                        // types of plane zl + 2 (this thread's cells)
+    float xnext[XN];                          // the rows beyond the box of plane zl + 1
 
 #pragma unroll 1
     for (int i = 0; i < nlead; ++i) {
         const int zl = zlo + i, s = i & 1;
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {
+        for (int j = 0; j < TN; ++j) {
             const int k = tid + j * NT;
             tnext[j] = k < TTYPES ? type_src(zl + 2, k) : uint8_t(0);
         }
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
+        for (int j = 0; j < XN; ++j) {
             const int k = tid + j * NT;
             xnext[j] = (k < 380 && zl + 1 <= zhi) ? xrow_src(zl + 1, k) : 0.0f;
         }
+        float patch[Q];
+        if (edge && tid < band.cells) band_load(tid, zl, patch);
         if (!mbar_wait(&bar[s], unsigned(i >> 1) & 1u, ZT_POLL_LIMIT)) atomicOr(err, ERR_TIMEOUT);
         float* st = S.stage[s][0];
         if (edge) {
-            for (int k = tid; k < band.cells * Q; k += NT) {
-                const int a = k / band.cells;
-                int rb, c;
-                band.cell(k - a * band.cells, 1, rb, c);
-                st[a * TBSLOT + rb * TBX + c] =
-                    fin[a * fs + (long long)wz(zl - ez_rt(a)) * nxy + wrap1(y0 - 2 + rb, ny) * nx + wrap1(x0 - 4 + c, nx)];
+            if (tid < band.cells) band_store(tid, st, patch);
+            for (int k = tid + NT; k < band.cells; k += NT) {
+                band_load(k, zl, patch);
+                band_store(k, st, patch);
             }
             fence_proxy_async();
             __syncthreads();
@@ -890,41 +926,30 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
         const uint8_t* ty = S.type[zl & 7];
         float* rr = S.rho[zl & 3];
         float* pp = S.psi[ps5(zl)];
-        V2 fcur[Q];
+        V1 fcur[Q];
         {
             float v[Q];
-            const uint8_t t0 = ty[tcl], t1 = ty[tcl + 4 * TYX];
-            const bool fl0 = !(t0 & T_SOLID), fl1 = !(t1 & T_SOLID);
-            float d0 = 0.0f, d1 = 0.0f;
-            if (fl0) {
-                pull(NoRing2{}, st, stn, zl, ly + 2, lx + 4, t0, v);
+            const uint8_t t = ty[tcl];
+            const bool fl = !(t & T_SOLID);
+            V1 rho = {0.0f}, ps = {0.0f};
+            if (fl) {
+                pull(NoRing2{}, st, stn, zl, ly + 2, lx + 4, t, v);
+                V1 d = {v[0]};
 #pragma unroll
-                for (int a = 0; a < Q; ++a) d0 += v[a];
+                for (int a = 1; a < Q; ++a) d = d + V1{v[a]};
+                rho = V1{ph.rho_ref} + d;
+                ps = psi1(rho, ph, err);
             } else {
 #pragma unroll
                 for (int a = 0; a < Q; ++a) v[a] = 0.0f;
             }
 #pragma unroll
-            for (int a = 0; a < Q; ++a) fcur[a].v.x = v[a];
-            if (fl1) {
-                pull(NoRing2{}, st, stn, zl, ly + 6, lx + 4, t1, v);
-#pragma unroll
-                for (int a = 0; a < Q; ++a) d1 += v[a];
-            } else {
-#pragma unroll
-                for (int a = 0; a < Q; ++a) v[a] = 0.0f;
-            }
-#pragma unroll
-            for (int a = 0; a < Q; ++a) fcur[a].v.y = v[a];
-            const V2 rho = mk(ph.rho_ref + d0, ph.rho_ref + d1);
-            const V2 ps = psi2(rho, ph, fl0, fl1, err);
-            rr[rc] = fl0 ? rho.v.x : 0.0f;
-            rr[rc + 4 * TRX] = fl1 ? rho.v.y : 0.0f;
-            pp[pc] = fl0 ? ps.v.x : 0.0f;
-            pp[pc + 4 * TPX] = fl1 ? ps.v.y : 0.0f;
+            for (int a = 0; a < Q; ++a) fcur[a].v = v[a];
+            rr[rc] = rho.v;
+            pp[pc] = ps.v;
         }
         // halo cells: the 1-node ring (density and psi) and the 2-node ring (density)
-        for (int k = tid; k < TRING + TRING2; k += NT) {
+        for (int k = NT - 1 - tid; k < TRING + TRING2; k += NT) {   // (the first threads patch the edges)
             int px, py, pz, rb, c;
             if (k < TRING) {
                 Shell<TPX, TPY, 1, 2>::cell(k, px, py, pz);
@@ -941,16 +966,16 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
             if (fl) {
                 float v[Q];
                 pull(Ring2{}, st, stn, zl, rb, c, t, v);
-                float d = 0.0f;
+                V1 d = {v[0]};
 #pragma unroll
-                for (int a = 0; a < Q; ++a) d += v[a];
-                rho = ph.rho_ref + d;
+                for (int a = 1; a < Q; ++a) d = d + V1{v[a]};
+                rho = (V1{ph.rho_ref} + d).v;
             }
             rr[rb * TRX + c - 2] = rho;
-            if (k < TRING) pp[(rb - 1) * TPX + c - 3] = fl ? psi_checked(rho, ph, err) : 0.0f;
+            if (k < TRING) pp[(rb - 1) * TPX + c - 3] = fl ? psi1(V1{rho}, ph, err).v : 0.0f;
         }
         __syncthreads();
-        if (tid == 0 && zl + 2 <= zhi) issue(zl + 2, s);
+        if (lx == 0 && zl + 2 <= zhi) issue(zl + 2, s);
 
         // B. wall cells of plane zw = zl - 1: virtual density and its psi (the solid-fluid interaction
         // scheme keeps psi = 0 on solids); node types of plane zl + 2 and the rows beyond the box of
@@ -985,16 +1010,16 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
                     rw = raw > ph.rho_l ? ph.rho_l : raw;
                     rw = rw < ph.rho_g ? ph.rho_g : rw;
                 }
-                S.psi[ps5(zw)][k] = psi_checked(rw, ph, err);
+                S.psi[ps5(zw)][k] = psi1(V1{rw}, ph, err).v;
             }
         }
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {
+        for (int j = 0; j < TN; ++j) {
             const int k = tid + j * NT;
             if (k < TTYPES) S.type[(zl + 2) & 7][k] = tnext[j];
         }
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
+        for (int j = 0; j < XN; ++j) {
             const int k = tid + j * NT;
             if (k < 380) xrow_dst(zl + 1, k) = xnext[j];
         }
@@ -1004,71 +1029,71 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
         const int zc = zl - 2;
         if (zc >= zb) {
             const uint8_t* tc = S.type[zc & 7];
-            const bool fl0 = !(tc[tcl] & T_SOLID), fl1 = !(tc[tcl + 4 * TYX] & T_SOLID);
-            if (fl0 || fl1) {
-                V2(&f)[Q] = f2;
+            const bool in = x0 + lx >= xs && x0 + lx < nx && y0 + ly >= ys;
+            const bool fl = !(tc[tcl] & T_SOLID);
+            if constexpr (MODE == 1) {
+                if (in && !fl) out.node(zc * nxy + (y0 + ly) * nx + x0 + lx, 0.0f, 0.0f, 0.0f, 0.0f);
+            }
+            if (fl) {
+                V1(&f)[Q] = f2;
                 auto psi_at = [&](int dz, int off) {
-                    const float* q = S.psi[ps5(zc + dz)];
-                    return mk(q[pc + off], q[pc + 4 * TPX + off]);
+                    return V1{S.psi[ps5(zc + dz)][pc + off]};
                 };
-                const V2 psi_c = psi_at(0, 0);
-                V2 sx = bc(0.0f), sy = bc(0.0f), sz = bc(0.0f);
+                const V1 psi_c = psi_at(0, 0);
+                V1 sx = {0.0f}, sy = {0.0f}, sz = {0.0f};
 #pragma unroll
                 for (int a = 1; a < Q; ++a) {
                     if (L::opp(a) < a) continue;
                     const int ex = L::ex(a), ey = L::ey(a), ez = L::ez(a);
                     const int off = ex + ey * TPX;
-                    const V2 wd = float(L::wf(a)) * (psi_at(ez, off) - psi_at(-ez, -off));
+                    const V1 wd = float(L::wf(a)) * (psi_at(ez, off) - psi_at(-ez, -off));
                     if (ex) sx = ex > 0 ? sx + wd : sx - wd;
                     if (ey) sy = ey > 0 ? sy + wd : sy - wd;
                     if (ez) sz = ez > 0 ? sz + wd : sz - wd;
                 }
                 // Eq. 5
-                const V2 gpsi = (-ph.G) * psi_c;
-                const V2 Fmx = gpsi * sx, Fmy = gpsi * sy, Fmz = gpsi * sz;
-                V2 Fx = Fmx + bc(ph.fx), Fy = Fmy + bc(ph.fy), Fz = Fmz + bc(ph.fz);
-                V2 drho = f[0];
+                const V1 gpsi = (-ph.G) * psi_c;
+                const V1 Fmx = gpsi * sx, Fmy = gpsi * sy, Fmz = gpsi * sz;
+                V1 Fx = Fmx + V1{ph.fx}, Fy = Fmy + V1{ph.fy}, Fz = Fmz + V1{ph.fz};
+                V1 drho = f[0];
 #pragma unroll
                 for (int a = 1; a < Q; ++a) drho = drho + f[a];
-                const V2 jx = ((f[1] - f[2]) + (f[7] - f[8])) + ((f[9] - f[10]) + (f[11] - f[12])) + (f[13] - f[14]);
-                const V2 jy = ((f[3] - f[4]) + (f[7] - f[8])) + ((f[10] - f[9]) + (f[15] - f[16])) + (f[17] - f[18]);
-                const V2 jz = ((f[5] - f[6]) + (f[11] - f[12])) + ((f[14] - f[13]) + (f[15] - f[16])) + (f[18] - f[17]);
-                const V2 rho = bc(ph.rho_ref) + drho;
+                const V1 jx = ((f[1] - f[2]) + (f[7] - f[8])) + ((f[9] - f[10]) + (f[11] - f[12])) + (f[13] - f[14]);
+                const V1 jy = ((f[3] - f[4]) + (f[7] - f[8])) + ((f[10] - f[9]) + (f[15] - f[16])) + (f[17] - f[18]);
+                const V1 jz = ((f[5] - f[6]) + (f[11] - f[12])) + ((f[14] - f[13]) + (f[15] - f[16])) + (f[18] - f[17]);
+                const V1 rho = V1{ph.rho_ref} + drho;
                 // Eq. 8 (solid-fluid interaction scheme): F_ads = -G_w rho sum_a w_a s(x + e_a) e_a
                 if constexpr (SF) {
-                    float ax0 = 0.0f, ay0 = 0.0f, az0 = 0.0f, ax1 = 0.0f, ay1 = 0.0f, az1 = 0.0f;
+                    float ax = 0.0f, ay = 0.0f, az = 0.0f;
 #pragma unroll
                     for (int a = 1; a < Q; ++a) {
-                        const int ex = L::ex(a), ey = L::ey(a), ez = L::ez(a), off = ex + ey * TYX;
+                        const int ex = L::ex(a), ey = L::ey(a), ez = L::ez(a);
                         const float w = float(L::wf(a));
-                        const uint8_t* tz = S.type[(zc + ez) & 7];
-                        if (tz[tcl + off] & T_SOLID) {
-                            if (ex) ax0 += w * float(ex);
-                            if (ey) ay0 += w * float(ey);
-                            if (ez) az0 += w * float(ez);
-                        }
-                        if (tz[tcl + 4 * TYX + off] & T_SOLID) {
-                            if (ex) ax1 += w * float(ex);
-                            if (ey) ay1 += w * float(ey);
-                            if (ez) az1 += w * float(ez);
+                        if (S.type[(zc + ez) & 7][tcl + ex + ey * TYX] & T_SOLID) {
+                            if (ex) ax += w * float(ex);
+                            if (ey) ay += w * float(ey);
+                            if (ez) az += w * float(ez);
                         }
                     }
-                    const V2 gr = (-ph.wall_param) * rho;
-                    Fx = (Fmx + gr * mk(ax0, ax1)) + bc(ph.fx);
-                    Fy = (Fmy + gr * mk(ay0, ay1)) + bc(ph.fy);
-                    Fz = (Fmz + gr * mk(az0, az1)) + bc(ph.fz);
+                    const V1 gr = (-ph.wall_param) * rho;
+                    Fx = (Fmx + gr * V1{ax}) + V1{ph.fx};
+                    Fy = (Fmy + gr * V1{ay}) + V1{ph.fy};
+                    Fz = (Fmz + gr * V1{az}) + V1{ph.fz};
                 }
-                if ((fl0 && !(rho.v.x > 0.0f)) || (fl1 && !(rho.v.y > 0.0f))) atomicOr(err, ERR_RHO);
+                if (!(rho.v > 0.0f)) atomicOr(err, ERR_RHO);
                 // Eq. 4: rho u = sum e f + F/2
-                const V2 inv = div2(bc(1.0f), rho);
-                const V2 ux = fma2(0.5f, Fx, jx) * inv, uy = fma2(0.5f, Fy, jy) * inv, uz = fma2(0.5f, Fz, jz) * inv;
-                const V2 X = div2(fma2(Fmx, Fmx, fma2(Fmy, Fmy, Fmz * Fmz)), psi_c * psi_c);
-                collide3p(f, drho, rho, ux, uy, uz, Fx, Fy, Fz, X, kr);
-                const int gi = zc * nxy + (y0 + ly) * nx + x0 + lx;
+                const V1 inv = div2(V1{1.0f}, rho);
+                const V1 ux = fma2(0.5f, Fx, jx) * inv, uy = fma2(0.5f, Fy, jy) * inv, uz = fma2(0.5f, Fz, jz) * inv;
+                if constexpr (MODE == 1) {
+                    if (in) out.node(zc * nxy + (y0 + ly) * nx + x0 + lx, rho.v, ux.v, uy.v, uz.v);
+                } else {
+                    const V1 X = div2(fma2(Fmx, Fmx, fma2(Fmy, Fmy, Fmz * Fmz)), psi_c * psi_c);
+                    collide3p(f, drho, rho, ux, uy, uz, Fx, Fy, Fz, X, kr);
+                    const long long gi = (long long)zc * fxy + (y0 + ly) * fp + x0 + lx;
+                    if (in) {
 #pragma unroll
-                for (int a = 0; a < Q; ++a) {
-                    if (fl0) fout[a * fs + gi] = f[a].v.x;
-                    if (fl1) fout[a * fs + gi + 4 * nx] = f[a].v.y;
+                        for (int a = 0; a < Q; ++a) fout[a * fs + gi] = f[a].v;
+                    }
                 }
             }
         }
@@ -1080,55 +1105,38 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
     }
 }
 
-// Can the march box column (x0, y0) with TMA loads?  (Full 32 x 8 columns of grids at least 64 x 16 x 4;
-// the host's work list uses the same test.)
+// Full columns of grids of at least 64 x 16 x 4: what lbm_d3q19_work_list calls boxed.
 __host__ __device__ __forceinline__ bool ztma_boxed(int x0, int y0, int nx, int ny, int nz) {
     return x0 + TTX <= nx && y0 + TTY <= ny && nx >= 64 && ny >= 16 && nz >= 4;
 }
 
-__global__ void __launch_bounds__(TTX* ZTY, 2)
+// One CTA per item.  The last column of a grid whose width is not a multiple of 32 (8 in y) is moved inside
+// the grid, as far as the boxes' 16-byte boundary allows: up to 3 of its columns then lie beyond x = nx - 1
+// and hold periodic images, patched like the halo.  It writes only the nodes that no full column owns.  (Such
+// columns went to the z-pair march on narrow blocks before: the 200 x 200 x 280 grid, one column in seven,
+// took 561 us a step, 455 us now.)
+template <int MODE>
+__global__ void __launch_bounds__(TNT, 2)
     ztma_step(const float* __restrict__ fin, float* __restrict__ fout, const void* tmap, Geo g, Phys<float> ph,
-              Rates3P kr, unsigned* err, const ZItem* __restrict__ items) {
+              Rates3P kr, unsigned* err, const ZItem* __restrict__ items, ZTOut out) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const ZItem it = items[blockIdx.x];
-    const int x0 = it.bx * TTX, y0 = it.by * TTY, zb = it.z0, ze = it.z1;
-    const bool boxed = tmap != nullptr && ztma_boxed(x0, y0, g.nx, g.ny, g.nz);
-    const bool sf = ph.wall_kind == 2;
-    if (boxed) {
-        ZTSmem& S = *reinterpret_cast<ZTSmem*>(smem_raw);
-        if (threadIdx.x == 0 && threadIdx.y == 0) {
-            mbar_init(&S.bar[0]);
-            mbar_init(&S.bar[1]);
-            fence_mbar_init();
-        }
-        __syncthreads();
-        // tmap: the input buffer's map (box TBX x TBY x 1)
-        if (!it.solid)
-            ztma_chunk_bulk(fin, fout, tmap, g, ph, kr, x0, y0, zb, ze, err, S.b, S.bar);
-        else if (sf)
-            ztma_chunk_solid<true>(fin, fout, tmap, g, ph, kr, x0, y0, zb, ze, err, S.s, S.bar);
-        else
-            ztma_chunk_solid<false>(fin, fout, tmap, g, ph, kr, x0, y0, zb, ze, err, S.s, S.bar);
-        return;
+    const int xs = it.bx * TTX, ys = it.by * TTY, zb = it.z0, ze = it.z1;   // first nodes of its own
+    const int x0 = xs + TTX <= g.nx ? xs : (g.nx - TTX + 3) / 4 * 4, y0 = min(ys, g.ny - TTY);
+    ZTSmem& S = *reinterpret_cast<ZTSmem*>(smem_raw);
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        mbar_init(&S.bar[0]);
+        mbar_init(&S.bar[1]);
+        fence_mbar_init();
     }
-    // a column the march cannot box: its 32-plane chunk by the z-pair march on the two 32 x 4 halves,
-    // with their chunk flags
-    const int ty4 = (g.ny + ZTY - 1) / ZTY, tx = (g.nx + ZTX - 1) / ZTX;
-    const int h0 = ((zb / ZCH) * ty4 + 2 * it.by) * tx + it.bx;
-    const bool has1 = y0 + ZTY < g.ny;
-    const bool s0 = g.tile_solid ? g.tile_solid[h0] != 0 : true;
-    const bool s1 = has1 && (g.tile_solid ? g.tile_solid[h0 + tx] != 0 : true);
-    ZPSmem<ZTX, ZTY>& sm = *reinterpret_cast<ZPSmem<ZTX, ZTY>*>(smem_raw);
-    for (int h = 0; h < (has1 ? 2 : 1); ++h) {
-        const bool solid = h ? s1 : s0;
-        if (h) __syncthreads();   // the first half is done with shared memory
-        if (solid && sf)
-            zpair_chunk<true, true>(fin, fout, g, ph, kr, x0, y0 + h * ZTY, zb, err, sm);
-        else if (solid)
-            zpair_chunk<true>(fin, fout, g, ph, kr, x0, y0 + h * ZTY, zb, err, sm);
-        else
-            zpair_chunk<false>(fin, fout, g, ph, kr, x0, y0 + h * ZTY, zb, err, sm);
-    }
+    __syncthreads();
+    // tmap: the input buffer's map (box TBX x TBY x 1)
+    if (!it.solid)
+        ztma_chunk_bulk<MODE>(fin, fout, tmap, g, ph, kr, x0, y0, xs, ys, zb, ze, err, S.b, S.bar, out);
+    else if (ph.wall_kind == 2)
+        ztma_chunk_solid<true, MODE>(fin, fout, tmap, g, ph, kr, x0, y0, xs, ys, zb, ze, err, S.s, S.bar, out);
+    else
+        ztma_chunk_solid<false, MODE>(fin, fout, tmap, g, ph, kr, x0, y0, xs, ys, zb, ze, err, S.s, S.bar, out);
 }
 
 }  // namespace
@@ -1156,22 +1164,33 @@ cudaError_t launch_zpair_step(const void* fin, void* fout, const Geo& g, const D
     return cudaGetLastError();
 }
 
-cudaError_t launch_ztma_step(const void* fin, void* fout, const void* tmap, const Geo& g, const DevParams& p,
-                             cudaStream_t s) {
+template <int MODE>
+static cudaError_t launch_ztma(const void* fin, void* fout, const void* tmap, const Geo& g, const DevParams& p,
+                               const ZTOut& out, cudaStream_t s) {
     static bool attr[64] = {false};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!attr[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(ztma_step, cudaFuncAttributeMaxDynamicSharedMemorySize, int(ZT_SMEM));
+        cudaError_t e = cudaFuncSetAttribute(ztma_step<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(ZT_SMEM));
         if (e != cudaSuccess) return e;
         attr[dev] = true;
     }
     if (!p.zitems || p.nzitems < 1) return cudaErrorInvalidValue;
-    ztma_step<<<p.nzitems, dim3(TTX, ZTY, 1), ZT_SMEM, s>>>(static_cast<const float*>(fin), static_cast<float*>(fout),
-                                                           tmap, g, make_phys<float>(p), make_rates3p(p), p.err,
-                                                           p.zitems);
+    ztma_step<MODE><<<p.nzitems, dim3(TTX, TTY, 1), ZT_SMEM, s>>>(static_cast<const float*>(fin), static_cast<float*>(fout),
+                                                                 tmap, g, make_phys<float>(p), make_rates3p(p), p.err,
+                                                                 p.zitems, out);
     return cudaGetLastError();
+}
+
+cudaError_t launch_ztma_step(const void* fin, void* fout, const void* tmap, const Geo& g, const DevParams& p,
+                             cudaStream_t s) {
+    return launch_ztma<0>(fin, fout, tmap, g, p, ZTOut{nullptr, nullptr, 0}, s);
+}
+
+cudaError_t launch_ztma_fields(const void* fin, const void* tmap, const Geo& g, const DevParams& p, double* rho,
+                               double* u, cudaStream_t s) {
+    return launch_ztma<1>(fin, nullptr, tmap, g, p, ZTOut{rho, u, g.N}, s);
 }
 
 void ztma_box_dims(int* bx, int* by) {
@@ -1183,26 +1202,35 @@ void ztma_box_dims(int* bx, int* by) {
 #define LBMWET_ZWL_MIN_RUN 8
 #endif
 
-std::vector<ZItem> ztma_work_list(const uint8_t* mask, int nx, int ny, int nz) {
-    constexpr int HALO = 3, MIN_RUN = LBMWET_ZWL_MIN_RUN;
+namespace {
+
+// The z-range of every column for which boxed(x0, y0) holds as runs of planes that need the solid path and
+// runs that do not (ordered by column); the other columns as 32-plane chunks flagged solid, in `chunks`.
+template <class Boxed>
+std::vector<ZItem> column_runs(const uint8_t* mask, int nx, int ny, int nz, int min_run, Boxed boxed,
+                               std::vector<ZItem>* chunks) {
+    constexpr int HALO = 3;
     const int gx = (nx + TTX - 1) / TTX, gy = (ny + TTY - 1) / TTY;
     // per plane and column: a solid within 3 nodes of the column's cells in x and y (periodic)
     const int t[3] = {TTX, TTY, 1};
     const std::vector<uint8_t> col = tile_solid_flags(mask, nx, ny, nz, t, 2, scan_threads((long long)nx * ny * nz));
-    std::vector<ZItem> items;
+    std::vector<ZItem> all;
     std::vector<uint8_t> need(nz);
     for (int by = 0; by < gy; ++by)
         for (int bx = 0; bx < gx; ++bx) {
-            if (!ztma_boxed(bx * TTX, by * TTY, nx, ny, nz)) {
-                for (int z0 = 0; z0 < nz; z0 += ZCH) items.push_back(ZItem{bx, by, z0, std::min(z0 + ZCH, nz), 1});
+            if (!boxed(bx * TTX, by * TTY)) {
+                for (int z0 = 0; z0 < nz; z0 += ZCH) chunks->push_back(ZItem{bx, by, z0, std::min(z0 + ZCH, nz), 1});
                 continue;
             }
-            // planes within 3 planes (periodic) of a plane with a solid near the column
+            // planes within 3 planes (periodic) of a plane with a solid near the column's cells; a column moved
+            // inside the grid also covers cells of its left and lower neighbours
+            const int bx0 = bx * TTX + TTX > nx && bx > 0 ? bx - 1 : bx, by0 = by * TTY + TTY > ny && by > 0 ? by - 1 : by;
             for (int z = 0; z < nz; ++z) {
                 uint8_t n = 0;
                 for (int d = -HALO; d <= HALO && !n; ++d) {
                     const int zz = ((z + d) % nz + nz) % nz;
-                    n = col[((size_t)zz * gy + by) * gx + bx];
+                    for (int cy = by0; cy <= by; ++cy)
+                        for (int cx = bx0; cx <= bx; ++cx) n |= col[((size_t)zz * gy + cy) * gx + cx];
                 }
                 need[z] = n;
             }
@@ -1215,28 +1243,86 @@ std::vector<ZItem> ztma_work_list(const uint8_t* mask, int nx, int ny, int nz) {
                 z0 = z1;
             }
             for (ZItem& r : runs)
-                if (!r.solid && r.z1 - r.z0 < MIN_RUN && runs.size() > 1) r.solid = 1;
-            std::vector<ZItem> merged;
+                if (!r.solid && r.z1 - r.z0 < min_run && runs.size() > 1) r.solid = 1;
+            const size_t first = all.size();
             for (const ZItem& r : runs) {
-                if (!merged.empty() && merged.back().solid == r.solid) merged.back().z1 = r.z1;
-                else merged.push_back(r);
-            }
-            // pieces cut at the multiples of TCH planes, so that items of neighbouring columns start
-            // on the same planes and share their halo reads in L2; a first or last piece shorter than
-            // MIN_RUN joins its neighbour (items of up to TCH + MIN_RUN - 1 planes)
-            for (const ZItem& r : merged) {
-                std::vector<int> cuts{r.z0};
-                for (int z = (r.z0 / TCH + 1) * TCH; z < r.z1; z += TCH) cuts.push_back(z);
-                cuts.push_back(r.z1);
-                if (cuts.size() > 2 && cuts[1] - cuts[0] < MIN_RUN) cuts.erase(cuts.begin() + 1);
-                if (cuts.size() > 2 && cuts[cuts.size() - 1] - cuts[cuts.size() - 2] < MIN_RUN)
-                    cuts.erase(cuts.end() - 2);
-                for (size_t k = 0; k + 1 < cuts.size(); ++k)
-                    items.push_back(ZItem{bx, by, cuts[k], cuts[k + 1], r.solid});
+                if (all.size() > first && all.back().solid == r.solid) all.back().z1 = r.z1;
+                else all.push_back(r);
             }
         }
+    return all;
+}
+
+// Runs cut at the multiples of 32 planes, so that items of neighbouring columns start on the same planes and
+// share their halo reads in L2; a first or last piece shorter than LBMWET_ZWL_MIN_RUN joins its neighbour
+// (items of up to 39 planes).
+std::vector<ZItem> aligned_items(const std::vector<ZItem>& runs, std::vector<ZItem> items) {
+    constexpr int MIN_RUN = LBMWET_ZWL_MIN_RUN;
+    for (const ZItem& r : runs) {
+        std::vector<int> cuts{r.z0};
+        for (int z = (r.z0 / TCH + 1) * TCH; z < r.z1; z += TCH) cuts.push_back(z);
+        cuts.push_back(r.z1);
+        if (cuts.size() > 2 && cuts[1] - cuts[0] < MIN_RUN) cuts.erase(cuts.begin() + 1);
+        if (cuts.size() > 2 && cuts[cuts.size() - 1] - cuts[cuts.size() - 2] < MIN_RUN) cuts.erase(cuts.end() - 2);
+        for (size_t k = 0; k + 1 < cuts.size(); ++k) items.push_back(ZItem{r.bx, r.by, cuts[k], cuts[k + 1], r.solid});
+    }
     std::stable_sort(items.begin(), items.end(), [](const ZItem& a, const ZItem& b) {
         return a.z0 != b.z0 ? a.z0 < b.z0 : (a.by != b.by ? a.by < b.by : a.bx < b.bx);
+    });
+    return items;
+}
+
+}  // namespace
+
+std::vector<ZItem> ztma_work_list(const uint8_t* mask, int nx, int ny, int nz) {
+    std::vector<ZItem> chunks;
+    const std::vector<ZItem> runs = column_runs(
+        mask, nx, ny, nz, LBMWET_ZWL_MIN_RUN, [&](int x0, int y0) { return ztma_boxed(x0, y0, nx, ny, nz); }, &chunks);
+    return aligned_items(runs, chunks);
+}
+
+// The window of a box (36 columns and 14 rows with the rows beyond it) leaves the grid on one side at most,
+// also where the last column is moved inside.
+bool ztma_marches(int nx, int ny, int nz) { return nx >= 40 && ny >= 16 && nz >= 4; }
+
+std::vector<ZItem> ztma_items(const uint8_t* mask, int nx, int ny, int nz, int slots) {
+    const long long columns = (long long)((nx + TTX - 1) / TTX) * ((ny + TTY - 1) / TTY);
+    const bool large = columns * ((nz + TCH - 1) / TCH) >= 2LL * slots;
+    std::vector<ZItem> none;
+    const std::vector<ZItem> runs =
+        column_runs(mask, nx, ny, nz, large ? LBMWET_ZWL_MIN_RUN : 4, [](int, int) { return true; }, &none);
+    if (large) return aligned_items(runs, none);
+    // A grid of less than two waves: shorter pieces, of lengths chosen for the least time.  A piece of c planes
+    // takes c + 3 plane times on the bulk path (two halo planes, start-up) and c + 5 on the solid path, whose
+    // plane takes three times as long (256^3: 2.3 and 6.7 us); a launch takes as long as its longest piece and
+    // at least its total over the slots.  The solid pieces start first.
+    auto pieces = [](int len, int c) { return (len + c - 1) / c; };
+    double best = 1e300;
+    int cb = TCH, cs = TCH;
+    for (int b : {32, 26, 22, 18, 16, 14, 12, 11, 10, 9, 8, 7, 6, 5, 4, 3, 2})
+        for (int q : {32, 16, 12, 8, 6, 5, 4, 3, 2, 1}) {
+            double total = 0.0, longest = 0.0;
+            for (const ZItem& r : runs) {
+                const int len = r.z1 - r.z0, n = pieces(len, r.solid ? q : b), c = (len + n - 1) / n;
+                const double t = r.solid ? 3.0 * (c + 5) : c + 3.0;
+                total += n * t;
+                longest = std::max(longest, t);
+            }
+            const double cost = std::max(longest, total / slots + 0.3 * longest);
+            if (cost < best) {
+                best = cost;
+                cb = b;
+                cs = q;
+            }
+        }
+    std::vector<ZItem> items;
+    for (const ZItem& r : runs) {
+        const int len = r.z1 - r.z0, n = pieces(len, r.solid ? cs : cb);
+        for (int k = 0; k < n; ++k) items.push_back(ZItem{r.bx, r.by, r.z0 + k * len / n, r.z0 + (k + 1) * len / n, r.solid});
+    }
+    std::stable_sort(items.begin(), items.end(), [](const ZItem& a, const ZItem& b) {
+        return a.solid != b.solid ? a.solid > b.solid
+                                  : (a.z0 != b.z0 ? a.z0 < b.z0 : (a.by != b.by ? a.by < b.by : a.bx < b.bx));
     });
     return items;
 }
