@@ -753,13 +753,18 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
     p.zf0 = h->f[0];
     if (h->D == 3 && c.precision == LBM_FP32_DEV && p.step3 == 0 && ztma_marches(nx, ny, nz)) {
         int bx, by;
-        ztma_box_dims(&bx, &by);
-        CUtensorMap maps[2];
-        if (encode_z_map(&maps[0], h->f[0], nx, ny, nz, fpitch, bx, by) &&
-            encode_z_map(&maps[1], h->f[1], nx, ny, nz, fpitch, bx, by)) {
-            CKI(dmalloc(&h->d_zmaps, sizeof(maps), h->stream), "cudaMalloc tensor maps");
+        const int nmaps = ztma_maps(0, &bx, &by);
+        std::vector<CUtensorMap> maps(2 * nmaps);
+        bool ok = true;
+        for (int k = 0; k < 2 * nmaps; ++k) {
+            ztma_maps(k % nmaps, &bx, &by);
+            ok = ok && encode_z_map(&maps[k], h->f[k / nmaps], nx, ny, nz, fpitch, bx, by);
+        }
+        if (ok) {
+            CKI(dmalloc(&h->d_zmaps, sizeof(CUtensorMap) * maps.size(), h->stream), "cudaMalloc tensor maps");
             // (from pageable memory: staged before the call returns, so `maps` may go out of scope)
-            CKI(cudaMemcpyAsync(h->d_zmaps, maps, sizeof(maps), cudaMemcpyHostToDevice, h->stream), "copy tensor maps");
+            CKI(cudaMemcpyAsync(h->d_zmaps, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice,
+                                h->stream), "copy tensor maps");
             const std::vector<ZItem> items = ztma_items(solid_mask, nx, ny, nz, 2 * device_sms());   // (2 CTAs per SM)
             CKI(dmalloc(&h->d_zitems, sizeof(ZItem) * items.size(), h->stream), "cudaMalloc work list");
             CKI(cudaMemcpyAsync(h->d_zitems, items.data(), sizeof(ZItem) * items.size(), cudaMemcpyHostToDevice,

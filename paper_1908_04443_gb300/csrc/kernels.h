@@ -38,7 +38,7 @@ struct DevParams {
     int tile_w, tile_h, tile_z;
     // D3Q19 FP32 step kernel: 0 the TMA-staged z-march, 1 the z-pair march, 2 the scalar z-march
     int step3;
-    const void* ztmap;           // TMA tensor maps of the two 3D FP32 distribution buffers (device, 2 x 128 B)
+    const void* ztmap;           // TMA tensor maps of the two 3D FP32 distribution buffers (device, ztma_maps x 128 B each)
     const void* zf0;             // the buffer the first map describes
     const struct ZItem* zitems;  // its work list: one item per CTA (see ZItem)
     int nzitems;
@@ -178,7 +178,8 @@ cudaError_t launch_zpair_step(const void* fin, void* fout, const Geo& g, const D
 // bx x by x 1, see ztma_box_dims), 128 bytes.
 cudaError_t launch_ztma_step(const void* fin, void* fout, const void* tmap, const Geo& g, const DevParams& p,
                              cudaStream_t s);
-void ztma_box_dims(int* bx, int* by);
+// Box (columns, rows) of tensor map k of a buffer; returns the number of maps, which lie behind one another.
+int ztma_maps(int k, int* bx, int* by);
 // Work list of the TMA-staged z-march for a grid with solid mask `mask` (host, nx*ny*nz bytes):
 // every boxed 32 x 8 column cut along z into runs that need the solid path and runs that do not
 // (bulk runs shorter than 8 planes join the solid path), each run cut at the multiples of 32 planes

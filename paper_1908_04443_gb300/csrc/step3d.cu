@@ -323,7 +323,8 @@ void zmarch_tile_shape(int prec, int* tx, int* ty, int* tz) {
 cudaError_t launch_step3d(int prec, int mode, const void* fin, void* fout, const Geo& g, const DevParams& p,
                           double* rho, double* u, cudaStream_t s) {
     if (prec == PREC_FP32 && p.ztmap) {
-        const void* map = static_cast<const char*>(p.ztmap) + (fin == p.zf0 ? 0 : 128);
+        int bx, by;
+        const void* map = static_cast<const char*>(p.ztmap) + (fin == p.zf0 ? 0 : 128 * ztma_maps(0, &bx, &by));
         return mode == 0 ? launch_ztma_step(fin, fout, map, g, p, s) : launch_ztma_fields(fin, map, g, p, rho, u, s);
     }
     if (prec == PREC_FP32 && mode == 0 && p.step3 != 2) return launch_zpair_step(fin, fout, g, p, s);

@@ -15,7 +15,8 @@
 // with LBMWET_ZP_REPULL = 0, the own distributions, 4 planes).  Results equal the scalar z-march's up to FP32 rounding (operations regrouped).
 #include <algorithm>
 #include <cmath>
-#include <type_traits>
+#include <map>
+#include <utility>
 
 #include "kernels.h"
 #include "lattice.cuh"
@@ -481,12 +482,10 @@ __global__ void __launch_bounds__(ZTX* ZTY, LBMWET_ZP_MINB)
 // 32 x 8 column, one cell per thread, over the planes of a work item, and marches plane by plane through
 // shared memory.  (128 threads with two cells each in packed FP32x2 arithmetic take the same time on 256^3,
 // 532 against 536 us, and longer where items are few: 64^3 42.7 against 39.8, 128^3 124 against 108.)
-//   * every lead plane zl is staged by TMA: for each direction a, the box of f*_a on plane zl - ez(a)
-//     over x0 - 4 .. x0 + 35 (x starts on a 16-byte boundary) and y0 - 2 .. y0 + 9 (y0 - 3 .. y0 + 10
-//     in chunks holding solids, whose walls need densities two nodes out), so that the pull (Eq. 3)
-//     of any cell of the column and of its halo reads its 19 values at constant offsets from one
-//     shared-memory address; two stages on two mbarriers keep the next plane's 19 boxes in flight
-//     while the current one is used;
+//   * every lead plane zl is staged by TMA: for each direction a, the box of f*_a on plane zl - ez(a) that the
+//     cells of the column and its halo pull from (the window shifted by -e_a, x from a 16-byte boundary),
+//     so that the pull (Eq. 3) of any cell reads its 19 values at constant offsets; two stages on two
+//     mbarriers keep the next plane's 19 boxes in flight while the current one is used;
 //   * where the box crosses a periodic edge of the grid (TMA cannot wrap), the out-of-range columns
 //     and rows it needs are loaded by the threads and written over the box's zero fill after its
 //     wait (one plane ahead, from registers, in chunks without solids);
@@ -505,36 +504,43 @@ __global__ void __launch_bounds__(ZTX* ZTY, LBMWET_ZP_MINB)
 constexpr int TTX = 32, TTY = 8, TCH = ZCH;
 static_assert(TTX == ZTX && TTY == 2 * ZTY, "a TMA column is two z-pair columns");
 constexpr int TNT = TTX * TTY;                // threads: one per cell
-constexpr int TBX = TTX + 8;                  // box columns: x0 - 4 .. x0 + 35
-constexpr int TBY = TTY + 4;                  // box rows: y0 - 2 .. y0 + 9
-constexpr int TBSLOT = TBY * TBX;             // floats per direction and stage, chunks without solids (480)
-static_assert((TBSLOT * 4) % 128 == 0, "every direction's box starts on a 128-byte boundary");
-constexpr int TPX = TTX + 2, TPY = TTY + 2;   // psi window: the column + 1-node ring (box cols 3..36)
+constexpr int TPX = TTX + 2, TPY = TTY + 2;   // psi window: the column + 1-node ring
 constexpr int TRX = TTX + 4, TRY = TTY + 4;   // density window (solid chunks): + 2-node ring
 constexpr int TYX = TTX + 6, TYY = TTY + 6;   // node-type window (solid chunks): + 3-node ring
 constexpr int TRING = 2 * TPX + 2 * (TPY - 2);                 // 84 cells of the 1-node ring
 constexpr int TRING2 = 2 * TRX + 2 * (TRY - 2);                // 92 cells of the 2-node ring
 constexpr int TTYPES = TYX * TYY;                              // 532 type cells per plane
-constexpr unsigned TBYTES_BULK = 19u * TBY * TBX * 4u;
-// the directions with ey = +1 (3, 7, 10, 15, 17) and ey = -1 (4, 8, 9, 16, 18), five bits each
-constexpr unsigned XROW_UP = 3u | 7u << 5 | 10u << 10 | 15u << 15 | 17u << 20;
-constexpr unsigned XROW_DN = 4u | 8u << 5 | 9u << 10 | 16u << 15 | 18u << 20;
-__host__ __device__ constexpr int xrow_slot(int a) {   // position of a among its five directions
-    return a == 3 || a == 4 ? 0 : a == 7 || a == 8 ? 1 : a == 10 || a == 9 ? 2 : a == 15 || a == 16 ? 3 : 4;
+// The box of direction a covers what the window's cells pull along a: the window shifted by -e_a, widened to
+// columns that start on a 16-byte boundary.  In bulk chunks (window: psi) 10 rows from y0 - 1 - ey and 40 columns
+// from x0 - 4, or 36 where ex != 0: from x0 - 4 (ex = 1), from x0 (ex = -1).  In solid chunks (window: density) 12
+// rows from y0 - 2 - ey and 40 columns from x0 - 4.
+constexpr int BROWS = TPY, SROWS = TRY, TBX = TTX + 8;
+__host__ __device__ constexpr int box_cols(int ex) { return ex == 0 ? TTX + 8 : TTX + 4; }
+__host__ __device__ constexpr int box_lead(int ex) { return ex < 0 ? 0 : 4; }   // columns before x0
+// floats of a stage before direction a's box, each box on a 128-byte boundary (bulk: 416 for ex = 0, else 384)
+__host__ __device__ constexpr int bslot(int a) {
+    return 416 * (a > 0) + 384 * (a > 1) + 384 * (a > 2) + 416 * (a < 3 ? 0 : (a < 7 ? a - 3 : 4)) +
+           384 * (a < 7 ? 0 : (a < 15 ? a - 7 : 8)) + 416 * (a < 15 ? 0 : a - 15);
 }
+constexpr int BSTAGE = bslot(19), BST = 2;   // floats of a bulk stage, and its stages
+constexpr int SSLOT = 480;
+static_assert(416 >= BROWS * box_cols(0) && 384 >= BROWS * box_cols(1) && SSLOT >= SROWS * TBX, "boxes fit their slots");
+static_assert(BSTAGE == 9 * 416 + 10 * 384 && BSTAGE % 32 == 0 && SSLOT % 32 == 0, "128-byte boundaries");
+constexpr unsigned BULK_BYTES = 4u * BROWS * (9u * box_cols(0) + 10u * box_cols(1));   // 9 directions with ex = 0
+constexpr unsigned SOLID_BYTES = 4u * 19u * SROWS * TBX;
+// tensor maps of a buffer, 128 bytes each: 40 x 10, 36 x 10 and 40 x 12 boxes
+constexpr int ZMAPS = 3;
 
-// Shared memory of the two kinds of chunk, overlaid: both keep two planes of boxes in flight (the
-// same 12-row boxes); chunks holding solids add node types, a density ring and the two rows beyond
-// the box that their 2-node density ring pulls from.  The CTA stays under 97 KB, so that two CTAs
-// per SM leave the L1 at least 60 KB, which the loads of the periodic-edge patches need (with 107 KB
-// CTAs the 256^3 step ran at 0.65 of the HBM roofline instead of 0.78).
+// Shared memory of the two kinds of chunk, overlaid: both keep two planes of boxes in flight (three take
+// 5 % longer: the L1 shrinks); chunks holding solids add node types and a density ring.  The CTA stays under 97 KB, so that two CTAs per SM leave the L1
+// at least 60 KB, which the loads of the periodic-edge patches need (with 107 KB CTAs the 256^3 step ran at
+// 0.65 of the HBM roofline instead of 0.78).
 struct ZTBulk {
-    float stage[2][19][TBSLOT];
+    float stage[BST][BSTAGE];
     float psi[4][TPY * TPX];
 };
 struct ZTSolid {
-    float stage[2][19][TBSLOT];
-    float xrow[2][2][5][TBX];   // by plane parity: row y0 - 3 (directions with ey = 1), row y0 + 10 (ey = -1)
+    float stage[2][19 * SSLOT];
     float psi[5][TPY * TPX];
     float rho[4][TRY * TRX];
     uint8_t type[8][TTYPES];
@@ -544,7 +550,7 @@ struct ZTSmem {
         ZTBulk b;
         ZTSolid s;
     };
-    uint64_t bar[2];
+    uint64_t bar[BST];
 };
 constexpr size_t ZT_SMEM = sizeof(ZTSmem);
 
@@ -563,7 +569,17 @@ __device__ __forceinline__ void tma_box3(void* dst, const void* tmap, int cx, in
         : "memory");
 }
 
-// z component of D3Q19 velocity a for a run-time index (bit tables instead of an indexed array)
+// components of D3Q19 velocity a for a run-time index (bit tables instead of indexed arrays)
+__device__ __forceinline__ int ex_rt(int a) {
+    constexpr unsigned PLUS = (1u << 1) | (1u << 7) | (1u << 9) | (1u << 11) | (1u << 13);
+    constexpr unsigned MINUS = (1u << 2) | (1u << 8) | (1u << 10) | (1u << 12) | (1u << 14);
+    return int((PLUS >> a) & 1u) - int((MINUS >> a) & 1u);
+}
+__device__ __forceinline__ int ey_rt(int a) {
+    constexpr unsigned PLUS = (1u << 3) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 17);
+    constexpr unsigned MINUS = (1u << 4) | (1u << 8) | (1u << 9) | (1u << 16) | (1u << 18);
+    return int((PLUS >> a) & 1u) - int((MINUS >> a) & 1u);
+}
 __device__ __forceinline__ int ez_rt(int a) {
     constexpr unsigned PLUS = (1u << 5) | (1u << 11) | (1u << 14) | (1u << 15) | (1u << 18);
     constexpr unsigned MINUS = (1u << 6) | (1u << 12) | (1u << 13) | (1u << 16) | (1u << 17);
@@ -640,9 +656,9 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
     const int zlo = zb - 1, zhi = ze;   // lead planes zlo .. zhi, collided planes zb .. ze - 1
     const int nlead = zhi - zlo + 1;
 
-    // out-of-range cells of the used window (rows 0 .. 11, columns 2 .. 37): at most 2 rows and 5 columns,
-    // 2 * 36 + 5 * 10 = 122 < 128, one per thread, prefetched one plane ahead
-    const OutBand ob_(x0 - 4, y0 - 2, nx, ny, 0, TBY, 2, TBX - 2);
+    // out-of-range nodes among those pulled from (rows y0 - 2 .. y0 + 9, columns x0 - 2 .. x0 + 33): at most 2 rows
+    // and 5 columns, 2 * 36 + 5 * 10 = 122, one per thread, prefetched one plane ahead
+    const OutBand ob_(x0 - 4, y0 - 2, nx, ny, 0, TRY, 2, TBX - 2);
     const bool edge = ob_.cells > 0;
     int fr = 0, fcl = 0, fsrc = 0;
     const bool fixer = tid < ob_.cells;
@@ -655,48 +671,58 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
     // all held its warp, and the barrier behind it, for 19 instructions)
     auto issue = [&](int zl, int s) {
         fence_proxy_async();
-        if (ly == 0) mbar_expect_tx(&bar[s], TBYTES_BULK);
-        for (int a = ly; a < Q; a += TTY)
-            tma_box3(S.stage[s][a], tmap, x0 - 4, y0 - 2, a * nz + wrap1(zl - ez_rt(a), nz), &bar[s]);
+        if (ly == 0) mbar_expect_tx(&bar[s], BULK_BYTES);
+        for (int a = ly; a < Q; a += TTY) {
+            const int ex = ex_rt(a);
+            tma_box3(S.stage[s] + bslot(a), static_cast<const char*>(tmap) + (ex ? 128 : 0), x0 - box_lead(ex),
+                     y0 - 1 - ey_rt(a), a * nz + wrap1(zl - ez_rt(a), nz), &bar[s]);
+        }
     };
 
     if (lx == 0) {
-        issue(zlo, 0);
-        issue(zlo + 1, 1);
+        for (int k = 0; k < BST && zlo + k <= zhi; ++k) issue(zlo + k, k);
     }
     if (edge && fixer) {
 #pragma unroll
         for (int a = 0; a < Q; ++a) fix[a] = fin[a * fs + (long long)wrap1(zlo - L::ez(a), nz) * fxy + fsrc];
     }
 
-    // own cells in box and psi-window coordinates
-    const int ob = (ly + 2) * TBX + lx + 4;
+    // own cell in the psi window
     const int pc = (ly + 1) * TPX + lx + 1;
     // the nodes this item writes (a column moved inside the grid shares some with its neighbours)
     const bool wr = x0 + lx >= xs && x0 + lx < nx && y0 + ly >= ys;
     // this thread's halo-ring cell (the last 84 threads; the first ones patch the edges)
-    int rb = 0, rp = 0;
+    int rx = 0, ry = 0;
     const bool ringer = TNT - 1 - tid < TRING;
     if (ringer) {
-        int px, py, pz;
-        Shell<TPX, TPY, 1, 2>::cell(TNT - 1 - tid, px, py, pz);
-        rb = (py + 1) * TBX + px + 3;
-        rp = py * TPX + px;
+        int pz;
+        Shell<TPX, TPY, 1, 2>::cell(TNT - 1 - tid, rx, ry, pz);
     }
+    // what cell (px, py) of the psi window pulls along a: row py of the box, px - 1 - ex columns from x0
+    auto pulled = [](const float* st, int a, int px, int py) {
+        return st[bslot(a) + py * box_cols(L::ex(a)) + px - 1 - L::ex(a) + box_lead(L::ex(a))];
+    };
 
     V1 fprev[Q];
 #pragma unroll
     for (int a = 0; a < Q; ++a) fprev[a].v = 0.0f;
 
+    int s = 0;           // stage of the lead plane
+    unsigned phase = 0;  // of its barrier
 #pragma unroll 1
     for (int i = 0; i < nlead; ++i) {
-        const int zl = zlo + i, s = i & 1;
-        if (!mbar_wait(&bar[s], unsigned(i >> 1) & 1u, ZT_POLL_LIMIT)) atomicOr(err, ERR_TIMEOUT);
-        float* st = S.stage[s][0];
+        const int zl = zlo + i;
+        if (!mbar_wait(&bar[s], phase, ZT_POLL_LIMIT)) atomicOr(err, ERR_TIMEOUT);
+        float* st = S.stage[s];
         if (edge) {
             if (fixer) {
+                // node (x0 - 4 + fcl, y0 - 2 + fr) in every direction's box that covers it
 #pragma unroll
-                for (int a = 0; a < Q; ++a) st[a * TBSLOT + fr * TBX + fcl] = fix[a];
+                for (int a = 0; a < Q; ++a) {
+                    const int r = fr - 1 + L::ey(a), c = fcl - 4 + box_lead(L::ex(a));
+                    if (unsigned(r) < unsigned(BROWS) && unsigned(c) < unsigned(box_cols(L::ex(a))))
+                        st[bslot(a) + r * box_cols(L::ex(a)) + c] = fix[a];
+                }
                 fence_proxy_async();
             }
             if (fixer && zl + 1 <= zhi) {
@@ -709,7 +735,7 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
         // A. rho and psi of lead plane zl: the column (own values kept) and its halo ring
         V1 fcur[Q];
 #pragma unroll
-        for (int a = 0; a < Q; ++a) fcur[a].v = st[ob + a * TBSLOT - L::ey(a) * TBX - L::ex(a)];
+        for (int a = 0; a < Q; ++a) fcur[a].v = pulled(st, a, lx + 1, ly + 1);
         {
             V1 d = fcur[0];
 #pragma unroll
@@ -717,13 +743,17 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
             S.psi[zl & 3][pc] = psi1(V1{ph.rho_ref} + d, ph, err).v;
         }
         if (ringer) {
-            V1 d = {st[rb]};
+            V1 d = {pulled(st, 0, rx, ry)};
 #pragma unroll
-            for (int a = 1; a < Q; ++a) d = d + V1{st[rb + a * TBSLOT - L::ey(a) * TBX - L::ex(a)]};
-            S.psi[zl & 3][rp] = psi1(V1{ph.rho_ref} + d, ph, err).v;
+            for (int a = 1; a < Q; ++a) d = d + V1{pulled(st, a, rx, ry)};
+            S.psi[zl & 3][ry * TPX + rx] = psi1(V1{ph.rho_ref} + d, ph, err).v;
         }
         __syncthreads();
-        if (lx == 0 && zl + 2 <= zhi) issue(zl + 2, s);
+        if (lx == 0 && zl + BST <= zhi) issue(zl + BST, s);
+        if (++s == BST) {
+            s = 0;
+            phase ^= 1u;
+        }
 
         // C. collide plane zc = zl - 1
         const int zc = zl - 1;
@@ -778,7 +808,7 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
 
 // A chunk holding solids within 3 nodes: node types of planes zl - 3 .. zl + 2 in a ring, bounce-back
 // links, a 2-node density ring for the wall cells' Eq. 17, lag 2 between lead and collided plane.
-// Coordinates (rb, c) are those of the box: row rb is grid row y0 - 2 + rb, column c is x0 - 4 + c.
+// Coordinates (rb, c) of a cell: row rb is grid row y0 - 2 + rb, column c is x0 - 4 + c.
 template <bool SF, int MODE>
 __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, float* __restrict__ fout,
                                                  const void* tmap, const Geo& g, const Phys<float>& ph,
@@ -798,42 +828,22 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
         const int tr = k / TYX, tc = k % TYX;
         return g.type[(long long)wz(z) * nxy + wrap1(y0 - 3 + tr, ny) * nx + wrap1(x0 - 3 + tc, nx)];
     };
-    // the rows beyond the box that the 2-node ring pulls from (box row -1 for ey = 1, row 12 for
-    // ey = -1), columns 1 .. 38: item k < 380 of plane z
-    auto xrow_src = [&](int z, int k) {
-        const int row = k / 190, rem = k - row * 190, d = rem / 38, col = 1 + rem % 38;
-        const int a = int(((row ? XROW_DN : XROW_UP) >> (5 * d)) & 31u);
-        return fin[a * fs + (long long)wz(z - ez_rt(a)) * fxy + wrap1(row ? y0 + 10 : y0 - 3, ny) * fp +
-                   wrap1(x0 - 4 + col, nx)];
-    };
-    auto xrow_dst = [&](int z, int k) -> float& {
-        const int row = k / 190, rem = k - row * 190, d = rem / 38, col = 1 + rem % 38;
-        return S.xrow[z & 1][row][d][col];
-    };
-    // out-of-range cells of the used window (rows 0 .. 11, columns 1 .. 38): at most 2 rows and 6 columns, 136
-    // cells; a thread's first cell is loaded before each wait, the few beyond NT after it, all directions of
-    // a cell together (one at a time, the loads' latencies added up to 9 us a plane)
-    const OutBand band(x0 - 4, y0 - 2, nx, ny, 0, TBY, 1, TBX - 1);
+    // out-of-range nodes among those pulled from (rows y0 - 3 .. y0 + 10, columns x0 - 3 .. x0 + 34): at most 3 rows
+    // and 6 columns, 3 * 38 + 6 * 11 = 180, one per thread, loaded before each wait
+    const OutBand band(x0 - 4, y0 - 3, nx, ny, 0, TYY, 1, TBX - 1);
     const bool edge = band.cells > 0;
-    auto band_load = [&](int k, int zl, float (&v)[Q]) {
-        int rb, c;
-        band.cell(k, 1, rb, c);
-        const float* p = fin + (long long)wrap1(y0 - 2 + rb, ny) * fp + wrap1(x0 - 4 + c, nx);
-        const int pz[3] = {wz(zl - 1) * fxy, wz(zl) * fxy, wz(zl + 1) * fxy};
-#pragma unroll
-        for (int a = 0; a < Q; ++a) v[a] = p[a * fs + pz[1 - L::ez(a)]];
-    };
-    auto band_store = [&](int k, float* st, const float (&v)[Q]) {
-        int rb, c;
-        band.cell(k, 1, rb, c);
-#pragma unroll
-        for (int a = 0; a < Q; ++a) st[a * TBSLOT + rb * TBX + c] = v[a];
-    };
+    int fr = 0, fcl = 0;
+    const float* fsrc = nullptr;
+    if (tid < band.cells) {
+        band.cell(tid, 1, fr, fcl);
+        fsrc = fin + (long long)wrap1(y0 - 3 + fr, ny) * fp + wrap1(x0 - 4 + fcl, nx);
+    }
     auto issue = [&](int zl, int s) {   // lane 0 of every warp, as in bulk
         fence_proxy_async();
-        if (ly == 0) mbar_expect_tx(&bar[s], TBYTES_BULK);
+        if (ly == 0) mbar_expect_tx(&bar[s], SOLID_BYTES);
         for (int a = ly; a < Q; a += TTY)
-            tma_box3(S.stage[s][a], tmap, x0 - 4, y0 - 2, a * nz + wz(zl - ez_rt(a)), &bar[s]);
+            tma_box3(S.stage[s] + a * SSLOT, static_cast<const char*>(tmap) + 256, x0 - 4, y0 - 2 - ey_rt(a),
+                     a * nz + wz(zl - ez_rt(a)), &bar[s]);
     };
     if (lx == 0) {
         issue(zlo, 0);
@@ -841,54 +851,44 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
     }
     for (int z = zlo - 3; z <= zlo + 1; ++z)
         for (int k = tid; k < TTYPES; k += NT) S.type[z & 7][k] = type_src(z, k);
-    for (int k = tid; k < 380; k += NT) xrow_dst(zlo, k) = xrow_src(zlo, k);
     __syncthreads();
 
     // post-collision value f*_{opp(a)} of box cell (rb, c) on plane z (bounce-back source)
     auto bb_src = [&](int a, int z, int rb, int c) {
         return fin[L::opp(a) * fs + (long long)wz(z) * fxy + wrap1(y0 - 2 + rb, ny) * fp + wrap1(x0 - 4 + c, nx)];
     };
-    // pull of a fluid cell (rb, c) of plane zl with its type t; RING2: the cell may lie on box row 0
-    // or 11, whose pulls reach the rows beyond the box
-    // stn: the other stage (lead plane zl + 1, waited for) or null.  Bounce-back sources f*_abar of the
-    // cell's own plane: for e_az = 0 in this stage's box of abar, for e_az = -1 in the next stage's
-    // (its box of abar holds plane zl), otherwise plain loads.
-    auto pull = [&](auto ring2, const float* st, const float* stn, int zl, int rb, int c, uint8_t t,
-                    float (&v)[Q]) {
+    // pull of a fluid cell (rb, c) of plane zl with its type t: row rb of every direction's box.  stn: the other
+    // stage (lead plane zl + 1, waited for) or null.  Bounce-back sources f*_abar of the cell itself lie in the
+    // box of abar, row rb - e_ay (outside it for some cells of the outer ring), of this stage for e_az = 0 and of
+    // the next stage for e_az = -1; the others are plain loads.
+    auto pull = [&](const float* st, const float* stn, int zl, int rb, int c, uint8_t t, float (&v)[Q]) {
 #pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            const int ey = L::ey(a), sr = rb - ey;
-            if (decltype(ring2)::value && ey != 0 && (sr < 0 || sr >= TBY))
-                v[a] = S.xrow[zl & 1][sr < 0 ? 0 : 1][xrow_slot(a)][c - L::ex(a)];
-            else
-                v[a] = st[a * TBSLOT + sr * TBX + c - L::ex(a)];
-        }
+        for (int a = 0; a < Q; ++a) v[a] = st[a * SSLOT + rb * TBX + c - L::ex(a)];
         if (!(t & T_BULK)) {
 #pragma unroll
             for (int a = 1; a < Q; ++a) {
                 const uint8_t tu = S.type[(zl - L::ez(a)) & 7][(rb - L::ey(a) + 1) * TYX + c - L::ex(a) - 1];
                 if (tu & T_SOLID) {
-                    if (L::ez(a) == 0)
-                        v[a] = st[L::opp(a) * TBSLOT + rb * TBX + c];
-                    else if (L::ez(a) < 0 && stn)
-                        v[a] = stn[L::opp(a) * TBSLOT + rb * TBX + c];
+                    const int r = rb - L::ey(a);
+                    const bool in = L::ey(a) == 0 || unsigned(r) < unsigned(SROWS);
+                    if (L::ez(a) == 0 && in)
+                        v[a] = st[L::opp(a) * SSLOT + r * TBX + c];
+                    else if (L::ez(a) < 0 && in && stn)
+                        v[a] = stn[L::opp(a) * SSLOT + r * TBX + c];
                     else
                         v[a] = bb_src(a, zl, rb, c);
                 }
             }
         }
     };
-    using NoRing2 = std::integral_constant<bool, false>;
-    using Ring2 = std::integral_constant<bool, true>;
     const int pc = (ly + 1) * TPX + lx + 1;   // own cell in the psi window
     const int rc = (ly + 2) * TRX + lx + 2;   // own cell in the density window
     const int tcl = (ly + 3) * TYX + lx + 3;  // own cell in the type window
     V1 f1[Q], f2[Q];                          // own values of planes zl - 1 and zl - 2
 #pragma unroll
     for (int a = 0; a < Q; ++a) f1[a].v = f2[a].v = 0.0f;
-    constexpr int TN = (TTYPES + NT - 1) / NT, XN = (380 + NT - 1) / NT;
+    constexpr int TN = (TTYPES + NT - 1) / NT;
     uint8_t tnext[TN];                        // types of plane zl + 2 (this thread's cells)
-    float xnext[XN];                          // the rows beyond the box of plane zl + 1
 
 #pragma unroll 1
     for (int i = 0; i < nlead; ++i) {
@@ -898,20 +898,22 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
             const int k = tid + j * NT;
             tnext[j] = k < TTYPES ? type_src(zl + 2, k) : uint8_t(0);
         }
-#pragma unroll
-        for (int j = 0; j < XN; ++j) {
-            const int k = tid + j * NT;
-            xnext[j] = (k < 380 && zl + 1 <= zhi) ? xrow_src(zl + 1, k) : 0.0f;
-        }
         float patch[Q];
-        if (edge && tid < band.cells) band_load(tid, zl, patch);
+        if (edge && tid < band.cells) {
+            const int pz[3] = {wz(zl - 1) * fxy, wz(zl) * fxy, wz(zl + 1) * fxy};
+#pragma unroll
+            for (int a = 0; a < Q; ++a) patch[a] = fsrc[a * fs + pz[1 - L::ez(a)]];
+        }
         if (!mbar_wait(&bar[s], unsigned(i >> 1) & 1u, ZT_POLL_LIMIT)) atomicOr(err, ERR_TIMEOUT);
-        float* st = S.stage[s][0];
+        float* st = S.stage[s];
         if (edge) {
-            if (tid < band.cells) band_store(tid, st, patch);
-            for (int k = tid + NT; k < band.cells; k += NT) {
-                band_load(k, zl, patch);
-                band_store(k, st, patch);
+            if (tid < band.cells) {
+                // node (x0 - 4 + fcl, y0 - 3 + fr) in every direction's box that covers it
+#pragma unroll
+                for (int a = 0; a < Q; ++a) {
+                    const int r = fr - 1 + L::ey(a);
+                    if (unsigned(r) < unsigned(SROWS)) st[a * SSLOT + r * TBX + fcl] = patch[a];
+                }
             }
             fence_proxy_async();
             __syncthreads();
@@ -920,7 +922,7 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
         const float* stn = nullptr;
         if (!edge && zl + 1 <= zhi) {
             if (!mbar_wait(&bar[s ^ 1], unsigned((i + 1) >> 1) & 1u, ZT_POLL_LIMIT)) atomicOr(err, ERR_TIMEOUT);
-            stn = S.stage[s ^ 1][0];
+            stn = S.stage[s ^ 1];
         }
         // A. densities of the density window, psi of the psi window (fluid cells), own values kept
         const uint8_t* ty = S.type[zl & 7];
@@ -933,7 +935,7 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
             const bool fl = !(t & T_SOLID);
             V1 rho = {0.0f}, ps = {0.0f};
             if (fl) {
-                pull(NoRing2{}, st, stn, zl, ly + 2, lx + 4, t, v);
+                pull(st, stn, zl, ly + 2, lx + 4, t, v);
                 V1 d = {v[0]};
 #pragma unroll
                 for (int a = 1; a < Q; ++a) d = d + V1{v[a]};
@@ -965,7 +967,7 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
             float rho = 0.0f;
             if (fl) {
                 float v[Q];
-                pull(Ring2{}, st, stn, zl, rb, c, t, v);
+                pull(st, stn, zl, rb, c, t, v);
                 V1 d = {v[0]};
 #pragma unroll
                 for (int a = 1; a < Q; ++a) d = d + V1{v[a]};
@@ -978,8 +980,7 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
         if (lx == 0 && zl + 2 <= zhi) issue(zl + 2, s);
 
         // B. wall cells of plane zw = zl - 1: virtual density and its psi (the solid-fluid interaction
-        // scheme keeps psi = 0 on solids); node types of plane zl + 2 and the rows beyond the box of
-        // plane zl + 1 into their rings
+        // scheme keeps psi = 0 on solids); node types of plane zl + 2 into their ring
         const int zw = zl - 1;
         if (!SF && zw >= zb - 1) {
             const uint8_t* tw = S.type[zw & 7];
@@ -1017,11 +1018,6 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
         for (int j = 0; j < TN; ++j) {
             const int k = tid + j * NT;
             if (k < TTYPES) S.type[(zl + 2) & 7][k] = tnext[j];
-        }
-#pragma unroll
-        for (int j = 0; j < XN; ++j) {
-            const int k = tid + j * NT;
-            if (k < 380) xrow_dst(zl + 1, k) = xnext[j];
         }
         __syncthreads();
 
@@ -1125,12 +1121,11 @@ __global__ void __launch_bounds__(TNT, 2)
     const int x0 = xs + TTX <= g.nx ? xs : (g.nx - TTX + 3) / 4 * 4, y0 = min(ys, g.ny - TTY);
     ZTSmem& S = *reinterpret_cast<ZTSmem*>(smem_raw);
     if (threadIdx.x == 0 && threadIdx.y == 0) {
-        mbar_init(&S.bar[0]);
-        mbar_init(&S.bar[1]);
+        for (int k = 0; k < BST; ++k) mbar_init(&S.bar[k]);
         fence_mbar_init();
     }
     __syncthreads();
-    // tmap: the input buffer's map (box TBX x TBY x 1)
+    // tmap: the input buffer's maps
     if (!it.solid)
         ztma_chunk_bulk<MODE>(fin, fout, tmap, g, ph, kr, x0, y0, xs, ys, zb, ze, err, S.b, S.bar, out);
     else if (ph.wall_kind == 2)
@@ -1193,9 +1188,10 @@ cudaError_t launch_ztma_fields(const void* fin, const void* tmap, const Geo& g, 
     return launch_ztma<1>(fin, nullptr, tmap, g, p, ZTOut{rho, u, g.N}, s);
 }
 
-void ztma_box_dims(int* bx, int* by) {
-    *bx = TBX;
-    *by = TBY;
+int ztma_maps(int k, int* bx, int* by) {
+    *bx = k == 1 ? box_cols(1) : TBX;
+    *by = k == 2 ? SROWS : BROWS;
+    return ZMAPS;
 }
 
 #ifndef LBMWET_ZWL_MIN_RUN   // shortest bulk run kept on the bulk path, and shortest piece (planes)
@@ -1291,21 +1287,39 @@ std::vector<ZItem> ztma_items(const uint8_t* mask, int nx, int ny, int nz, int s
     std::vector<ZItem> none;
     const std::vector<ZItem> runs =
         column_runs(mask, nx, ny, nz, large ? LBMWET_ZWL_MIN_RUN : 4, [](int, int) { return true; }, &none);
-    if (large) return aligned_items(runs, none);
+    if (large) {
+        // the last layer of bulk pieces in quarters, so that the launch ends on short items (256^3: 561 us a
+        // step with whole ones, 547 with halves, 542 with quarters)
+        std::vector<ZItem> items;
+        const std::vector<ZItem> whole = aligned_items(runs, none);
+        const int zt = (nz - 1) / TCH * TCH;
+        auto last = [&](const ZItem& r) { return r.z0 >= zt && !r.solid && r.z1 - r.z0 >= 8; };
+        for (const ZItem& r : whole)
+            if (!last(r)) items.push_back(r);
+        for (int k = 0; k < 4; ++k)
+            for (const ZItem& r : whole) {
+                const int len = r.z1 - r.z0;
+                if (last(r)) items.push_back(ZItem{r.bx, r.by, r.z0 + k * len / 4, r.z0 + (k + 1) * len / 4, 0});
+            }
+        return items;
+    }
     // A grid of less than two waves: shorter pieces, of lengths chosen for the least time.  A piece of c planes
     // takes c + 3 plane times on the bulk path (two halo planes, start-up) and c + 5 on the solid path, whose
     // plane takes three times as long (256^3: 2.3 and 6.7 us); a launch takes as long as its longest piece and
     // at least its total over the slots.  The solid pieces start first.
     auto pieces = [](int len, int c) { return (len + c - 1) / c; };
+    std::map<std::pair<int, int>, int> lengths;   // (planes, solid) -> runs
+    for (const ZItem& r : runs) ++lengths[{r.z1 - r.z0, r.solid}];
     double best = 1e300;
     int cb = TCH, cs = TCH;
     for (int b : {32, 26, 22, 18, 16, 14, 12, 11, 10, 9, 8, 7, 6, 5, 4, 3, 2})
         for (int q : {32, 16, 12, 8, 6, 5, 4, 3, 2, 1}) {
             double total = 0.0, longest = 0.0;
-            for (const ZItem& r : runs) {
-                const int len = r.z1 - r.z0, n = pieces(len, r.solid ? q : b), c = (len + n - 1) / n;
-                const double t = r.solid ? 3.0 * (c + 5) : c + 3.0;
-                total += n * t;
+            for (const auto& kv : lengths) {
+                const int len = kv.first.first, solid = kv.first.second, n = pieces(len, solid ? q : b);
+                const int c = (len + n - 1) / n;
+                const double t = solid ? 3.0 * (c + 5) : c + 3.0;
+                total += double(kv.second) * n * t;
                 longest = std::max(longest, t);
             }
             const double cost = std::max(longest, total / slots + 0.3 * longest);
