@@ -16,6 +16,7 @@
 
 #include "adjoint.h"
 #include "lattice.cuh"
+#include "pdl.cuh"
 
 namespace lbmwet {
 
@@ -43,6 +44,7 @@ __global__ void __launch_bounds__(TX* TY) adj_gather_push(DevParams p, const C* 
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const int tid = threadIdx.y * TX + threadIdx.x;
     const C G = C(p.G);
+    pdl_wait();
     // 0. types, psi and Fmbar on the tile + 2-node halo
     for (int i = tid; i < RX * RY; i += NT) {
         const int gx = wrap_any(x0 + i % RX - 2, nx), gy = wrap_any(y0 + i / RX - 2, ny);
@@ -149,11 +151,10 @@ cudaError_t adjoint_step_t(const void* fstar_k, const void* mu_next, void* mu_pr
     cudaError_t e = launch_adjoint_local(std::is_same<S, double>::value ? PREC_FP64 : PREC_FP32, fstar_k, p, f, s);
     if (e != cudaSuccess) return e;
     dim3 grid((p.nx + GX - 1) / GX, (p.ny + GY - 1) / GY, 1);
-    adj_gather_push<S, GX, GY><<<grid, dim3(GX, GY, 1), 0, s>>>(
-        p, static_cast<const S*>(f.psi), static_cast<const S*>(f.dpsi), static_cast<const S*>(f.drw_k),
-        static_cast<const S*>(f.drw_a), static_cast<const S*>(f.fmb_x), static_cast<const S*>(f.fmb_y),
-        static_cast<const S*>(f.psib), static_cast<const S*>(f.lam), dkappa, static_cast<S*>(mu_prev));
-    return cudaGetLastError();
+    return launch_pdl(adj_gather_push<S, GX, GY>, grid, dim3(GX, GY, 1), 0, s, p, static_cast<const S*>(f.psi),
+                      static_cast<const S*>(f.dpsi), static_cast<const S*>(f.drw_k), static_cast<const S*>(f.drw_a),
+                      static_cast<const S*>(f.fmb_x), static_cast<const S*>(f.fmb_y), static_cast<const S*>(f.psib),
+                      static_cast<const S*>(f.lam), dkappa, static_cast<S*>(mu_prev));
 }
 
 unsigned grid_of(long long n) {

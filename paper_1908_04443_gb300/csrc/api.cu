@@ -1932,34 +1932,41 @@ extern "C" lbm_status lbm_adjoint(lbm_handle* h, const double* drho_final_dev, d
     const int64_t nck = (int64_t)h->ckpt.size();
     const size_t es = h->prec == LBM_FP64 ? sizeof(double) : sizeof(float);
     // Two segment buffers: slot 0 of a buffer receives a copy of a segment's checkpoint, slots 1.. the
-    // recomputed states.  Pass t reverses segment nck - t (recomputed by pass t - 1) and, on a second
-    // branch of the same CUDA graph, recomputes segment nck - 1 - t into the other buffer: the two
-    // branches share no data, so the recomputation hides behind the latency-bound reverse kernels.
-    // The checkpoint copy is issued before the graph, which therefore depends only on the two segment
-    // lengths, the adjoint-buffer parity and the buffer index, and is reused across passes.
+    // recomputed states.  Pass t reverses segment nck - t (recomputed by pass t - 1) on the handle's stream
+    // and, on a second stream, recomputes segment nck - 1 - t into the other buffer: the two share no data,
+    // so the recomputation hides behind the latency-bound reverse kernels.  Every launch is used once, so
+    // they are issued directly, each set up while the one before it ends (launch_pdl): capturing and
+    // instantiating graphs of the passes on every call kept the GPU idle in between, the more so with
+    // programmatic edges.  300 steps on 256 x 256, FP32, with 3 checkpoints (forward and adjoint): graphs
+    // 8.6 ms, graphs of programmatic launches 8.7, direct plain launches 8.8, this 6.9.  The buffers come
+    // from the pool, as cudaMalloc and cudaFree of this half a gigabyte wait for the device; more than
+    // ADJ_POOL_BYTES go back to the driver after the call, since the pool would keep them.
+    constexpr size_t ADJ_POOL_BYTES = size_t(1) << 30;
     void* seg[2] = {nullptr, nullptr};
     void* mu[2] = {nullptr, nullptr};
     void* scratch = nullptr;
     double* dk = nullptr;
-    cudaStream_t cap = nullptr, cap2 = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
-    struct Key {
-        int64_t rev_len, rec_len;
-        int par, rec_buf;
+    const size_t seg_bytes = h->fbytes * (size_t)every, dk_bytes = sizeof(double) * (nw ? nw : 1);
+    const size_t scratch_bytes = es * adjoint_scratch_elems(h->N);
+    const bool pooled = (nck > 1 ? 2 : 1) * seg_bytes + 2 * h->fbytes + scratch_bytes + dk_bytes <= ADJ_POOL_BYTES;
+    auto get = [&](auto** q, size_t bytes) { return pooled ? dmalloc(q, bytes, h->stream) : cudaMalloc(q, bytes); };
+    auto put = [&](void* q) {
+        if (pooled) dfree(q, h->stream);
+        else cudaFree(q);
     };
-    std::vector<std::pair<Key, cudaGraphExec_t>> graphs;
     lbm_status st = LBM_OK;
-    cudaError_t e = cudaMalloc(&seg[0], h->fbytes * (size_t)every);
-    if (e == cudaSuccess && nck > 1) e = cudaMalloc(&seg[1], h->fbytes * (size_t)every);
-    if (e == cudaSuccess) e = cudaMalloc(&mu[0], h->fbytes);
-    if (e == cudaSuccess) e = cudaMalloc(&mu[1], h->fbytes);
-    if (e == cudaSuccess) e = cudaMalloc(&scratch, es * adjoint_scratch_elems(h->N));
-    if (e == cudaSuccess) e = cudaMalloc(&dk, sizeof(double) * (nw ? nw : 1));
-    if (e == cudaSuccess) e = cudaMemsetAsync(dk, 0, sizeof(double) * (nw ? nw : 1), h->stream);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cap2, cudaStreamNonBlocking);
+    cudaError_t e = get(&seg[0], seg_bytes);
+    if (e == cudaSuccess && nck > 1) e = get(&seg[1], seg_bytes);
+    if (e == cudaSuccess) e = get(&mu[0], h->fbytes);
+    if (e == cudaSuccess) e = get(&mu[1], h->fbytes);
+    if (e == cudaSuccess) e = get(&scratch, scratch_bytes);
+    if (e == cudaSuccess) e = get(&dk, dk_bytes);
+    if (e == cudaSuccess) e = cudaMemsetAsync(dk, 0, dk_bytes, h->stream);
+    if (e == cudaSuccess && !h->cap_stream) e = cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
+    const cudaStream_t side = h->cap_stream;
     AdjointScratch w{scratch};
     int cur = 0;
     if (e == cudaSuccess) e = launch_adjoint_final(h->prec, drho_final_dev, mu[cur], h->dp, h->stream);
@@ -1967,64 +1974,42 @@ extern "C" lbm_status lbm_adjoint(lbm_handle* h, const double* drho_final_dev, d
         return static_cast<void*>(static_cast<char*>(seg[b]) + (size_t)i * h->fbytes);
     };
     auto seg_len = [&](int64_t c) { return c >= 0 && c < nck ? std::min(every, n - c * every) : int64_t(0); };
-    // one graph: reverse rev_len steps in buffer rec_buf ^ 1 || recompute rec_len - 1 steps in rec_buf
-    auto capture = [&](const Key& k, cudaGraphExec_t* ex) -> cudaError_t {
-        cudaGraph_t g = nullptr;
-        cudaError_t r0 = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-        if (r0 != cudaSuccess) return r0;
-        cudaError_t r = cudaEventRecord(fork, cap);
-        if (r == cudaSuccess) r = cudaStreamWaitEvent(cap2, fork, 0);
-        for (int64_t i = 0; i + 1 < k.rec_len && r == cudaSuccess; ++i)
-            r = launch_step(h->lat, h->prec, slot(k.rec_buf, i), slot(k.rec_buf, i + 1), h->dp, cap2);
-        int c2 = k.par;
-        for (int64_t i = k.rev_len - 1; i >= 0 && r == cudaSuccess; --i) {
-            r = launch_adjoint_step(h->prec, slot(k.rec_buf ^ 1, i), mu[c2], mu[c2 ^ 1], h->dp, w, dk, cap);
-            c2 ^= 1;
-        }
-        if (r == cudaSuccess) r = cudaEventRecord(join, cap2);
-        if (r == cudaSuccess) r = cudaStreamWaitEvent(cap, join, 0);
-        cudaError_t r1 = cudaStreamEndCapture(cap, &g);
-        if (r == cudaSuccess) r = r1;
-        if (r == cudaSuccess) r = cudaGraphInstantiate(ex, g, 0);
-        if (g) cudaGraphDestroy(g);
-        return r;
-    };
     for (int64_t t = 0; t <= nck && e == cudaSuccess; ++t) {
         // the buffer of pass t's recomputation; with one segment only buffer 0 exists and t = 1 only reverses
-        const Key k{seg_len(nck - t), seg_len(nck - 1 - t), cur, int(t & 1)};
-        if (k.rec_len > 0)
-            e = cudaMemcpyAsync(slot(k.rec_buf, 0), h->ckpt[nck - 1 - t], h->fbytes, cudaMemcpyDeviceToDevice,
-                                h->stream);
-        if (e != cudaSuccess) break;
-        cudaGraphExec_t ex = nullptr;
-        for (auto& kv : graphs)
-            if (kv.first.rev_len == k.rev_len && kv.first.rec_len == k.rec_len && kv.first.par == k.par &&
-                kv.first.rec_buf == k.rec_buf)
-                ex = kv.second;
-        if (!ex) {
-            e = capture(k, &ex);
-            if (e != cudaSuccess) break;
-            graphs.push_back({k, ex});
+        const int64_t rev_len = seg_len(nck - t), rec_len = seg_len(nck - 1 - t);
+        const int rec_buf = int(t & 1);
+        if (rec_len > 0) {   // the side stream starts when the pass before, which read this buffer, has ended
+            e = cudaEventRecord(fork, h->stream);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(side, fork, 0);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(slot(rec_buf, 0), h->ckpt[nck - 1 - t], h->fbytes, cudaMemcpyDeviceToDevice, side);
         }
-        e = cudaGraphLaunch(ex, h->stream);
-        if (k.rev_len % 2) cur ^= 1;
-        h->launches += (k.rec_len > 0 ? k.rec_len - 1 : 0) + 2 * k.rev_len;
+        // issued in turn, so that neither stream waits for the host to have issued all of the other's work
+        for (int64_t i = 0; i < std::max(rev_len, rec_len - 1) && e == cudaSuccess; ++i) {
+            if (i < rev_len) {
+                e = launch_adjoint_step(h->prec, slot(rec_buf ^ 1, rev_len - 1 - i), mu[cur], mu[cur ^ 1], h->dp, w, dk,
+                                        h->stream);
+                cur ^= 1;
+            }
+            if (e == cudaSuccess && i + 1 < rec_len)
+                e = launch_step(h->lat, h->prec, slot(rec_buf, i), slot(rec_buf, i + 1), h->dp, side);
+        }
+        if (e == cudaSuccess && rec_len > 0) {
+            e = cudaEventRecord(join, side);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, join, 0);
+        }
+        h->launches += (rec_len > 0 ? rec_len - 1 : 0) + 2 * rev_len;
     }
     if (e == cudaSuccess && nw)
         e = cudaMemcpyAsync(dkappa_host, dk, sizeof(double) * nw, cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) st = cuda_fail(h, e, "adjoint");
-    for (auto& kv : graphs) cudaGraphExecDestroy(kv.second);
-    if (cap) cudaStreamDestroy(cap);
-    if (cap2) cudaStreamDestroy(cap2);
+    if (e != cudaSuccess) {
+        st = cuda_fail(h, e, "adjoint");
+        if (side) cudaStreamSynchronize(side);   // (its work reads the buffers that go back below)
+    }
     if (fork) cudaEventDestroy(fork);
     if (join) cudaEventDestroy(join);
-    cudaFree(seg[0]);
-    cudaFree(seg[1]);
-    cudaFree(mu[0]);
-    cudaFree(mu[1]);
-    cudaFree(scratch);
-    cudaFree(dk);
+    for (void* q : {seg[0], seg[1], mu[0], mu[1], scratch, static_cast<void*>(dk)}) put(q);
     if (st != LBM_OK) return st;
     return check_device_error(h);
 }

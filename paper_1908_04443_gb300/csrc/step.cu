@@ -20,6 +20,7 @@
 #include "adjoint.h"
 #include "kernels.h"
 #include "lattice.cuh"
+#include "pdl.cuh"
 #include "tile_common.cuh"
 
 namespace lbmwet {
@@ -470,6 +471,7 @@ __global__ void __launch_bounds__(TileShape<L, S>::X* TileShape<L, S>::Y* TileSh
     __shared__ TileSmem<L, C, TS::X, TS::Y, TS::Z> sm;
     const int tile = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
     const bool solid = g.tile_solid ? g.tile_solid[tile] != 0 : true;
+    pdl_wait();
     if (solid)
         tile_body_w<L, S, C, TS::X, TS::Y, TS::Z, MODE, true>(fin, fout, g, ph, blockIdx.x * TS::X, blockIdx.y * TS::Y,
                                                               blockIdx.z * TS::Z, true, err, rho_out, u_out, sm);
@@ -520,6 +522,7 @@ __global__ void __launch_bounds__(TileShape<D2Q9, S>::X* TileShape<D2Q9, S>::Y, 
     __shared__ TileSmem<D2Q9, S, TS::X, TS::Y, 1, true> sm;
     const int tile = blockIdx.y * gridDim.x + blockIdx.x;
     const bool solid = g.tile_solid ? g.tile_solid[tile] != 0 : true;
+    pdl_wait();
     tile_body_w<D2Q9, S, S, TS::X, TS::Y, 1, 2, true>(fin, nullptr, g, ph, blockIdx.x * TS::X, blockIdx.y * TS::Y, 0,
                                                        solid, err, nullptr, nullptr, sm, &io);
 }
@@ -747,9 +750,8 @@ static cudaError_t launch_tile(const void* fin, void* fout, const DevParams& p, 
     using TS = TileShape<L, S>;
     dim3 grid((p.nx + TS::X - 1) / TS::X, (p.ny + TS::Y - 1) / TS::Y, (p.nz + TS::Z - 1) / TS::Z);
     dim3 block(TS::X, TS::Y, TS::Z);
-    fused_step<L, S, S, MODE><<<grid, block, 0, s>>>(static_cast<const S*>(fin), static_cast<S*>(fout), geo_of(p),
-                                                     make_phys<S>(p), p.err, rho, u);
-    return cudaGetLastError();
+    return launch_pdl(fused_step<L, S, S, MODE>, grid, block, 0, s, static_cast<const S*>(fin), static_cast<S*>(fout),
+                      geo_of(p), make_phys<S>(p), p.err, rho, u);
 }
 
 template <int MODE>
@@ -803,9 +805,8 @@ static cudaError_t adj_local_t(const void* fstar, const DevParams& p, const Adjo
     io.drw_k = static_cast<S*>(w.drw_k);
     io.drw_a = static_cast<S*>(w.drw_a);
     dim3 grid((p.nx + TS::X - 1) / TS::X, (p.ny + TS::Y - 1) / TS::Y, 1);
-    adjoint_local_tile<S><<<grid, dim3(TS::X, TS::Y, 1), 0, s>>>(static_cast<const S*>(fstar), geo_of(p),
-                                                                  make_phys<S>(p), p.err, io);
-    return cudaGetLastError();
+    return launch_pdl(adjoint_local_tile<S>, grid, dim3(TS::X, TS::Y, 1), 0, s, static_cast<const S*>(fstar), geo_of(p),
+                      make_phys<S>(p), p.err, io);
 }
 
 cudaError_t launch_adjoint_local(int prec, const void* fstar, const DevParams& p, const AdjointFields& w,

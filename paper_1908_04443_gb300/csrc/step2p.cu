@@ -20,6 +20,7 @@
 
 #include "kernels.h"
 #include "lattice.cuh"
+#include "pdl.cuh"
 #include "pack2.cuh"
 #include "tile_common.cuh"
 
@@ -477,6 +478,7 @@ __global__ void __launch_bounds__(PTX* PTY, LBMWET_PAIR_MINB)
     __shared__ float hst[9 * PairSmem::SHELL];
     const int tile = blockIdx.y * gridDim.x + blockIdx.x;
     const bool solid = tile_solid ? tile_solid[tile] != 0 : true;
+    pdl_wait();
     if (solid) pair_tile<true>(g, 0, ph, kr, blockIdx.x * PTX, blockIdx.y * PNY, err, sm, hst);
     else pair_tile<false>(g, 0, ph, kr, blockIdx.x * PTX, blockIdx.y * PNY, err, sm, hst);
 }
@@ -527,10 +529,11 @@ __global__ void __launch_bounds__(PTX* PTY, LBMWET_PAIR_MINB)
     if (tid == 0) {
         s_idx[0] = blockIdx.x;
         s_idx[1] = blockIdx.x + grid;
-        if (blockIdx.x < n_items) claim = atomicAdd(sched, 1u);
         mbar_init(&bar);
         fence_mbar_init();
     }
+    pdl_wait();
+    if (tid == 0 && blockIdx.x < n_items) claim = atomicAdd(sched, 1u);   // (the launch before resets the counter)
     __syncthreads();
     // 1: the tile pulls from a TMA box, 0: from global memory
     auto box_kind = [](const BatchItem& r) -> int {
@@ -655,15 +658,14 @@ int pair_ctas_per_sm() {
 cudaError_t launch_pair_step(const void* fin, void* fout, const DevParams& p, cudaStream_t s) {
     const PairGrid g = pair_grid(fin, fout, p);
     dim3 grid((p.nx + PTX - 1) / PTX, (p.ny + PNY - 1) / PNY, 1);
-    pair_step<<<grid, dim3(PTX, PTY, 1), 0, s>>>(g, p.pair_solid, make_phys<float>(p), make_pair_rates(p), p.err);
-    return cudaGetLastError();
+    return launch_pdl(pair_step, grid, dim3(PTX, PTY, 1), 0, s, g, p.pair_solid, make_phys<float>(p), make_pair_rates(p),
+                      p.err);
 }
 
 cudaError_t launch_pair_batched(int parity, const DevParams& p, const BatchItem* items, int n_items, int ctas,
                                 unsigned* sched, cudaStream_t s) {
-    pair_step_batched<<<ctas, dim3(PTX, PTY, 1), 0, s>>>(parity, items, n_items, make_phys<float>(p),
-                                                         make_pair_rates(p), p.err, sched);
-    return cudaGetLastError();
+    return launch_pdl(pair_step_batched, dim3(ctas), dim3(PTX, PTY, 1), 0, s, parity, items, n_items, make_phys<float>(p),
+                      make_pair_rates(p), p.err, sched);
 }
 
 }  // namespace lbmwet

@@ -12,6 +12,7 @@
 #include "fp64.cuh"
 #include "kernels.h"
 #include "lattice.cuh"
+#include "pdl.cuh"
 #include "tile_common.cuh"
 
 namespace lbmwet {
@@ -220,7 +221,9 @@ __global__ void __launch_bounds__(NT, RESIDENT)
              double* __restrict__ u_out) {
     __shared__ Smem sm;
     const int x0 = int(blockIdx.x) << wl, y0 = int(blockIdx.y) * h, zb = int(blockIdx.z) * zc;
-    if (flags[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x])
+    const bool solid = flags[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] != 0;
+    pdl_wait();
+    if (solid)
         brick64<MODE, true>(fin, fout, g, ph, x0, y0, zb, wl, h, zc, err, rho_out, u_out, sm);
     else
         brick64<MODE, false>(fin, fout, g, ph, x0, y0, zb, wl, h, zc, err, rho_out, u_out, sm);
@@ -260,12 +263,10 @@ cudaError_t launch_d3q19_fp64(int mode, const void* fin, void* fout, const Geo& 
     const dim3 grid((p.nx + p.tile_w - 1) / p.tile_w, (p.ny + p.tile_h - 1) / p.tile_h, (p.nz + p.tile_z - 1) / p.tile_z);
     const double* in = static_cast<const double*>(fin);
     if (mode == 0)
-        step3d64<0><<<grid, NT, 0, s>>>(in, static_cast<double*>(fout), g, p.pair_solid, make_phys<double>(p), wl, p.tile_h,
-                                        p.tile_z, p.err, nullptr, nullptr);
-    else
-        step3d64<1><<<grid, NT, 0, s>>>(in, nullptr, g, p.pair_solid, make_phys<double>(p), wl, p.tile_h, p.tile_z, p.err,
-                                        rho, u);
-    return cudaGetLastError();
+        return launch_pdl(step3d64<0>, grid, dim3(NT), 0, s, in, static_cast<double*>(fout), g, p.pair_solid,
+                          make_phys<double>(p), wl, p.tile_h, p.tile_z, p.err, nullptr, nullptr);
+    return launch_pdl(step3d64<1>, grid, dim3(NT), 0, s, in, nullptr, g, p.pair_solid, make_phys<double>(p), wl, p.tile_h,
+                      p.tile_z, p.err, rho, u);
 }
 
 }  // namespace lbmwet

@@ -20,6 +20,7 @@
 
 #include "kernels.h"
 #include "lattice.cuh"
+#include "pdl.cuh"
 #include "maskscan.h"
 #include "pack2.cuh"
 #include "tile_common.cuh"
@@ -1124,6 +1125,7 @@ __global__ void __launch_bounds__(TNT, 2)
         for (int k = 0; k < BST; ++k) mbar_init(&S.bar[k]);
         fence_mbar_init();
     }
+    pdl_wait();
     __syncthreads();
     // tmap: the input buffer's maps
     if (!it.solid)
@@ -1172,10 +1174,8 @@ static cudaError_t launch_ztma(const void* fin, void* fout, const void* tmap, co
         attr[dev] = true;
     }
     if (!p.zitems || p.nzitems < 1) return cudaErrorInvalidValue;
-    ztma_step<MODE><<<p.nzitems, dim3(TTX, TTY, 1), ZT_SMEM, s>>>(static_cast<const float*>(fin), static_cast<float*>(fout),
-                                                                 tmap, g, make_phys<float>(p), make_rates3p(p), p.err,
-                                                                 p.zitems, out);
-    return cudaGetLastError();
+    return launch_pdl(ztma_step<MODE>, dim3(p.nzitems), dim3(TTX, TTY, 1), ZT_SMEM, s, static_cast<const float*>(fin),
+                      static_cast<float*>(fout), tmap, g, make_phys<float>(p), make_rates3p(p), p.err, p.zitems, out);
 }
 
 cudaError_t launch_ztma_step(const void* fin, void* fout, const void* tmap, const Geo& g, const DevParams& p,

@@ -13,6 +13,7 @@
 #include "fp64.cuh"
 #include "kernels.h"
 #include "lattice.cuh"
+#include "pdl.cuh"
 #include "tile_common.cuh"
 
 namespace lbmwet {
@@ -242,7 +243,9 @@ __global__ void __launch_bounds__(NT, 2) step64(PairGrid g, const uint8_t* __res
                                                 double* __restrict__ u_out) {
     __shared__ Smem64 sm;
     const int x0 = int(blockIdx.x) << wl, y0 = int(blockIdx.y) * h;
-    if (flags[blockIdx.y * gridDim.x + blockIdx.x])
+    const bool solid = flags[blockIdx.y * gridDim.x + blockIdx.x] != 0;
+    pdl_wait();
+    if (solid)
         body64<MODE, true>(g, 0, ph, x0, y0, wl, h, err, rho_out, u_out, sm);
     else
         body64<MODE, false>(g, 0, ph, x0, y0, wl, h, err, rho_out, u_out, sm);
@@ -253,7 +256,9 @@ __global__ void __launch_bounds__(NT, 2) step64_batched(int parity, const BatchI
                                                         Phys<double> ph, int wl, int h, unsigned* err) {
     __shared__ Smem64 sm;
     const BatchItem& g = items[blockIdx.x];
-    if (g.solid) body64<0, true>(g, parity, ph, g.x0, g.y0, wl, h, err, nullptr, nullptr, sm);
+    const bool solid = g.solid != 0;
+    pdl_wait();
+    if (solid) body64<0, true>(g, parity, ph, g.x0, g.y0, wl, h, err, nullptr, nullptr, sm);
     else body64<0, false>(g, parity, ph, g.x0, g.y0, wl, h, err, nullptr, nullptr, sm);
 }
 
@@ -317,18 +322,17 @@ cudaError_t launch_d2q9_fp64(int mode, const void* fin, void* fout, const DevPar
     const PairGrid g = pair_grid(fin, fout, p);
     const dim3 grid((p.nx + p.tile_w - 1) / p.tile_w, (p.ny + p.tile_h - 1) / p.tile_h, 1);
     if (mode == 0)
-        step64<0><<<grid, NT, 0, s>>>(g, p.pair_solid, make_phys<double>(p), log2_of(p.tile_w), p.tile_h, p.err, nullptr,
-                                      nullptr);
-    else
-        step64<1><<<grid, NT, 0, s>>>(g, p.pair_solid, make_phys<double>(p), log2_of(p.tile_w), p.tile_h, p.err, rho, u);
-    return cudaGetLastError();
+        return launch_pdl(step64<0>, grid, dim3(NT), 0, s, g, p.pair_solid, make_phys<double>(p), log2_of(p.tile_w), p.tile_h,
+                          p.err, nullptr, nullptr);
+    return launch_pdl(step64<1>, grid, dim3(NT), 0, s, g, p.pair_solid, make_phys<double>(p), log2_of(p.tile_w), p.tile_h,
+                      p.err, rho, u);
 }
 
 cudaError_t launch_d2q9_fp64_batched(int parity, const DevParams& p, const BatchItem* items, int n_items, int tw, int th,
                                      cudaStream_t s) {
     if (n_items < 1) return cudaSuccess;
-    step64_batched<<<n_items, NT, 0, s>>>(parity, items, make_phys<double>(p), log2_of(tw), th, p.err);
-    return cudaGetLastError();
+    return launch_pdl(step64_batched, dim3(n_items), dim3(NT), 0, s, parity, items, make_phys<double>(p), log2_of(tw), th,
+                      p.err);
 }
 
 cudaError_t launch_d2q9_fp64_fields(const FieldGrid* grids, int ngrids, int total_tiles, const DevParams& p,
