@@ -22,9 +22,14 @@ namespace lbmwet {
 
 namespace {
 
+// v into 0 .. n-1: a division only where one wrap is not enough (grids narrower than a tile)
 __device__ __forceinline__ int wrap_any(int v, int n) {
-    v %= n;
-    return v < 0 ? v + n : v;
+    v = v < 0 ? v + n : (v >= n ? v - n : v);
+    if (unsigned(v) >= unsigned(n)) {
+        v %= n;
+        if (v < 0) v += n;
+    }
+    return v;
 }
 
 // psi-bar gathered through Eq. 5, rho-bar / kappa-bar, and the push (transpose of the pull), for a
@@ -44,19 +49,46 @@ __global__ void __launch_bounds__(TX* TY) adj_gather_push(DevParams p, const C* 
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const int tid = threadIdx.y * TX + threadIdx.x;
     const C G = C(p.G);
-    pdl_wait();
     // 0. types, psi and Fmbar on the tile + 2-node halo
-    for (int i = tid; i < RX * RY; i += NT) {
-        const int gx = wrap_any(x0 + i % RX - 2, nx), gy = wrap_any(y0 + i / RX - 2, ny);
-        const int g = gy * nx + gx;
-        s_t[i] = p.type[g];
-        s_psi[i] = psi[g];
-        s_fx[i] = fmb_x[g];
-        s_fy[i] = fmb_y[g];
+    constexpr int NR = (RX * RY + NT - 1) / NT, NP = (PX * PY + NT - 1) / NT;
+    int gr[NR];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+        const int i = tid + k * NT;
+        gr[k] = wrap_any(y0 + i / RX - 2, ny) * nx + wrap_any(x0 + i % RX - 2, nx);
+        if (i < RX * RY) s_t[i] = p.type[gr[k]];
     }
+    pdl_wait();   // (the types are as the grid's set-up left them)
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+        const int i = tid + k * NT;
+        if (i < RX * RY) {
+            s_psi[i] = psi[gr[k]];
+            s_fx[i] = fmb_x[gr[k]];
+            s_fy[i] = fmb_y[gr[k]];
+        }
+    }
+    // what steps 1 and 2 read per node: asked for here, so that the three steps wait for memory once
+    const int lx = threadIdx.x, ly = threadIdx.y;
+    const int gx = x0 + lx, gy = y0 + ly, gn = gy * nx + gx;
+    const bool in = gx < nx && gy < ny;
+    int gp[NP];
+    C own_pb[NP], own_dp[NP], own_lam[9];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+        const int i = tid + k * NT;
+        gp[k] = wrap_any(y0 + i / PX - 1, ny) * nx + wrap_any(x0 + i % PX - 1, nx);
+        own_pb[k] = i < PX * PY ? psib[gp[k]] : C(0);
+        own_dp[k] = i < PX * PY ? dpsi[gp[k]] : C(0);
+    }
+#pragma unroll
+    for (int a = 0; a < 9; ++a) own_lam[a] = in ? lam[a * N + gn] : C(0);   // (solid nodes: not used)
     __syncthreads();
     // 1. psi-bar on the tile + 1-node halo; fluid -> rho-bar, wall -> kappa-bar and the Eq. 17 weight
-    for (int i = tid; i < PX * PY; i += NT) {
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+        const int i = tid + k * NT;
+        if (i >= PX * PY) break;
         const int px = i % PX, py = i / PX;
         const int r = (py + 1) * RX + px + 1;
         const uint8_t t = s_t[r];
@@ -66,16 +98,15 @@ __global__ void __launch_bounds__(TX* TY) adj_gather_push(DevParams p, const C* 
             s_wb[i] = C(0);
             continue;
         }
-        const int gx = wrap_any(x0 + px - 1, nx), gy = wrap_any(y0 + py - 1, ny);
-        const int g = gy * nx + gx;
-        C pb = fluid ? psib[g] : C(0);
+        const int g = gp[k];
+        C pb = fluid ? own_pb[k] : C(0);
 #pragma unroll
         for (int a = 1; a < 9; ++a) {
             const int rs = r - D2Q9::ex(a) - D2Q9::ey(a) * RX;
             if (s_t[rs] & T_SOLID) continue;
             pb += -G * s_psi[rs] * C(D2Q9::wf(a)) * (s_fx[rs] * C(D2Q9::ex(a)) + s_fy[rs] * C(D2Q9::ey(a)));
         }
-        const C rb = pb * dpsi[g];
+        const C rb = pb * own_dp[k];
         if (fluid) {
             s_rb[i] = rb;
             s_wb[i] = C(0);
@@ -88,8 +119,7 @@ __global__ void __launch_bounds__(TX* TY) adj_gather_push(DevParams p, const C* 
     }
     __syncthreads();
     // 2. lambda = lam + rho-bar at the tile's fluid nodes, pushed to mu (the transpose of the pull)
-    const int lx = threadIdx.x, ly = threadIdx.y;
-    if (x0 + lx >= nx || y0 + ly >= ny) return;
+    if (!in) return;
     const int r = (ly + 2) * RX + lx + 2;
     if (s_t[r] & T_SOLID) return;
     const int pi = (ly + 1) * PX + lx + 1;
@@ -99,13 +129,12 @@ __global__ void __launch_bounds__(TX* TY) adj_gather_push(DevParams p, const C* 
         if (s_t[r + D2Q9::ex(a) + D2Q9::ey(a) * RX] & T_WALL)
             rb += C(D2Q9::wf(a)) * s_wb[pi + D2Q9::ex(a) + D2Q9::ey(a) * PX];
     }
-    const int gx = x0 + lx, gy = y0 + ly, g = gy * nx + gx;
 #pragma unroll
     for (int a = 0; a < 9; ++a) {
-        const C l = lam[a * N + g] + rb;
+        const C l = own_lam[a] + rb;
         const int rs = r - D2Q9::ex(a) - D2Q9::ey(a) * RX;
         if (s_t[rs] & T_SOLID) {
-            mu_out[D2Q9::opp(a) * N + g] = l;
+            mu_out[D2Q9::opp(a) * N + gn] = l;
         } else {
             const int sx = wrap_any(gx - D2Q9::ex(a), nx), sy = wrap_any(gy - D2Q9::ey(a), ny);
             mu_out[a * N + sy * nx + sx] = l;

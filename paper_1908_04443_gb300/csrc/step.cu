@@ -185,8 +185,12 @@ __device__ __forceinline__ void tile_body(const S* __restrict__ fin, S* __restri
     const int my_ti = tix(lx + 3, ly + 3, lz + YZH);
     const uint8_t my_type = type_at(my_ti);
     const bool my_fluid = !(my_type & T_SOLID);
-    C f[Q];
+    C f[Q], m[MODE == 2 ? Q : 1];
     C my_drho = C(0);
+    if constexpr (MODE == 2) {   // asked for here: the collision waits for it otherwise
+#pragma unroll
+        for (int a = 0; a < Q; ++a) m[a] = my_fluid ? adj->mu[a * N + gi] : C(0);
+    }
     {
         C rho = C(0);
         if (my_fluid) {
@@ -392,9 +396,7 @@ __device__ __forceinline__ void tile_body(const S* __restrict__ fin, S* __restri
     }
     if constexpr (MODE == 2) {
         if constexpr (D == 2) {
-            C m[Q], fb[Q];
-#pragma unroll
-            for (int a = 0; a < Q; ++a) m[a] = adj->mu[a * N + gi];
+            C fb[Q];
             C bx, by, pb;
             collide_d2q9_adjoint<C>(f, m, rho, ux, uy, Fx, Fy, Fmx, Fmy, psi_c, ph.r, fb, bx, by, pb);
 #pragma unroll
@@ -404,9 +406,7 @@ __device__ __forceinline__ void tile_body(const S* __restrict__ fin, S* __restri
             // F_m = -G psi(x) sum w psi(x+e) e: its dependence on psi(x) is F_m / psi(x)
             adj->psib[gi] = pb + (bx * Fmx + by * Fmy) / psi_c;
             adj->psi[gi] = psi_c;
-            adj->dpsi[gi] = psi_slope(rho, psi_c, ph);
-            adj->drw_k[gi] = C(0);
-            adj->drw_a[gi] = C(0);
+            adj->dpsi[gi] = psi_slope(rho, psi_c, ph);   // (drw_k and drw_a are read at wall nodes only)
         }
         return;
     }
