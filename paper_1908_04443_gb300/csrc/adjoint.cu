@@ -2,7 +2,8 @@
 //
 // Forward step k (GPU storage): stored post-collision f*_k --pull (Eq. 3, Fig. 3)--> f (post-
 // streaming) --rho, psi, rho_w (Eqs. 4, 6, 16-17), F_m (Eq. 5), collision (Eqs. 2, 7)--> f*_{k+1}.
-// Its adjoint maps mu_{k+1} = dL/df*_{k+1} to mu_k = dL/df*_k and adds dL/dkappa_j, in two kernels:
+// Its adjoint maps mu_{k+1} = dL/df*_{k+1} to mu_k = dL/df*_k and adds dL/dkappa_j, in FP64 in two kernels (in
+// FP32 in one, adjoint_step_fused in step.cu):
 //   A (the forward tile body in its adjoint mode, step.cu): recompute rho, psi and rho_w of the
 //     state pulled from f*_k; per fluid node the reverse of the collision, lambda_loc = dL/df,
 //     Fmbar = dL/dF_m and the node's own psi-bar; psi'(rho), and at wall nodes d rho_w/d kappa and
@@ -12,7 +13,6 @@
 //     lambda = lambda_loc + rho-bar (own psi and wall neighbours' averages) and the transpose of the
 //     pull (a push) into mu_k.
 #include <cmath>
-#include <type_traits>
 
 #include "adjoint.h"
 #include "lattice.cuh"
@@ -34,13 +34,14 @@ __device__ __forceinline__ int wrap_any(int v, int n) {
 
 // psi-bar gathered through Eq. 5, rho-bar / kappa-bar, and the push (transpose of the pull), for a
 // TX x TY tile.  psi-bar(y) = psib(y) + sum_a [x = y - e_a fluid] (-G psi(x) w_a e_a . Fmbar(x)).
-template <class C, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY) adj_gather_push(DevParams p, const C* __restrict__ psi,
-                                                          const C* __restrict__ dpsi, const C* __restrict__ drw_k,
-                                                          const C* __restrict__ drw_a, const C* __restrict__ fmb_x,
-                                                          const C* __restrict__ fmb_y, const C* __restrict__ psib,
-                                                          const C* __restrict__ lam, double* __restrict__ dkappa,
-                                                          C* __restrict__ mu_out) {
+template <int TX, int TY>
+__global__ void __launch_bounds__(TX* TY) adj_gather_push(DevParams p, const double* __restrict__ psi,
+                                                          const double* __restrict__ dpsi, const double* __restrict__ drw_k,
+                                                          const double* __restrict__ drw_a, const double* __restrict__ fmb_x,
+                                                          const double* __restrict__ fmb_y, const double* __restrict__ psib,
+                                                          const double* __restrict__ lam, double* __restrict__ dkappa,
+                                                          double* __restrict__ mu_out) {
+    using C = double;
     constexpr int RX = TX + 4, RY = TY + 4, PX = TX + 2, PY = TY + 2, NT = TX * TY;
     __shared__ uint8_t s_t[RY * RX];
     __shared__ C s_psi[RY * RX], s_fx[RY * RX], s_fy[RY * RX];
@@ -162,9 +163,9 @@ __global__ void __launch_bounds__(256) adj_final_push(DevParams p, const double*
 
 constexpr int GX = 32, GY = 8;
 
-template <class S>
-cudaError_t adjoint_step_t(const void* fstar_k, const void* mu_next, void* mu_prev, const DevParams& p,
+cudaError_t adjoint_step_fp64(const void* fstar_k, const void* mu_next, void* mu_prev, const DevParams& p,
                            const AdjointScratch& w, double* dkappa, cudaStream_t s) {
+    using S = double;
     const size_t N = size_t(p.N);
     S* b = static_cast<S*>(w.buf);
     AdjointFields f;
@@ -177,10 +178,10 @@ cudaError_t adjoint_step_t(const void* fstar_k, const void* mu_next, void* mu_pr
     f.dpsi = b + 13 * N;
     f.drw_k = b + 14 * N;
     f.drw_a = b + 15 * N;
-    cudaError_t e = launch_adjoint_local(std::is_same<S, double>::value ? PREC_FP64 : PREC_FP32, fstar_k, p, f, s);
+    cudaError_t e = launch_adjoint_local(fstar_k, p, f, s);
     if (e != cudaSuccess) return e;
     dim3 grid((p.nx + GX - 1) / GX, (p.ny + GY - 1) / GY, 1);
-    return launch_pdl(adj_gather_push<S, GX, GY>, grid, dim3(GX, GY, 1), 0, s, p, static_cast<const S*>(f.psi),
+    return launch_pdl(adj_gather_push<GX, GY>, grid, dim3(GX, GY, 1), 0, s, p, static_cast<const S*>(f.psi),
                       static_cast<const S*>(f.dpsi), static_cast<const S*>(f.drw_k), static_cast<const S*>(f.drw_a),
                       static_cast<const S*>(f.fmb_x), static_cast<const S*>(f.fmb_y), static_cast<const S*>(f.psib),
                       static_cast<const S*>(f.lam), dkappa, static_cast<S*>(mu_prev));
@@ -194,12 +195,13 @@ unsigned grid_of(long long n) {
 
 }  // namespace
 
-size_t adjoint_scratch_elems(long long N) { return size_t(N) * 16; }
+size_t adjoint_scratch_bytes(int prec, long long N) { return prec == PREC_FP64 ? size_t(N) * 16 * sizeof(double) : 0; }
+int adjoint_step_launches(int prec) { return prec == PREC_FP64 ? 2 : 1; }
 
 cudaError_t launch_adjoint_step(int prec, const void* fstar_k, const void* mu_next, void* mu_prev, const DevParams& p,
                                 const AdjointScratch& w, double* dkappa, cudaStream_t s) {
-    if (prec == PREC_FP64) return adjoint_step_t<double>(fstar_k, mu_next, mu_prev, p, w, dkappa, s);
-    return adjoint_step_t<float>(fstar_k, mu_next, mu_prev, p, w, dkappa, s);
+    if (prec == PREC_FP64) return adjoint_step_fp64(fstar_k, mu_next, mu_prev, p, w, dkappa, s);
+    return launch_adjoint_fused(fstar_k, mu_next, mu_prev, dkappa, p, s);
 }
 
 cudaError_t launch_adjoint_final(int prec, const double* drho_final, void* mu, const DevParams& p, cudaStream_t s) {

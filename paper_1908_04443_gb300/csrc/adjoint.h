@@ -5,22 +5,26 @@
 
 namespace lbmwet {
 
-// Work buffer of the adjoint step: adjoint_scratch_elems(N) values of the storage precision.
+// Work buffer of the adjoint step: adjoint_scratch_bytes(prec, N) bytes (none in FP32).
 struct AdjointScratch {
     void* buf;
 };
-size_t adjoint_scratch_elems(long long N);
+size_t adjoint_scratch_bytes(int prec, long long N);
+int adjoint_step_launches(int prec);
 
-// Node fields of the adjoint step (storage precision; [a][node] for mu and lam, one per node else).
+// Node fields of the FP64 adjoint step ([a][node] for mu and lam, one per node else).
 struct AdjointFields {
     const void* mu;
     void *lam, *fmb_x, *fmb_y, *psib, *psi, *dpsi, *drw_k, *drw_a;
 };
 
-// Local part of an adjoint step (tile kernel sharing the forward's halo machinery): recomputes the
+// Local part of an FP64 adjoint step (tile kernel sharing the forward's halo machinery): recomputes the
 // state pulled from f*_k and writes, per node, the reverse of the collision and psi data.
-cudaError_t launch_adjoint_local(int prec, const void* fstar, const DevParams& p, const AdjointFields& w,
-                                 cudaStream_t s);
+cudaError_t launch_adjoint_local(const void* fstar, const DevParams& p, const AdjointFields& w, cudaStream_t s);
+
+// A whole FP32 adjoint step.
+cudaError_t launch_adjoint_fused(const void* fstar, const void* mu_next, void* mu_prev, double* dkappa,
+                                 const DevParams& p, cudaStream_t s);
 
 // One adjoint step: given the stored forward state f*_k (whose pull is the post-streaming state
 // that step k collides) and mu_next = dL/df*_{k+1}, write mu_prev = dL/df*_k and add the step's

@@ -1930,15 +1930,14 @@ extern "C" lbm_status lbm_adjoint(lbm_handle* h, const double* drho_final_dev, d
     const size_t nw = h->wall_nodes.size();
     const int64_t every = h->rec_every, n = h->rec_steps;
     const int64_t nck = (int64_t)h->ckpt.size();
-    const size_t es = h->prec == LBM_FP64 ? sizeof(double) : sizeof(float);
     // Two segment buffers: slot 0 of a buffer receives a copy of a segment's checkpoint, slots 1.. the
     // recomputed states.  Pass t reverses segment nck - t (recomputed by pass t - 1) on the handle's stream
     // and, on a second stream, recomputes segment nck - 1 - t into the other buffer: the two share no data,
     // so the recomputation hides behind the latency-bound reverse kernels.  Every launch is used once, so
     // they are issued directly, each set up while the one before it ends (launch_pdl): capturing and
     // instantiating graphs of the passes on every call kept the GPU idle in between, the more so with
-    // programmatic edges.  300 steps on 256 x 256, FP32, with 3 checkpoints (forward and adjoint): graphs
-    // 8.6 ms, graphs of programmatic launches 8.7, direct plain launches 8.8, this 6.9.  The buffers come
+    // programmatic edges.  300 steps on 256 x 256, FP32, with 3 checkpoints (forward and adjoint, reverse steps
+    // of two launches): graphs 8.6 ms, graphs of programmatic launches 8.7, direct plain launches 8.8, this 6.9.  The buffers come
     // from the pool, as cudaMalloc and cudaFree of this half a gigabyte wait for the device; more than
     // ADJ_POOL_BYTES go back to the driver after the call, since the pool would keep them.
     constexpr size_t ADJ_POOL_BYTES = size_t(1) << 30;
@@ -1948,7 +1947,7 @@ extern "C" lbm_status lbm_adjoint(lbm_handle* h, const double* drho_final_dev, d
     double* dk = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
     const size_t seg_bytes = h->fbytes * (size_t)every, dk_bytes = sizeof(double) * (nw ? nw : 1);
-    const size_t scratch_bytes = es * adjoint_scratch_elems(h->N);
+    const size_t scratch_bytes = adjoint_scratch_bytes(h->prec, h->N);
     const bool pooled = (nck > 1 ? 2 : 1) * seg_bytes + 2 * h->fbytes + scratch_bytes + dk_bytes <= ADJ_POOL_BYTES;
     auto get = [&](auto** q, size_t bytes) { return pooled ? dmalloc(q, bytes, h->stream) : cudaMalloc(q, bytes); };
     auto put = [&](void* q) {
@@ -1960,7 +1959,7 @@ extern "C" lbm_status lbm_adjoint(lbm_handle* h, const double* drho_final_dev, d
     if (e == cudaSuccess && nck > 1) e = get(&seg[1], seg_bytes);
     if (e == cudaSuccess) e = get(&mu[0], h->fbytes);
     if (e == cudaSuccess) e = get(&mu[1], h->fbytes);
-    if (e == cudaSuccess) e = get(&scratch, scratch_bytes);
+    if (e == cudaSuccess && scratch_bytes) e = get(&scratch, scratch_bytes);
     if (e == cudaSuccess) e = get(&dk, dk_bytes);
     if (e == cudaSuccess) e = cudaMemsetAsync(dk, 0, dk_bytes, h->stream);
     if (e == cudaSuccess && !h->cap_stream) e = cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking);
@@ -1998,7 +1997,7 @@ extern "C" lbm_status lbm_adjoint(lbm_handle* h, const double* drho_final_dev, d
             e = cudaEventRecord(join, side);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, join, 0);
         }
-        h->launches += (rec_len > 0 ? rec_len - 1 : 0) + 2 * rev_len;
+        h->launches += (rec_len > 0 ? rec_len - 1 : 0) + adjoint_step_launches(h->prec) * rev_len;
     }
     if (e == cudaSuccess && nw)
         e = cudaMemcpyAsync(dkappa_host, dk, sizeof(double) * nw, cudaMemcpyDeviceToHost, h->stream);

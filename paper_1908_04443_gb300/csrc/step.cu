@@ -53,6 +53,7 @@ struct AdjIO {
     C* dpsi;          // d psi/d rho at rho or rho_w
     C* drw_k;         // walls: d rho_w / d kappa (0 when the limiter clamps)
     C* drw_a;         // walls: d rho_w / d rho_ave / den
+    C* own;           // MODE 3: the thread's own lam (9), psib and dpsi
 };
 
 // d psi / d rho = (p'(rho) - 1/3) / (G psi), with p' from the equation of state
@@ -75,7 +76,8 @@ __device__ __forceinline__ C psi_slope(C rho, C psi, const Phys<C>& e) {
 }
 
 // One tile: x0, y0, z0 is its first node.  All threads of the CTA call this together.
-// MODE 0: time step (writes f*); 1: fields (writes rho, u); 2: adjoint local part (writes AdjIO).
+// MODE 0: time step (writes f*); 1: fields (writes rho, u); 2: adjoint local part (writes AdjIO); 3: the same
+// for every cell of the tile, inside the grid or a periodic image, with fmb_x and fmb_y per cell of the tile.
 // SOLID = false compiles the body of a tile with no solid node within its box (every cell a bulk
 // fluid node: no node-type staging, no bounce-back, no wall nodes).  WRAP 0 compiles a tile whose
 // pulls touch no cell beyond the grid (no periodic wrapping: neighbours at constant offsets),
@@ -84,8 +86,8 @@ template <class L, class S, class C, int TX, int TY, int TZ, int MODE, bool SOLI
 __device__ __forceinline__ void tile_body(const S* __restrict__ fin, S* __restrict__ fout, const Geo& g,
                                           const Phys<C>& ph, int x0, int y0, int z0, bool tile_solid_arg,
                                           unsigned* err, double* __restrict__ rho_out, double* __restrict__ u_out,
-                                          TileSmem<L, C, TX, TY, TZ, MODE == 2>& sm, const AdjIO<C>* adj = nullptr) {
-    using T = TileSmem<L, C, TX, TY, TZ, MODE == 2>;
+                                          TileSmem<L, C, TX, TY, TZ, MODE >= 2>& sm, const AdjIO<C>* adj = nullptr) {
+    using T = TileSmem<L, C, TX, TY, TZ, MODE >= 2>;
     constexpr int D = L::D, Q = L::Q;
     const bool tile_solid = SOLID && tile_solid_arg;
     constexpr int NT = TX * TY * TZ;
@@ -185,9 +187,9 @@ __device__ __forceinline__ void tile_body(const S* __restrict__ fin, S* __restri
     const int my_ti = tix(lx + 3, ly + 3, lz + YZH);
     const uint8_t my_type = type_at(my_ti);
     const bool my_fluid = !(my_type & T_SOLID);
-    C f[Q], m[MODE == 2 ? Q : 1];
+    C f[Q], m[MODE >= 2 ? Q : 1];
     C my_drho = C(0);
-    if constexpr (MODE == 2) {   // asked for here: the collision waits for it otherwise
+    if constexpr (MODE >= 2) {   // asked for here: the collision waits for it otherwise
 #pragma unroll
         for (int a = 0; a < Q; ++a) m[a] = my_fluid ? adj->mu[a * N + gi] : C(0);
     }
@@ -298,25 +300,25 @@ __device__ __forceinline__ void tile_body(const S* __restrict__ fin, S* __restri
                     const C raw = (kap >= C(0)) ? (C(1) + kap) * rho_ave : rho_ave + kap;
                     rw = raw > ph.rho_l ? ph.rho_l : raw;
                     rw = rw < ph.rho_g ? ph.rho_g : rw;
-                    if constexpr (MODE == 2) {
+                    if constexpr (MODE >= 2) {
                         const bool free = raw < ph.rho_l && raw > ph.rho_g;   // limiter inactive
                         sm.wdk[i] = free ? (kap >= C(0) ? rho_ave : C(1)) : C(0);
                         sm.wda[i] = free ? (kap >= C(0) ? C(1) + kap : C(1)) / den : C(0);
                     }
                 }
             }
-            if constexpr (MODE == 2) {
+            if constexpr (MODE >= 2) {
                 if (ph.wall_kind != 0) sm.wdk[i] = sm.wda[i] = C(0);   // the adjoint covers IVD only
             }
             sm.psi[i] = psi_checked(rw, ph, err);
-            if constexpr (MODE == 2) sm.wdpsi[i] = psi_slope(rw, sm.psi[i], ph);
+            if constexpr (MODE >= 2) sm.wdpsi[i] = psi_slope(rw, sm.psi[i], ph);
         }
         __syncthreads();
     }
 
     // 3. force, velocity and collision of the tile's fluid node
     const bool valid = (x0 + lx < nx) && (y0 + ly < ny) && (D == 2 || z0 + lz < nz);
-    if (!valid) return;
+    if (MODE != 3 && !valid) return;
     const int pc = pix(lx + 1, ly + 1, lz + PZH);
     if (!my_fluid) {
         if (MODE == 1) {
@@ -333,6 +335,13 @@ __device__ __forceinline__ void tile_body(const S* __restrict__ fin, S* __restri
             adj->fmb_x[gi] = C(0);
             adj->fmb_y[gi] = C(0);
             adj->psib[gi] = C(0);
+        }
+        if constexpr (MODE == 3) {
+            adj->fmb_x[tid] = adj->fmb_y[tid] = C(0);
+#pragma unroll
+            for (int a = 0; a < Q; ++a) adj->own[a] = C(0);
+            adj->own[Q] = C(0);
+            adj->own[Q + 1] = (my_type & T_WALL) ? sm.wdpsi[pc] : C(0);
         }
         return;
     }
@@ -394,19 +403,29 @@ __device__ __forceinline__ void tile_body(const S* __restrict__ fin, S* __restri
         }
         return;
     }
-    if constexpr (MODE == 2) {
+    if constexpr (MODE >= 2) {
         if constexpr (D == 2) {
             C fb[Q];
             C bx, by, pb;
             collide_d2q9_adjoint<C>(f, m, rho, ux, uy, Fx, Fy, Fmx, Fmy, psi_c, ph.r, fb, bx, by, pb);
-#pragma unroll
-            for (int a = 0; a < Q; ++a) adj->lam[a * N + gi] = fb[a];
-            adj->fmb_x[gi] = bx;
-            adj->fmb_y[gi] = by;
             // F_m = -G psi(x) sum w psi(x+e) e: its dependence on psi(x) is F_m / psi(x)
-            adj->psib[gi] = pb + (bx * Fmx + by * Fmy) / psi_c;
-            adj->psi[gi] = psi_c;
-            adj->dpsi[gi] = psi_slope(rho, psi_c, ph);   // (drw_k and drw_a are read at wall nodes only)
+            const C own_pb = pb + (bx * Fmx + by * Fmy) / psi_c, slope = psi_slope(rho, psi_c, ph);
+            if constexpr (MODE == 3) {
+                adj->fmb_x[tid] = bx;
+                adj->fmb_y[tid] = by;
+#pragma unroll
+                for (int a = 0; a < Q; ++a) adj->own[a] = fb[a];
+                adj->own[Q] = own_pb;
+                adj->own[Q + 1] = slope;
+            } else {
+#pragma unroll
+                for (int a = 0; a < Q; ++a) adj->lam[a * N + gi] = fb[a];
+                adj->fmb_x[gi] = bx;
+                adj->fmb_y[gi] = by;
+                adj->psib[gi] = own_pb;
+                adj->psi[gi] = psi_c;
+                adj->dpsi[gi] = slope;   // (drw_k and drw_a are read at wall nodes only)
+            }
         }
         return;
     }
@@ -449,7 +468,7 @@ template <class L, class S, class C, int TX, int TY, int TZ, int MODE, bool SOLI
 __device__ __forceinline__ void tile_body_w(const S* __restrict__ fin, S* __restrict__ fout, const Geo& g,
                                             const Phys<C>& ph, int x0, int y0, int z0, bool tile_solid_arg,
                                             unsigned* err, double* __restrict__ rho_out, double* __restrict__ u_out,
-                                            TileSmem<L, C, TX, TY, TZ, MODE == 2>& sm, const AdjIO<C>* adj = nullptr) {
+                                            TileSmem<L, C, TX, TY, TZ, MODE >= 2>& sm, const AdjIO<C>* adj = nullptr) {
     const int w = tile_wrap<L::D, TX, TY, TZ>(x0, y0, z0, g.nx, g.ny, g.nz);
     if (w == 0)
         tile_body<L, S, C, TX, TY, TZ, MODE, SOLID, 0>(fin, fout, g, ph, x0, y0, z0, tile_solid_arg, err, rho_out,
@@ -525,6 +544,76 @@ __global__ void __launch_bounds__(TileShape<D2Q9, S>::X* TileShape<D2Q9, S>::Y, 
     pdl_wait();
     tile_body_w<D2Q9, S, S, TS::X, TS::Y, 1, 2, true>(fin, nullptr, g, ph, blockIdx.x * TS::X, blockIdx.y * TS::Y, 0,
                                                        solid, err, nullptr, nullptr, sm, &io);
+}
+
+// A whole reverse step in one launch (FP32): the local part on 32 x 16 cells, whose inner 28 x 12 are the CTA's
+// own, then, from shared memory, what adj_gather_push does from global memory.  psi-bar of a wall node needs
+// Fmbar of its neighbours, and rho-bar of the wall node's neighbours needs psi-bar: a halo of two nodes, 1.52
+// times the local part.  On the grids the adjoint is used on a reverse step is bound by its chain of memory
+// latencies and by launches, not by arithmetic (256 x 256: 12.2 us in two launches, 9.3 in this one beside the
+// recomputation; 300 steps, forward and adjoint, 6.62 -> 5.61 ms; 32 x 8 cells 6.2, 32 x 24 cells 5.8), and
+// the 16 values a node that the two launches hand over go no more through memory.
+// The FP64 local part is bound by the FP64 pipe and stays in its own kernel, without a halo.
+constexpr int AFX = 32, AFY = 16;
+__global__ void __launch_bounds__(AFX* AFY, 2)
+    adjoint_step_fused(const float* __restrict__ fin, const float* __restrict__ mu, float* __restrict__ mu_out,
+                       double* __restrict__ dkappa, Geo g, Phys<float> ph, unsigned* err) {
+    using L = D2Q9;
+    using T = TileSmem<L, float, AFX, AFY, 1, true>;
+    constexpr int Q = 9, YX = T::YX, PX = T::PX;
+    __shared__ T sm;
+    __shared__ float s_fx[AFX * AFY], s_fy[AFX * AFY], s_wb[AFX * AFY];
+    const int x0 = int(blockIdx.x) * (AFX - 4) - 2, y0 = int(blockIdx.y) * (AFY - 4) - 2;
+    const int lx = threadIdx.x, ly = threadIdx.y, tid = ly * AFX + lx;
+    float own[Q + 2];
+    AdjIO<float> io{};
+    io.mu = mu;
+    io.fmb_x = s_fx;
+    io.fmb_y = s_fy;
+    io.own = own;
+    pdl_wait();
+    tile_body_w<L, float, float, AFX, AFY, 1, 3, true>(fin, nullptr, g, ph, x0, y0, 0, true, err, nullptr, nullptr, sm,
+                                                       &io);
+    __syncthreads();
+    // 1. psi-bar on the own nodes + 1-node halo; fluid -> rho-bar, wall -> kappa-bar and the Eq. 17 weight
+    const int ti = (ly + 3) * YX + lx + 3, pc = (ly + 1) * PX + lx + 1;
+    const uint8_t t = sm.type[ti];
+    const bool fluid = !(t & T_SOLID), wall = !fluid && (t & T_WALL);
+    const bool mine = lx >= 2 && lx < AFX - 2 && ly >= 2 && ly < AFY - 2 && x0 + lx < g.nx && y0 + ly < g.ny;
+    float rb = 0.0f;
+    if (lx >= 1 && lx < AFX - 1 && ly >= 1 && ly < AFY - 1 && (fluid || wall)) {
+        float pb = own[Q];
+#pragma unroll
+        for (int a = 1; a < Q; ++a) {
+            const int ex = L::ex(a), ey = L::ey(a);
+            if (sm.type[ti - ex - ey * YX] & T_SOLID) continue;
+            const int n = tid - ex - ey * AFX;
+            pb += -ph.G * sm.psi[pc - ex - ey * PX] * float(L::wf(a)) * (s_fx[n] * float(ex) + s_fy[n] * float(ey));
+        }
+        rb = pb * own[Q + 1];
+        if (wall) {
+            s_wb[tid] = rb * sm.wda[pc];
+            if (mine && g.kappa_w) dkappa[g.wall_id[(y0 + ly) * g.nx + x0 + lx]] += double(rb * sm.wdk[pc]);
+        }
+    }
+    __syncthreads();
+    // 2. lambda = lam + rho-bar at the own fluid nodes, pushed to mu (the transpose of the pull)
+    if (!mine || !fluid) return;
+#pragma unroll
+    for (int a = 1; a < Q; ++a) {
+        const int ex = L::ex(a), ey = L::ey(a);
+        if (sm.type[ti + ex + ey * YX] & T_WALL) rb += float(L::wf(a)) * s_wb[tid + ex + ey * AFX];
+    }
+    const int gx = x0 + lx, gy = y0 + ly, N = g.N;
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+        const int ex = L::ex(a), ey = L::ey(a);
+        const float l = own[a] + rb;
+        if (sm.type[ti - ex - ey * YX] & T_SOLID)
+            mu_out[L::opp(a) * N + gy * g.nx + gx] = l;
+        else
+            mu_out[a * N + wrap1(gy - ey, g.ny) * g.nx + wrap1(gx - ex, g.nx)] = l;
+    }
 }
 
 // Batched step: CTAs walk the work list; each item is one tile of one instance.  The next item's
@@ -791,10 +880,10 @@ cudaError_t launch_step_batched(int parity, const DevParams& p, const BatchInsta
     return cudaGetLastError();
 }
 
-template <class S>
-static cudaError_t adj_local_t(const void* fstar, const DevParams& p, const AdjointFields& w, cudaStream_t s) {
+cudaError_t launch_adjoint_local(const void* fstar, const DevParams& p, const AdjointFields& w, cudaStream_t s) {
+    using S = double;
     using TS = TileShape<D2Q9, S>;
-    AdjIO<S> io;
+    AdjIO<S> io{};
     io.mu = static_cast<const S*>(w.mu);
     io.lam = static_cast<S*>(w.lam);
     io.fmb_x = static_cast<S*>(w.fmb_x);
@@ -809,9 +898,12 @@ static cudaError_t adj_local_t(const void* fstar, const DevParams& p, const Adjo
                       make_phys<S>(p), p.err, io);
 }
 
-cudaError_t launch_adjoint_local(int prec, const void* fstar, const DevParams& p, const AdjointFields& w,
-                                 cudaStream_t s) {
-    return prec == PREC_FP64 ? adj_local_t<double>(fstar, p, w, s) : adj_local_t<float>(fstar, p, w, s);
+cudaError_t launch_adjoint_fused(const void* fstar, const void* mu_next, void* mu_prev, double* dkappa,
+                                 const DevParams& p, cudaStream_t s) {
+    dim3 grid((p.nx + AFX - 5) / (AFX - 4), (p.ny + AFY - 5) / (AFY - 4), 1);
+    return launch_pdl(adjoint_step_fused, grid, dim3(AFX, AFY, 1), 0, s, static_cast<const float*>(fstar),
+                      static_cast<const float*>(mu_next), static_cast<float*>(mu_prev), dkappa, geo_of(p),
+                      make_phys<float>(p), p.err);
 }
 
 void step_tile_shape(int lat, int prec, int* tx, int* ty, int* tz) {

@@ -1111,7 +1111,7 @@ __host__ __device__ __forceinline__ bool ztma_boxed(int x0, int y0, int nx, int 
 // the grid, as far as the boxes' 16-byte boundary allows: up to 3 of its columns then lie beyond x = nx - 1
 // and hold periodic images, patched like the halo.  It writes only the nodes that no full column owns.  (Such
 // columns went to the z-pair march on narrow blocks before: the 200 x 200 x 280 grid, one column in seven,
-// took 561 us a step, 455 us now.)
+// took 561 us a step, 406 us now.)
 template <int MODE>
 __global__ void __launch_bounds__(TNT, 2)
     ztma_step(const float* __restrict__ fin, float* __restrict__ fout, const void* tmap, Geo g, Phys<float> ph,
