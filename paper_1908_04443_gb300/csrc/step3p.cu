@@ -551,6 +551,7 @@ struct ZTSmem {
         ZTBulk b;
         ZTSolid s;
     };
+    int4 box[19];   // per direction: offset in the stage (bytes) + 4 * tensor map + ez + 1, x, y, a * nz
     uint64_t bar[BST];
 };
 constexpr size_t ZT_SMEM = sizeof(ZTSmem);
@@ -585,6 +586,19 @@ __device__ __forceinline__ int ez_rt(int a) {
     constexpr unsigned PLUS = (1u << 5) | (1u << 11) | (1u << 14) | (1u << 15) | (1u << 18);
     constexpr unsigned MINUS = (1u << 6) | (1u << 12) | (1u << 13) | (1u << 16) | (1u << 17);
     return int((PLUS >> a) & 1u) - int((MINUS >> a) & 1u);
+}
+
+// Lane 0 of warp `warp` issues its share of the 19 boxes of plane zl (from a table in shared memory: working the
+// boxes out cost each warp a hundred instructions a plane).
+__device__ __forceinline__ void issue_boxes(float* stage, unsigned bytes, const int4* box, const void* tmap, int zl, int nz,
+                                            int warp, uint64_t* bar) {
+    fence_proxy_async();
+    if (warp == 0) mbar_expect_tx(bar, bytes);
+    for (int a = warp; a < 19; a += TTY) {
+        const int4 b = box[a];
+        tma_box3(reinterpret_cast<char*>(stage) + (b.x & ~127), static_cast<const char*>(tmap) + 128 * ((b.x >> 2) & 3), b.y,
+                 b.z, b.w + wrap1(zl + 1 - (b.x & 3), nz), bar);
+    }
 }
 
 // Out-of-range part of a box's used window (rows [rw0, rw1), columns [cw0, cw1) of a box whose
@@ -648,7 +662,8 @@ template <int MODE>
 __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, float* __restrict__ fout,
                                                 const void* tmap, const Geo& g, const Phys<float>& ph,
                                                 const Rates3P& kr, int x0, int y0, int xs, int ys, int zb, int ze,
-                                                unsigned* err, ZTBulk& S, uint64_t* bar, const ZTOut& out) {
+                                                unsigned* err, ZTBulk& S, const int4* box, uint64_t* bar,
+                                                const ZTOut& out) {
     using L = D3Q19;
     constexpr int Q = 19;
     const int nx = g.nx, ny = g.ny, nz = g.nz, fp = g.fp, fxy = fp * ny;   // (fp: row pitch of the distributions)
@@ -670,15 +685,7 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
     float fix[Q];
     // lane 0 of every warp: its share of the 19 boxes of lead plane zl into stage s (one thread issuing them
     // all held its warp, and the barrier behind it, for 19 instructions)
-    auto issue = [&](int zl, int s) {
-        fence_proxy_async();
-        if (ly == 0) mbar_expect_tx(&bar[s], BULK_BYTES);
-        for (int a = ly; a < Q; a += TTY) {
-            const int ex = ex_rt(a);
-            tma_box3(S.stage[s] + bslot(a), static_cast<const char*>(tmap) + (ex ? 128 : 0), x0 - box_lead(ex),
-                     y0 - 1 - ey_rt(a), a * nz + wrap1(zl - ez_rt(a), nz), &bar[s]);
-        }
-    };
+    auto issue = [&](int zl, int s) { issue_boxes(S.stage[s], BULK_BYTES, box, tmap, zl, nz, ly, &bar[s]); };
 
     if (lx == 0) {
         for (int k = 0; k < BST && zlo + k <= zhi; ++k) issue(zlo + k, k);
@@ -704,7 +711,7 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
         return st[bslot(a) + py * box_cols(L::ex(a)) + px - 1 - L::ex(a) + box_lead(L::ex(a))];
     };
 
-    V1 fprev[Q];
+    V1 fprev[Q], dprev = {0.0f};   // own values of plane zl - 1 and their sum
 #pragma unroll
     for (int a = 0; a < Q; ++a) fprev[a].v = 0.0f;
 
@@ -737,12 +744,10 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
         V1 fcur[Q];
 #pragma unroll
         for (int a = 0; a < Q; ++a) fcur[a].v = pulled(st, a, lx + 1, ly + 1);
-        {
-            V1 d = fcur[0];
+        V1 dcur = fcur[0];
 #pragma unroll
-            for (int a = 1; a < Q; ++a) d = d + fcur[a];
-            S.psi[zl & 3][pc] = psi1(V1{ph.rho_ref} + d, ph, err).v;
-        }
+        for (int a = 1; a < Q; ++a) dcur = dcur + fcur[a];
+        S.psi[zl & 3][pc] = psi1(V1{ph.rho_ref} + dcur, ph, err).v;
         if (ringer) {
             V1 d = {pulled(st, 0, rx, ry)};
 #pragma unroll
@@ -779,9 +784,7 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
             const V1 gpsi = (-ph.G) * psi_c;
             const V1 Fmx = gpsi * sx, Fmy = gpsi * sy, Fmz = gpsi * sz;
             const V1 Fx = Fmx + V1{ph.fx}, Fy = Fmy + V1{ph.fy}, Fz = Fmz + V1{ph.fz};
-            V1 drho = f[0];
-#pragma unroll
-            for (int a = 1; a < Q; ++a) drho = drho + f[a];
+            const V1 drho = dprev;
             const V1 jx = ((f[1] - f[2]) + (f[7] - f[8])) + ((f[9] - f[10]) + (f[11] - f[12])) + (f[13] - f[14]);
             const V1 jy = ((f[3] - f[4]) + (f[7] - f[8])) + ((f[10] - f[9]) + (f[15] - f[16])) + (f[17] - f[18]);
             const V1 jz = ((f[5] - f[6]) + (f[11] - f[12])) + ((f[14] - f[13]) + (f[15] - f[16])) + (f[18] - f[17]);
@@ -795,15 +798,16 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
             } else {
                 const V1 X = div2(fma2(Fmx, Fmx, fma2(Fmy, Fmy, Fmz * Fmz)), psi_c * psi_c);
                 collide3p(f, drho, rho, ux, uy, uz, Fx, Fy, Fz, X, kr);
-                float* o = fout + (long long)zc * fxy + (y0 + ly) * fp + x0 + lx;
+                const unsigned o = unsigned(zc * fxy + (y0 + ly) * fp + x0 + lx);
                 if (wr) {
 #pragma unroll
-                    for (int a = 0; a < Q; ++a) o[a * fs] = f[a].v;
+                    for (int a = 0; a < Q; ++a) (fout + a * fs)[o] = f[a].v;
                 }
             }
         }
 #pragma unroll
         for (int a = 0; a < Q; ++a) fprev[a] = fcur[a];
+        dprev = dcur;
     }
 }
 
@@ -814,7 +818,8 @@ template <bool SF, int MODE>
 __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, float* __restrict__ fout,
                                                  const void* tmap, const Geo& g, const Phys<float>& ph,
                                                  const Rates3P& kr, int x0, int y0, int xs, int ys, int zb, int ze,
-                                                 unsigned* err, ZTSolid& S, uint64_t* bar, const ZTOut& out) {
+                                                 unsigned* err, ZTSolid& S, const int4* box, uint64_t* bar,
+                                                 const ZTOut& out) {
     using L = D3Q19;
     constexpr int Q = 19, NT = TNT;
     const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny, fp = g.fp, fxy = fp * ny;
@@ -839,13 +844,7 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
         band.cell(tid, 1, fr, fcl);
         fsrc = fin + (long long)wrap1(y0 - 3 + fr, ny) * fp + wrap1(x0 - 4 + fcl, nx);
     }
-    auto issue = [&](int zl, int s) {   // lane 0 of every warp, as in bulk
-        fence_proxy_async();
-        if (ly == 0) mbar_expect_tx(&bar[s], SOLID_BYTES);
-        for (int a = ly; a < Q; a += TTY)
-            tma_box3(S.stage[s] + a * SSLOT, static_cast<const char*>(tmap) + 256, x0 - 4, y0 - 2 - ey_rt(a),
-                     a * nz + wz(zl - ez_rt(a)), &bar[s]);
-    };
+    auto issue = [&](int zl, int s) { issue_boxes(S.stage[s], SOLID_BYTES, box, tmap, zl, nz, ly, &bar[s]); };
     if (lx == 0) {
         issue(zlo, 0);
         issue(zlo + 1, 1);
@@ -885,7 +884,7 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
     const int pc = (ly + 1) * TPX + lx + 1;   // own cell in the psi window
     const int rc = (ly + 2) * TRX + lx + 2;   // own cell in the density window
     const int tcl = (ly + 3) * TYX + lx + 3;  // own cell in the type window
-    V1 f1[Q], f2[Q];                          // own values of planes zl - 1 and zl - 2
+    V1 f1[Q], f2[Q], d1 = {0.0f}, d2 = {0.0f};   // own values of planes zl - 1 and zl - 2, and their sums
 #pragma unroll
     for (int a = 0; a < Q; ++a) f1[a].v = f2[a].v = 0.0f;
     constexpr int TN = (TTYPES + NT - 1) / NT;
@@ -929,7 +928,7 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
         const uint8_t* ty = S.type[zl & 7];
         float* rr = S.rho[zl & 3];
         float* pp = S.psi[ps5(zl)];
-        V1 fcur[Q];
+        V1 fcur[Q], dcur = {0.0f};
         {
             float v[Q];
             const uint8_t t = ty[tcl];
@@ -937,10 +936,10 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
             V1 rho = {0.0f}, ps = {0.0f};
             if (fl) {
                 pull(st, stn, zl, ly + 2, lx + 4, t, v);
-                V1 d = {v[0]};
+                dcur = V1{v[0]};
 #pragma unroll
-                for (int a = 1; a < Q; ++a) d = d + V1{v[a]};
-                rho = V1{ph.rho_ref} + d;
+                for (int a = 1; a < Q; ++a) dcur = dcur + V1{v[a]};
+                rho = V1{ph.rho_ref} + dcur;
                 ps = psi1(rho, ph, err);
             } else {
 #pragma unroll
@@ -1052,9 +1051,7 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
                 const V1 gpsi = (-ph.G) * psi_c;
                 const V1 Fmx = gpsi * sx, Fmy = gpsi * sy, Fmz = gpsi * sz;
                 V1 Fx = Fmx + V1{ph.fx}, Fy = Fmy + V1{ph.fy}, Fz = Fmz + V1{ph.fz};
-                V1 drho = f[0];
-#pragma unroll
-                for (int a = 1; a < Q; ++a) drho = drho + f[a];
+                const V1 drho = d2;
                 const V1 jx = ((f[1] - f[2]) + (f[7] - f[8])) + ((f[9] - f[10]) + (f[11] - f[12])) + (f[13] - f[14]);
                 const V1 jy = ((f[3] - f[4]) + (f[7] - f[8])) + ((f[10] - f[9]) + (f[15] - f[16])) + (f[17] - f[18]);
                 const V1 jz = ((f[5] - f[6]) + (f[11] - f[12])) + ((f[14] - f[13]) + (f[15] - f[16])) + (f[18] - f[17]);
@@ -1086,10 +1083,10 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
                 } else {
                     const V1 X = div2(fma2(Fmx, Fmx, fma2(Fmy, Fmy, Fmz * Fmz)), psi_c * psi_c);
                     collide3p(f, drho, rho, ux, uy, uz, Fx, Fy, Fz, X, kr);
-                    const long long gi = (long long)zc * fxy + (y0 + ly) * fp + x0 + lx;
+                    const unsigned o = unsigned(zc * fxy + (y0 + ly) * fp + x0 + lx);
                     if (in) {
 #pragma unroll
-                        for (int a = 0; a < Q; ++a) fout[a * fs + gi] = f[a].v;
+                        for (int a = 0; a < Q; ++a) (fout + a * fs)[o] = f[a].v;
                     }
                 }
             }
@@ -1099,6 +1096,8 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
             f2[a] = f1[a];
             f1[a] = fcur[a];
         }
+        d2 = d1;
+        d1 = dcur;
     }
 }
 
@@ -1107,11 +1106,15 @@ __host__ __device__ __forceinline__ bool ztma_boxed(int x0, int y0, int nx, int 
     return x0 + TTX <= nx && y0 + TTY <= ny && nx >= 64 && ny >= 16 && nz >= 4;
 }
 
+// Bound by the instructions of a plane (256^3: issue slots 69 % busy at 26 warp instructions a node, DRAM at 79 %
+// of the copy rate): a table of the boxes in shared memory, the density's sum carried to the collision, and stores at a uniform
+// base plus one 32-bit offset took 256^3 from 541 to 502 us a step, 200 x 200 x 280 from 406 to 383, 97 x 83 x 75 from
+// 55.6 to 52.0.
 // One CTA per item.  The last column of a grid whose width is not a multiple of 32 (8 in y) is moved inside
 // the grid, as far as the boxes' 16-byte boundary allows: up to 3 of its columns then lie beyond x = nx - 1
 // and hold periodic images, patched like the halo.  It writes only the nodes that no full column owns.  (Such
 // columns went to the z-pair march on narrow blocks before: the 200 x 200 x 280 grid, one column in seven,
-// took 561 us a step, 406 us now.)
+// took 561 us a step, 383 us now.)
 template <int MODE>
 __global__ void __launch_bounds__(TNT, 2)
     ztma_step(const float* __restrict__ fin, float* __restrict__ fout, const void* tmap, Geo g, Phys<float> ph,
@@ -1125,15 +1128,20 @@ __global__ void __launch_bounds__(TNT, 2)
         for (int k = 0; k < BST; ++k) mbar_init(&S.bar[k]);
         fence_mbar_init();
     }
+    for (int a = threadIdx.y * TTX + threadIdx.x; a < 19; a += TNT) {
+        const int ex = ex_rt(a), ey = ey_rt(a), ez = ez_rt(a);
+        const int at = it.solid ? a * SSLOT * 4 + 4 * 2 : bslot(a) * 4 + 4 * (ex ? 1 : 0);
+        S.box[a] = make_int4(at + ez + 1, it.solid ? x0 - 4 : x0 - box_lead(ex), (it.solid ? y0 - 2 : y0 - 1) - ey, a * g.nz);
+    }
     pdl_wait();
     __syncthreads();
     // tmap: the input buffer's maps
     if (!it.solid)
-        ztma_chunk_bulk<MODE>(fin, fout, tmap, g, ph, kr, x0, y0, xs, ys, zb, ze, err, S.b, S.bar, out);
+        ztma_chunk_bulk<MODE>(fin, fout, tmap, g, ph, kr, x0, y0, xs, ys, zb, ze, err, S.b, S.box, S.bar, out);
     else if (ph.wall_kind == 2)
-        ztma_chunk_solid<true, MODE>(fin, fout, tmap, g, ph, kr, x0, y0, xs, ys, zb, ze, err, S.s, S.bar, out);
+        ztma_chunk_solid<true, MODE>(fin, fout, tmap, g, ph, kr, x0, y0, xs, ys, zb, ze, err, S.s, S.box, S.bar, out);
     else
-        ztma_chunk_solid<false, MODE>(fin, fout, tmap, g, ph, kr, x0, y0, xs, ys, zb, ze, err, S.s, S.bar, out);
+        ztma_chunk_solid<false, MODE>(fin, fout, tmap, g, ph, kr, x0, y0, xs, ys, zb, ze, err, S.s, S.box, S.bar, out);
 }
 
 }  // namespace
@@ -1289,7 +1297,7 @@ std::vector<ZItem> ztma_items(const uint8_t* mask, int nx, int ny, int nz, int s
         column_runs(mask, nx, ny, nz, large ? LBMWET_ZWL_MIN_RUN : 4, [](int, int) { return true; }, &none);
     if (large) {
         // the last layer of bulk pieces in quarters, so that the launch ends on short items (256^3: 561 us a
-        // step with whole ones, 547 with halves, 542 with quarters)
+        // step with whole ones, 547 with halves, 542 with quarters, before the plane's instructions were cut)
         std::vector<ZItem> items;
         const std::vector<ZItem> whole = aligned_items(runs, none);
         const int zt = (nz - 1) / TCH * TCH;
