@@ -45,19 +45,18 @@ UNIT = "MLUPS"
 # of the kernel code: when the code changes the figure is stale and reported as null.
 NCU_TRAFFIC = {
     # pair_step_batched, 600 x 400 sweep of 24 grids: dram__bytes_read.sum + dram__bytes_write.sum of
-    # one launch (214.32 + 159.71 MB as ncu prints them)
-    ("c2", "fp32", "96c84a23e00f20c2"): 374030000,
+    # one launch (215.38 + 153.15 MB as ncu prints them)
+    ("c2", "fp32", "054e40c8e439c43c"): 368530000,
     # ztma_step, 256^3 sphere: one launch (1.59 + 1.22 GB as ncu prints them)
     ("c3", "fp32", "0cdbad1c831bf63f"): 2810000000,
 }
 
 
-# FP64 floating-point operations per node update of the FP64 batched tile kernel
-# (fused_step_batched<D2Q9, double>) on the 600 x 400 sweep, from ncu: (2 x DFMA + DADD + DMUL thread
-# instructions of one launch) / nodes = (2 x 478,996,920 + 503,049,168 + 231,630,840) / 5,760,000;
-# keyed by a hash of the tile kernel's code.
+# FP64 floating-point operations per node update of the FP64 batched kernel (step64_batched) on the
+# 600 x 400 sweep, from ncu: (2 x DFMA + DADD + DMUL thread instructions of one launch) / nodes =
+# (2 x 210,531,267 + 358,584,387 + 163,519,771) / 5,760,000; keyed by a hash of the kernel's code.
 FP64_FLOPS_PER_NODE = {
-    ("c2", "f7839bf8d649589f"): 293.87,
+    ("c2", "1f132e5983c80437"): 163.75,
 }
 # FP64 peak of a GB300 from its unit counts and clock: 1.25 TFLOP/s nominal is 4 FP64 flops (2 FMA) per
 # SM per clock at 2.07 GHz, so 152 SMs x 4 x 2.07 GHz = 1258.6 GFLOP/s.
@@ -80,8 +79,8 @@ def _code_hash(files) -> str:
     return h.hexdigest()[:16]
 
 
-def tile_kernel_hash() -> str:
-    return _code_hash(("step.cu", "tile_common.cuh", "lattice.cuh", "kernels.h"))   # the tile kernel's sources
+def fp64_kernel_hash() -> str:
+    return _code_hash(("step64.cu", "fp64.cuh", "tile_common.cuh", "lattice.cuh", "kernels.h"))   # the FP64 2D kernel's
 
 
 def kernel_hash() -> str:
@@ -361,6 +360,7 @@ class Runner:
         self.L = L
         self.batch = len(cfgs) > 1
         self.lattice3 = cfgs[0].lattice == 1
+        self.fp64 = cfgs[0].precision == L.LBM_FP64
         if self.batch:
             self.b = L.lbm_batch_init(cfgs, masks, rho0s, None, stream)
             self.handles = [L.lbm_batch_handle(self.b, i) for i in range(len(cfgs))]
@@ -390,12 +390,14 @@ class Runner:
         if k == "ztma":
             return "ztma_step"
         if self.lattice3:
-            return "zpair_step" if k == "pair" else "zmarch_step"
+            return "step3d64" if self.fp64 else "zpair_step" if k == "pair" else "zmarch_step"
         if k == "ymarch":
             return "ymarch_step"
         if k == "pair":
             return "pair_step_batched" if self.batch else "pair_step"
         if k == "tile":
+            if self.fp64:
+                return "step64_batched" if self.batch else "step64"
             return "fused_step_batched" if self.batch else "fused_step"
         return "zmarch_step"
 
@@ -815,7 +817,7 @@ def device_rate(L, torch, stream, name, steps, flush, precision=None, extras=Non
     out.update(more)
     if precision == "fp64":
         # GB300's FP64 rate is far below its FP32 rate: the FP64 step is bound by the FP64 pipe
-        fpn = FP64_FLOPS_PER_NODE.get((name, tile_kernel_hash()))
+        fpn = FP64_FLOPS_PER_NODE.get((name, fp64_kernel_hash()))
         fp64_peak = L.lbm_probe_fp64_rate(stream)
         out["bound"] = "alu"
         out["alu_roofline"] = {
