@@ -47,16 +47,16 @@ NCU_TRAFFIC = {
     # pair_step_batched, 600 x 400 sweep of 24 grids: dram__bytes_read.sum + dram__bytes_write.sum of
     # one launch (215.38 + 153.15 MB as ncu prints them)
     ("c2", "fp32", "054e40c8e439c43c"): 368530000,
-    # ztma_step, 256^3 sphere: one launch (1.59 + 1.22 GB as ncu prints them)
-    ("c3", "fp32", "0cdbad1c831bf63f"): 2810000000,
+    # ztma_step, 256^3 sphere: one launch
+    ("c3", "fp32", "1645287eb60ebe95"): 2811863552,
 }
 
 
 # FP64 floating-point operations per node update of the FP64 batched kernel (step64_batched) on the
 # 600 x 400 sweep, from ncu: (2 x DFMA + DADD + DMUL thread instructions of one launch) / nodes =
-# (2 x 210,531,267 + 358,584,387 + 163,519,771) / 5,760,000; keyed by a hash of the kernel's code.
+# (2 x 217,849,056 + 371,237,280 + 169,225,560) / 5,760,000; keyed by a hash of the kernel's code.
 FP64_FLOPS_PER_NODE = {
-    ("c2", "1f132e5983c80437"): 163.75,
+    ("c2", "1f132e5983c80437"): 169.47,
 }
 # FP64 peak of a GB300 from its unit counts and clock: 1.25 TFLOP/s nominal is 4 FP64 flops (2 FMA) per
 # SM per clock at 2.07 GHz, so 152 SMs x 4 x 2.07 GHz = 1258.6 GFLOP/s.
