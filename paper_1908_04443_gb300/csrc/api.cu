@@ -20,6 +20,7 @@
 #include "eos_host.h"
 #include "kernels.h"
 #include "lattice.cuh"
+#include "layout.h"
 #include "maskscan.h"
 #include "reduce.h"
 #include "plan.h"
@@ -617,13 +618,10 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
     }
 
     const size_t ssize = c.precision == LBM_FP64 ? sizeof(double) : sizeof(float);
-    // distributions: 2D rows padded to a multiple of 32 nodes (128-byte rows in FP32: TMA needs
-    // 16-byte row strides, and a row that starts a cache line keeps a warp's 32 consecutive nodes in
-    // one line); 3D FP32 rows to a multiple of 4 nodes, so that every width has tensor maps
-    const int pad = h->D == 2 ? 32 : (c.precision == LBM_FP32_DEV ? 4 : 1);
-    const int fpitch = (nx + pad - 1) / pad * pad;
-    const long long fstride = (long long)fpitch * ny * nz;
-    h->fbytes = ssize * h->Q * (size_t)fstride;
+    const int step3 = c.step_kernel == LBM_KERNEL_PAIR ? 1 : (c.step_kernel == LBM_KERNEL_TILE ? 2 : 0);
+    const bool zmarch = h->D == 3 && c.precision == LBM_FP32_DEV && step3 == 0 && ztma_marches(nx, ny, nz);
+    int fpitch = 0;
+    long long fstride = 0;
     auto oom = [&](cudaError_t e, const char* what) {
         std::string m = std::string(what) + ": " + cudaGetErrorString(e);
         free_all(h);
@@ -633,8 +631,34 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
     cudaError_t e;
 #define CKI(call, what) \
     if ((e = (call)) != cudaSuccess) return oom(e, what)
-    CKI(guarded_malloc(&h->f[0], h->fbytes, h->stream), "cudaMalloc f");
-    CKI(guarded_malloc(&h->f[1], h->fbytes, h->stream), "cudaMalloc f");
+    auto alloc_f = [&](int pitch) {
+        fpitch = pitch;
+        fstride = (long long)pitch * ny * nz;
+        h->fbytes = ssize * h->Q * (size_t)fstride;
+        const cudaError_t e0 = guarded_malloc(&h->f[0], h->fbytes, h->stream);
+        return e0 == cudaSuccess ? guarded_malloc(&h->f[1], h->fbytes, h->stream) : e0;
+    };
+    CKI(alloc_f(row_pitch(h->D, zmarch, nx)), "cudaMalloc f");
+    // tensor maps of the TMA-staged z-march; without them the grid steps by the z-pair march
+    std::vector<CUtensorMap> zmaps;
+    if (zmarch) {
+        int bx, by;
+        const int nmaps = ztma_maps(0, &bx, &by);
+        zmaps.resize(2 * nmaps);
+        for (int k = 0; k < 2 * nmaps; ++k) {
+            ztma_maps(k % nmaps, &bx, &by);
+            if (encode_z_map(&zmaps[k], h->f[k / nmaps], nx, ny, nz, fpitch, bx, by)) continue;
+            zmaps.clear();
+            break;
+        }
+        if (zmaps.empty() && fpitch != nx) {   // (whose rows are not padded, see row_pitch)
+            for (void*& f : h->f) {
+                guarded_free(f, h->stream);
+                f = nullptr;
+            }
+            CKI(alloc_f(row_pitch(h->D, false, nx)), "cudaMalloc f");
+        }
+    }
     CKI(dmalloc(&h->d_type, N, h->stream), "cudaMalloc type");
     // (FP64: followed by the flags of the grid's FP64 tiles)
     std::vector<uint8_t> flags = h->tile_solid;
@@ -748,31 +772,21 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
     if (fw > 0) p.pair_solid = h->d_tile_solid + h->tile_solid.size();
     p.err = h->d_err;
     // D3Q19 FP32 step kernel and the tensor maps of the TMA-staged z-march
-    p.step3 = c.step_kernel == LBM_KERNEL_PAIR ? 1 : (c.step_kernel == LBM_KERNEL_TILE ? 2 : 0);
+    p.step3 = step3;
     p.ztmap = nullptr;
     p.zf0 = h->f[0];
-    if (h->D == 3 && c.precision == LBM_FP32_DEV && p.step3 == 0 && ztma_marches(nx, ny, nz)) {
-        int bx, by;
-        const int nmaps = ztma_maps(0, &bx, &by);
-        std::vector<CUtensorMap> maps(2 * nmaps);
-        bool ok = true;
-        for (int k = 0; k < 2 * nmaps; ++k) {
-            ztma_maps(k % nmaps, &bx, &by);
-            ok = ok && encode_z_map(&maps[k], h->f[k / nmaps], nx, ny, nz, fpitch, bx, by);
-        }
-        if (ok) {
-            CKI(dmalloc(&h->d_zmaps, sizeof(CUtensorMap) * maps.size(), h->stream), "cudaMalloc tensor maps");
-            // (from pageable memory: staged before the call returns, so `maps` may go out of scope)
-            CKI(cudaMemcpyAsync(h->d_zmaps, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice,
-                                h->stream), "copy tensor maps");
-            const std::vector<ZItem> items = ztma_items(solid_mask, nx, ny, nz, 2 * device_sms());   // (2 CTAs per SM)
-            CKI(dmalloc(&h->d_zitems, sizeof(ZItem) * items.size(), h->stream), "cudaMalloc work list");
-            CKI(cudaMemcpyAsync(h->d_zitems, items.data(), sizeof(ZItem) * items.size(), cudaMemcpyHostToDevice,
-                                h->stream), "copy work list");
-            p.zitems = h->d_zitems;
-            p.nzitems = int(items.size());
-            p.ztmap = h->d_zmaps;
-        }
+    if (!zmaps.empty()) {
+        CKI(dmalloc(&h->d_zmaps, sizeof(CUtensorMap) * zmaps.size(), h->stream), "cudaMalloc tensor maps");
+        // (from pageable memory: staged before the call returns, so `zmaps` may go out of scope)
+        CKI(cudaMemcpyAsync(h->d_zmaps, zmaps.data(), sizeof(CUtensorMap) * zmaps.size(), cudaMemcpyHostToDevice,
+                            h->stream), "copy tensor maps");
+        const std::vector<ZItem> items = ztma_items(solid_mask, nx, ny, nz, 2 * device_sms());   // (2 CTAs per SM)
+        CKI(dmalloc(&h->d_zitems, sizeof(ZItem) * items.size(), h->stream), "cudaMalloc work list");
+        CKI(cudaMemcpyAsync(h->d_zitems, items.data(), sizeof(ZItem) * items.size(), cudaMemcpyHostToDevice,
+                            h->stream), "copy work list");
+        p.zitems = h->d_zitems;
+        p.nzitems = int(items.size());
+        p.ztmap = h->d_zmaps;
     }
 
     // initial state f = f^eq(rho0, u0), stored so that the first pull yields it

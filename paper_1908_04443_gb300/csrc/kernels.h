@@ -190,7 +190,6 @@ std::vector<ZItem> ztma_work_list(const uint8_t* mask, int nx, int ny, int nz);
 // inside the grid), and shorter pieces where the grid would not fill the chip.  Only for grids that the march
 // covers (ztma_marches).
 std::vector<ZItem> ztma_items(const uint8_t* mask, int nx, int ny, int nz, int slots);
-bool ztma_marches(int nx, int ny, int nz);
 // The fields pass on the same items.
 cudaError_t launch_ztma_fields(const void* fin, const void* tmap, const Geo& g, const DevParams& p, double* rho,
                                double* u, cudaStream_t s);

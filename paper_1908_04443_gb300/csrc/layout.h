@@ -1,0 +1,20 @@
+// Layout of the distribution buffers f[a][z][y][x] (host rules; no device code).
+#pragma once
+
+namespace lbmwet {
+
+// Grids that the TMA-staged z-march takes: the window of a box (36 columns and 14 rows with the rows beyond
+// it) leaves the grid on one side at most, also where the last column is moved inside.
+inline bool ztma_marches(int nx, int ny, int nz) { return nx >= 40 && ny >= 16 && nz >= 4; }
+
+// Nodes per stored row.  2D: a multiple of 32 (128-byte rows in FP32: TMA needs 16-byte row strides, and a row
+// that starts a cache line keeps a warp's 32 consecutive nodes in one line).  3D: a multiple of 4 where the
+// z-march runs (`zmarch`), so that every width has tensor maps; its direction offsets are 64-bit.  The other
+// D3Q19 kernels form a * stride + node in 32 bits, which the limit on the nodes (2^31 / 19) covers only as long
+// as the rows are not padded.
+inline int row_pitch(int dim, bool zmarch, int nx) {
+    const int pad = dim == 2 ? 32 : (zmarch ? 4 : 1);
+    return (nx + pad - 1) / pad * pad;
+}
+
+}  // namespace lbmwet

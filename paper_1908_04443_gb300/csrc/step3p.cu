@@ -1285,10 +1285,6 @@ std::vector<ZItem> ztma_work_list(const uint8_t* mask, int nx, int ny, int nz) {
     return aligned_items(runs, chunks);
 }
 
-// The window of a box (36 columns and 14 rows with the rows beyond it) leaves the grid on one side at most,
-// also where the last column is moved inside.
-bool ztma_marches(int nx, int ny, int nz) { return nx >= 40 && ny >= 16 && nz >= 4; }
-
 std::vector<ZItem> ztma_items(const uint8_t* mask, int nx, int ny, int nz, int slots) {
     const long long columns = (long long)((nx + TTX - 1) / TTX) * ((ny + TTY - 1) / TTY);
     const bool large = columns * ((nz + TCH - 1) / TCH) >= 2LL * slots;
