@@ -638,7 +638,7 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
         const cudaError_t e0 = guarded_malloc(&h->f[0], h->fbytes, h->stream);
         return e0 == cudaSuccess ? guarded_malloc(&h->f[1], h->fbytes, h->stream) : e0;
     };
-    CKI(alloc_f(row_pitch(h->D, zmarch, nx)), "cudaMalloc f");
+    CKI(alloc_f(row_pitch(h->D, zmarch, nx, ny)), "cudaMalloc f");
     // tensor maps of the TMA-staged z-march; without them the grid steps by the z-pair march
     std::vector<CUtensorMap> zmaps;
     if (zmarch) {
@@ -656,7 +656,7 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
                 guarded_free(f, h->stream);
                 f = nullptr;
             }
-            CKI(alloc_f(row_pitch(h->D, false, nx)), "cudaMalloc f");
+            CKI(alloc_f(row_pitch(h->D, false, nx, ny)), "cudaMalloc f");
         }
     }
     CKI(dmalloc(&h->d_type, N, h->stream), "cudaMalloc type");

@@ -10,11 +10,12 @@ inline bool ztma_marches(int nx, int ny, int nz) { return nx >= 40 && ny >= 16 &
 // Nodes per stored row.  2D: a multiple of 32 (128-byte rows in FP32: TMA needs 16-byte row strides, and a row
 // that starts a cache line keeps a warp's 32 consecutive nodes in one line).  3D: a multiple of 4 where the
 // z-march runs (`zmarch`), so that every width has tensor maps; its direction offsets are 64-bit.  The other
-// D3Q19 kernels form a * stride + node in 32 bits, which the limit on the nodes (2^31 / 19) covers only as long
-// as the rows are not padded.
-inline int row_pitch(int dim, bool zmarch, int nx) {
-    const int pad = dim == 2 ? 32 : (zmarch ? 4 : 1);
-    return (nx + pad - 1) / pad * pad;
+// kernels form a * stride + node in 32 bits, which the limit on the nodes (2^31 / 19) covers only as long as the
+// rows are not padded: 3D rows are not, nor are those of 2D grids so narrow and tall (15 columns or fewer, 7.4
+// million rows or more) that the padding would pass it.
+inline int row_pitch(int dim, bool zmarch, int nx, int ny) {
+    const int pad = dim == 2 ? 32 : (zmarch ? 4 : 1), fp = (nx + pad - 1) / pad * pad;
+    return dim == 2 && 9LL * fp * ny > 0x7fffffff ? nx : fp;
 }
 
 }  // namespace lbmwet

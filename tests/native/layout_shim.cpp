@@ -5,6 +5,6 @@
 extern "C" {
 
 int layout_marches(int nx, int ny, int nz) { return lbmwet::ztma_marches(nx, ny, nz); }
-int layout_pitch(int dim, int zmarch, int nx) { return lbmwet::row_pitch(dim, zmarch != 0, nx); }
+int layout_pitch(int dim, int zmarch, int nx, int ny) { return lbmwet::row_pitch(dim, zmarch != 0, nx, ny); }
 
 }  // extern "C"

@@ -44,10 +44,27 @@ def grids_3d():
 def test_3d_offsets_fit_their_type(lib, fp32, kernel):
     for nx, ny, nz in grids_3d():
         march = fp32 and kernel == "auto" and bool(lib.layout_marches(nx, ny, nz))
-        fp = lib.layout_pitch(3, int(march), nx)
+        fp = lib.layout_pitch(3, int(march), nx, ny)
         assert nx <= fp < nx + 4
         if march:
             assert fp % 4 == 0                                   # 64-bit direction offsets; rows TMA can address
             assert fp * ny * nz <= INT_MAX                       # 32-bit within one direction
         else:
             assert 19 * fp * ny * nz <= INT_MAX, (nx, ny, nz)
+
+
+def test_2d_offsets_fit(lib):
+    """Narrow, tall grids (batches, the y-march and the set-up take them) as well as ordinary ones, whose rows
+    stay padded to 32 nodes."""
+    rng = random.Random(8)
+    grids = [(1, LIMIT), (7, LIMIT // 7), (15, LIMIT // 15), (16, LIMIT // 16), (31, LIMIT // 31), (33, LIMIT // 33),
+             (7, 7456540), (7, 7456541), (600, 400), (10630, 10630)]
+    for _ in range(2000):
+        nx = int(2 ** rng.uniform(0, 14))
+        grids.append((nx, max(1, int(LIMIT / nx * rng.choice([1.0, 1.0, rng.random()])))))
+    for nx, ny in grids:
+        assert nx * ny <= LIMIT
+        fp = lib.layout_pitch(2, 0, nx, ny)
+        padded = (nx + 31) // 32 * 32
+        assert 9 * fp * ny <= INT_MAX, (nx, ny)
+        assert fp == (padded if 9 * padded * ny <= INT_MAX else nx)
