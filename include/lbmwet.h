@@ -101,9 +101,9 @@ typedef enum { LBM_BODY_NONE = 0, LBM_BODY_BALL = 1, LBM_BODY_PLANE = 2 } lbm_bo
  *   TMA, two planes in flight; items on planes near a solid also stage node types and do the bounce-back
  *   and virtual-density work; grids below 40 x 16 x 4 nodes run the z-pair march.  PAIR (FP32 only): the
  *   z-pair march, 32 x 4 columns, two planes per thread.  TILE: the scalar z-march; in FP64 (the only
- *   D3Q19 kernel there) bricks sized for the grid.  AUTO: ZTMA in FP32 (PAIR on grids below 40 x 16 x 4
- *   whose rows are not a multiple of 16 bytes), TILE in FP64.  The FP32 kernels agree up to FP32
- *   rounding. */
+ *   D3Q19 kernel there) bricks sized for the grid.  AUTO: ZTMA in FP32, TILE in FP64.  A grid that
+ *   the TMA march does not take steps by PAIR, and lbm_step_kernel_used says so.  The FP32 kernels
+ *   agree up to FP32 rounding. */
 typedef enum { LBM_KERNEL_AUTO = 0, LBM_KERNEL_TILE = 1, LBM_KERNEL_YMARCH = 2, LBM_KERNEL_PAIR = 3,
                LBM_KERNEL_ZTMA = 4 } lbm_step_kernel;
 

@@ -1096,8 +1096,8 @@ int32_t lbm_step_kernel_used(const lbm_handle* h) {
     if (!h) return LBM_KERNEL_AUTO;
     if (h->D == 3) {
         if (h->prec == LBM_FP64 || h->dp.step3 == 2) return LBM_KERNEL_TILE;
-        // (a grid smaller than the march's columns and boxes runs the z-pair march under the same name)
-        return h->dp.step3 == 0 && (h->dp.ztmap || h->cfg.nx % 4 == 0) ? LBM_KERNEL_ZTMA : LBM_KERNEL_PAIR;
+        // (without tensor maps, as on a grid below the march's columns and boxes, the z-pair march runs)
+        return h->dp.ztmap ? LBM_KERNEL_ZTMA : LBM_KERNEL_PAIR;
     }
     if (h->ymarch) return LBM_KERNEL_YMARCH;
     return h->prec == LBM_FP32_DEV && h->dp.pair_solid ? LBM_KERNEL_PAIR : LBM_KERNEL_TILE;
