@@ -23,13 +23,16 @@ __device__ __forceinline__ V2 operator-(V2 a, V2 b) { return fma2(-1.0f, b, a); 
 __device__ __forceinline__ V2 operator-(V2 a) { return -1.0f * a; }
 __device__ __forceinline__ V2 div2(V2 a, V2 b) { return mk(__fdividef(a.v.x, b.v.x), __fdividef(a.v.y, b.v.y)); }
 
-// One FP32 value with the pair's operations, each rounded as a lane of the pair is.
+// One FP32 value with the pair's operations, fused where a pair's are: nvcc contracts a product and a sum to one
+// multiply-add (of pairs too), while a pair's difference is a multiply-add of its own.  With products and sums
+// rounded apart the error against 64 bits after 2 to 22 steps was 3 % larger (rms of density and velocity over
+// 25 runs on 17 grids; as it is, 0.1 % larger and 0.1 % smaller than with pairs).
 struct V1 {
     float v;
 };
-__device__ __forceinline__ V1 operator+(V1 a, V1 b) { return {__fadd_rn(a.v, b.v)}; }
-__device__ __forceinline__ V1 operator*(V1 a, V1 b) { return {__fmul_rn(a.v, b.v)}; }
-__device__ __forceinline__ V1 operator*(float s, V1 b) { return {__fmul_rn(s, b.v)}; }
+__device__ __forceinline__ V1 operator+(V1 a, V1 b) { return {a.v + b.v}; }
+__device__ __forceinline__ V1 operator*(V1 a, V1 b) { return {a.v * b.v}; }
+__device__ __forceinline__ V1 operator*(float s, V1 b) { return {s * b.v}; }
 __device__ __forceinline__ V1 fma2(V1 a, V1 b, V1 c) { return {__fmaf_rn(a.v, b.v, c.v)}; }
 __device__ __forceinline__ V1 fma2(float s, V1 b, V1 c) { return {__fmaf_rn(s, b.v, c.v)}; }
 __device__ __forceinline__ V1 operator-(V1 a, V1 b) { return {__fsub_rn(a.v, b.v)}; }

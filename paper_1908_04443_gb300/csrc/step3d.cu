@@ -215,36 +215,11 @@ __global__ void __launch_bounds__(ZShape<S>::X* ZShape<S>::Y, ZShape<S>::MINB)
 #pragma unroll
                 for (int a = 0; a < Q; ++a) f[a] = sm.f[ring(zc, 3)][a][ly * TX + lx];
                 const int pc = (ly + 1) * PX + lx + 1;
-                const C* p0 = sm.psi[ring(zc, 4)];
-                const C psi_c = p0[pc];
-                C sx = C(0), sy = C(0), sz = C(0);
-#pragma unroll
-                for (int a = 1; a < Q; ++a) {
-                    if (L::opp(a) < a) continue;
-                    const int ex = L::ex(a), ey = L::ey(a), ez = L::ez(a);
-                    const C* pp = sm.psi[ring(zc + ez, 4)];
-                    const C* pm = sm.psi[ring(zc - ez, 4)];
-                    const int off = ex + ey * PX;
-                    const C wd = C(L::wf(a)) * (pp[pc + off] - pm[pc - off]);
-                    if (ex) sx += C(ex) * wd;
-                    if (ey) sy += C(ey) * wd;
-                    if (ez) sz += C(ez) * wd;
-                }
-                const C Fmx = -ph.G * psi_c * sx, Fmy = -ph.G * psi_c * sy, Fmz = -ph.G * psi_c * sz;
-                C drho = C(0), jx = C(0), jy = C(0), jz = C(0);
-#pragma unroll
-                for (int a = 0; a < Q; ++a) {
-                    drho += f[a];
-                    if (L::ex(a)) jx += C(L::ex(a)) * f[a];
-                    if (L::ey(a)) jy += C(L::ey(a)) * f[a];
-                    if (L::ez(a)) jz += C(L::ez(a)) * f[a];
-                }
-                const C rho = ph.rho_ref + drho;
-                C Fx = Fmx + ph.fx, Fy = Fmy + ph.fy, Fz = Fmz + ph.fz;
-                // Eq. 8 (solid-fluid interaction scheme): F_ads = -G_w rho sum_a w_a s(x + e_a) e_a
-                if (solid && ph.wall_kind == 2 && !(t & T_BULK)) {
+                // Eq. 8 (solid-fluid interaction scheme): sum_a w_a s(x + e_a) e_a
+                const bool sf = solid && ph.wall_kind == 2 && !(t & T_BULK);
+                C ax = C(0), ay = C(0), az = C(0);
+                if (sf) {
                     const int tc = (ly + 3) * YX + lx + 3;
-                    C ax = C(0), ay = C(0), az = C(0);
 #pragma unroll
                     for (int a = 1; a < Q; ++a) {
                         const int ex = L::ex(a), ey = L::ey(a), ez = L::ez(a);
@@ -254,24 +229,19 @@ __global__ void __launch_bounds__(ZShape<S>::X* ZShape<S>::Y, ZShape<S>::MINB)
                             if (ez) az += C(L::wf(a) * ez);
                         }
                     }
-                    const C gr = -ph.wall_param * rho;
-                    Fx = (Fmx + gr * ax) + ph.fx;
-                    Fy = (Fmy + gr * ay) + ph.fy;
-                    Fz = (Fmz + gr * az) + ph.fz;
                 }
-                if (!(rho > C(0))) atomicOr(err, ERR_RHO);
-                const C inv = cdiv(C(1), rho);
-                const C ux = (jx + C(0.5) * Fx) * inv, uy = (jy + C(0.5) * Fy) * inv, uz = (jz + C(0.5) * Fz) * inv;
+                auto psi_at = [&](int ex, int ey, int ez) { return sm.psi[ring(zc + ez, 4)][pc + ex + ey * PX]; };
+                const Node3 n = node3([&](int a) { return f[a]; }, psi_at, sf, ax, ay, az, ph, err);
                 if (MODE == 1) {
-                    if (rho_out) rho_out[gi] = double(rho);
+                    if (rho_out) rho_out[gi] = double(n.rho);
                     if (u_out) {
-                        u_out[gi] = double(ux);
-                        u_out[N + gi] = double(uy);
-                        u_out[2 * N + gi] = double(uz);
+                        u_out[gi] = double(n.ux);
+                        u_out[N + gi] = double(n.uy);
+                        u_out[2 * N + gi] = double(n.uz);
                     }
                 } else {
-                    const C X = cdiv(Fmx * Fmx + Fmy * Fmy + Fmz * Fmz, psi_c * psi_c);
-                    collide_d3q19<C>(f, drho, rho, ux, uy, uz, Fx, Fy, Fz, X, ph.r);
+                    const C X = cdiv(n.Fmx * n.Fmx + n.Fmy * n.Fmy + n.Fmz * n.Fmz, n.psi * n.psi);
+                    collide_d3q19<C>(f, n.drho, n.rho, n.ux, n.uy, n.uz, n.Fx, n.Fy, n.Fz, X, ph.r);
 #pragma unroll
                     for (int a = 0; a < Q; ++a) fout[a * fs + zc * fxy + (y0 + ly) * fp + x0 + lx] = S(f[a]);
                 }

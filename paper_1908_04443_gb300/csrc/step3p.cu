@@ -656,6 +656,53 @@ struct ZTOut {
     }
 };
 
+// psi of a density: as the pair kernels' lanes for the step, as the scalar z-march for its fields pass (see node3).
+template <int MODE>
+__device__ __forceinline__ float psi_z(V1 rho, const Phys<float>& ph, unsigned* err) {
+    if constexpr (MODE == 1) return psi_checked(rho.v, ph, err);
+    return psi1(rho, ph, err).v;
+}
+
+// Force (Eqs. 5, 8), velocity (Eq. 4) and MRT collision (Eqs. 2, 7) of a node of the step, f in place.  drho: the
+// sum of f; psi_at(ex, ey, ez): psi at a neighbour; SF: (ax, ay, az) = sum_a w_a s(x + e_a) e_a of Eq. 8.
+template <bool SF, class P>
+__device__ __forceinline__ void march_collide(V1 (&f)[19], V1 drho, P psi_at, float ax, float ay, float az,
+                                              const Phys<float>& ph, const Rates3P& kr, unsigned* err) {
+    using L = D3Q19;
+    const V1 psi_c = {psi_at(0, 0, 0)};
+    V1 sx = {0.0f}, sy = {0.0f}, sz = {0.0f};
+#pragma unroll
+    for (int a = 1; a < 19; ++a) {
+        if (L::opp(a) < a) continue;
+        const int ex = L::ex(a), ey = L::ey(a), ez = L::ez(a);
+        const V1 wd = float(L::wf(a)) * (V1{psi_at(ex, ey, ez)} - V1{psi_at(-ex, -ey, -ez)});
+        if (ex) sx = ex > 0 ? sx + wd : sx - wd;
+        if (ey) sy = ey > 0 ? sy + wd : sy - wd;
+        if (ez) sz = ez > 0 ? sz + wd : sz - wd;
+    }
+    // Eq. 5
+    const V1 gpsi = (-ph.G) * psi_c;
+    const V1 Fmx = gpsi * sx, Fmy = gpsi * sy, Fmz = gpsi * sz;
+    V1 Fx = Fmx + V1{ph.fx}, Fy = Fmy + V1{ph.fy}, Fz = Fmz + V1{ph.fz};
+    const V1 jx = ((f[1] - f[2]) + (f[7] - f[8])) + ((f[9] - f[10]) + (f[11] - f[12])) + (f[13] - f[14]);
+    const V1 jy = ((f[3] - f[4]) + (f[7] - f[8])) + ((f[10] - f[9]) + (f[15] - f[16])) + (f[17] - f[18]);
+    const V1 jz = ((f[5] - f[6]) + (f[11] - f[12])) + ((f[14] - f[13]) + (f[15] - f[16])) + (f[18] - f[17]);
+    const V1 rho = V1{ph.rho_ref} + drho;
+    // Eq. 8: F_ads = -G_w rho (ax, ay, az)
+    if constexpr (SF) {
+        const V1 gr = (-ph.wall_param) * rho;
+        Fx = (Fmx + gr * V1{ax}) + V1{ph.fx};
+        Fy = (Fmy + gr * V1{ay}) + V1{ph.fy};
+        Fz = (Fmz + gr * V1{az}) + V1{ph.fz};
+    }
+    if (!(rho.v > 0.0f)) atomicOr(err, ERR_RHO);
+    // Eq. 4: rho u = sum e f + F/2
+    const V1 inv = div2(V1{1.0f}, rho);
+    const V1 ux = fma2(0.5f, Fx, jx) * inv, uy = fma2(0.5f, Fy, jy) * inv, uz = fma2(0.5f, Fz, jz) * inv;
+    const V1 X = div2(fma2(Fmx, Fmx, fma2(Fmy, Fmy, Fmz * Fmz)), psi_c * psi_c);
+    collide3p(f, drho, rho, ux, uy, uz, Fx, Fy, Fz, X, kr);
+}
+
 // A chunk without solids within 3 nodes: no walls, no bounce-back; lag 1 between the lead plane
 // and the collided plane.
 template <int MODE>
@@ -747,12 +794,12 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
         V1 dcur = fcur[0];
 #pragma unroll
         for (int a = 1; a < Q; ++a) dcur = dcur + fcur[a];
-        S.psi[zl & 3][pc] = psi1(V1{ph.rho_ref} + dcur, ph, err).v;
+        S.psi[zl & 3][pc] = psi_z<MODE>(V1{ph.rho_ref} + dcur, ph, err);
         if (ringer) {
             V1 d = {pulled(st, 0, rx, ry)};
 #pragma unroll
             for (int a = 1; a < Q; ++a) d = d + V1{pulled(st, a, rx, ry)};
-            S.psi[zl & 3][ry * TPX + rx] = psi1(V1{ph.rho_ref} + d, ph, err).v;
+            S.psi[zl & 3][ry * TPX + rx] = psi_z<MODE>(V1{ph.rho_ref} + d, ph, err);
         }
         __syncthreads();
         if (lx == 0 && zl + BST <= zhi) issue(zl + BST, s);
@@ -765,39 +812,12 @@ __device__ __forceinline__ void ztma_chunk_bulk(const float* __restrict__ fin, f
         const int zc = zl - 1;
         if (zc >= zb) {
             V1(&f)[Q] = fprev;
-            auto psi_at = [&](int dz, int off) {
-                return V1{S.psi[(zc + dz) & 3][pc + off]};
-            };
-            const V1 psi_c = psi_at(0, 0);
-            V1 sx = {0.0f}, sy = {0.0f}, sz = {0.0f};
-#pragma unroll
-            for (int a = 1; a < Q; ++a) {
-                if (L::opp(a) < a) continue;
-                const int ex = L::ex(a), ey = L::ey(a), ez = L::ez(a);
-                const int off = ex + ey * TPX;
-                const V1 wd = float(L::wf(a)) * (psi_at(ez, off) - psi_at(-ez, -off));
-                if (ex) sx = ex > 0 ? sx + wd : sx - wd;
-                if (ey) sy = ey > 0 ? sy + wd : sy - wd;
-                if (ez) sz = ez > 0 ? sz + wd : sz - wd;
-            }
-            // Eq. 5
-            const V1 gpsi = (-ph.G) * psi_c;
-            const V1 Fmx = gpsi * sx, Fmy = gpsi * sy, Fmz = gpsi * sz;
-            const V1 Fx = Fmx + V1{ph.fx}, Fy = Fmy + V1{ph.fy}, Fz = Fmz + V1{ph.fz};
-            const V1 drho = dprev;
-            const V1 jx = ((f[1] - f[2]) + (f[7] - f[8])) + ((f[9] - f[10]) + (f[11] - f[12])) + (f[13] - f[14]);
-            const V1 jy = ((f[3] - f[4]) + (f[7] - f[8])) + ((f[10] - f[9]) + (f[15] - f[16])) + (f[17] - f[18]);
-            const V1 jz = ((f[5] - f[6]) + (f[11] - f[12])) + ((f[14] - f[13]) + (f[15] - f[16])) + (f[18] - f[17]);
-            const V1 rho = V1{ph.rho_ref} + drho;
-            if (!(rho.v > 0.0f)) atomicOr(err, ERR_RHO);
-            // Eq. 4: rho u = sum e f + F/2
-            const V1 inv = div2(V1{1.0f}, rho);
-            const V1 ux = fma2(0.5f, Fx, jx) * inv, uy = fma2(0.5f, Fy, jy) * inv, uz = fma2(0.5f, Fz, jz) * inv;
+            auto psi_at = [&](int ex, int ey, int ez) { return S.psi[(zc + ez) & 3][pc + ex + ey * TPX]; };
             if constexpr (MODE == 1) {
-                if (wr) out.node((zc * ny + y0 + ly) * nx + x0 + lx, rho.v, ux.v, uy.v, uz.v);
+                const Node3 n = node3([&](int a) { return f[a].v; }, psi_at, false, 0.0f, 0.0f, 0.0f, ph, err);
+                if (wr) out.node((zc * ny + y0 + ly) * nx + x0 + lx, n.rho, n.ux, n.uy, n.uz);
             } else {
-                const V1 X = div2(fma2(Fmx, Fmx, fma2(Fmy, Fmy, Fmz * Fmz)), psi_c * psi_c);
-                collide3p(f, drho, rho, ux, uy, uz, Fx, Fy, Fz, X, kr);
+                march_collide<false>(f, dprev, psi_at, 0.0f, 0.0f, 0.0f, ph, kr, err);
                 const unsigned o = unsigned(zc * fxy + (y0 + ly) * fp + x0 + lx);
                 if (wr) {
 #pragma unroll
@@ -933,14 +953,15 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
             float v[Q];
             const uint8_t t = ty[tcl];
             const bool fl = !(t & T_SOLID);
-            V1 rho = {0.0f}, ps = {0.0f};
+            V1 rho = {0.0f};
+            float ps = 0.0f;
             if (fl) {
                 pull(st, stn, zl, ly + 2, lx + 4, t, v);
                 dcur = V1{v[0]};
 #pragma unroll
                 for (int a = 1; a < Q; ++a) dcur = dcur + V1{v[a]};
                 rho = V1{ph.rho_ref} + dcur;
-                ps = psi1(rho, ph, err);
+                ps = psi_z<MODE>(rho, ph, err);
             } else {
 #pragma unroll
                 for (int a = 0; a < Q; ++a) v[a] = 0.0f;
@@ -948,7 +969,7 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
 #pragma unroll
             for (int a = 0; a < Q; ++a) fcur[a].v = v[a];
             rr[rc] = rho.v;
-            pp[pc] = ps.v;
+            pp[pc] = ps;
         }
         // halo cells: the 1-node ring (density and psi) and the 2-node ring (density)
         for (int k = NT - 1 - tid; k < TRING + TRING2; k += NT) {   // (the first threads patch the edges)
@@ -974,7 +995,7 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
                 rho = (V1{ph.rho_ref} + d).v;
             }
             rr[rb * TRX + c - 2] = rho;
-            if (k < TRING) pp[(rb - 1) * TPX + c - 3] = fl ? psi1(V1{rho}, ph, err).v : 0.0f;
+            if (k < TRING) pp[(rb - 1) * TPX + c - 3] = fl ? psi_z<MODE>(V1{rho}, ph, err) : 0.0f;
         }
         __syncthreads();
         if (lx == 0 && zl + 2 <= zhi) issue(zl + 2, s);
@@ -1011,7 +1032,7 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
                     rw = raw > ph.rho_l ? ph.rho_l : raw;
                     rw = rw < ph.rho_g ? ph.rho_g : rw;
                 }
-                S.psi[ps5(zw)][k] = psi1(V1{rw}, ph, err).v;
+                S.psi[ps5(zw)][k] = psi_z<MODE>(V1{rw}, ph, err);
             }
         }
 #pragma unroll
@@ -1032,33 +1053,9 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
             }
             if (fl) {
                 V1(&f)[Q] = f2;
-                auto psi_at = [&](int dz, int off) {
-                    return V1{S.psi[ps5(zc + dz)][pc + off]};
-                };
-                const V1 psi_c = psi_at(0, 0);
-                V1 sx = {0.0f}, sy = {0.0f}, sz = {0.0f};
-#pragma unroll
-                for (int a = 1; a < Q; ++a) {
-                    if (L::opp(a) < a) continue;
-                    const int ex = L::ex(a), ey = L::ey(a), ez = L::ez(a);
-                    const int off = ex + ey * TPX;
-                    const V1 wd = float(L::wf(a)) * (psi_at(ez, off) - psi_at(-ez, -off));
-                    if (ex) sx = ex > 0 ? sx + wd : sx - wd;
-                    if (ey) sy = ey > 0 ? sy + wd : sy - wd;
-                    if (ez) sz = ez > 0 ? sz + wd : sz - wd;
-                }
-                // Eq. 5
-                const V1 gpsi = (-ph.G) * psi_c;
-                const V1 Fmx = gpsi * sx, Fmy = gpsi * sy, Fmz = gpsi * sz;
-                V1 Fx = Fmx + V1{ph.fx}, Fy = Fmy + V1{ph.fy}, Fz = Fmz + V1{ph.fz};
-                const V1 drho = d2;
-                const V1 jx = ((f[1] - f[2]) + (f[7] - f[8])) + ((f[9] - f[10]) + (f[11] - f[12])) + (f[13] - f[14]);
-                const V1 jy = ((f[3] - f[4]) + (f[7] - f[8])) + ((f[10] - f[9]) + (f[15] - f[16])) + (f[17] - f[18]);
-                const V1 jz = ((f[5] - f[6]) + (f[11] - f[12])) + ((f[14] - f[13]) + (f[15] - f[16])) + (f[18] - f[17]);
-                const V1 rho = V1{ph.rho_ref} + drho;
-                // Eq. 8 (solid-fluid interaction scheme): F_ads = -G_w rho sum_a w_a s(x + e_a) e_a
+                // Eq. 8 (solid-fluid interaction scheme): sum_a w_a s(x + e_a) e_a
+                float ax = 0.0f, ay = 0.0f, az = 0.0f;
                 if constexpr (SF) {
-                    float ax = 0.0f, ay = 0.0f, az = 0.0f;
 #pragma unroll
                     for (int a = 1; a < Q; ++a) {
                         const int ex = L::ex(a), ey = L::ey(a), ez = L::ez(a);
@@ -1069,20 +1066,14 @@ __device__ __forceinline__ void ztma_chunk_solid(const float* __restrict__ fin, 
                             if (ez) az += w * float(ez);
                         }
                     }
-                    const V1 gr = (-ph.wall_param) * rho;
-                    Fx = (Fmx + gr * V1{ax}) + V1{ph.fx};
-                    Fy = (Fmy + gr * V1{ay}) + V1{ph.fy};
-                    Fz = (Fmz + gr * V1{az}) + V1{ph.fz};
                 }
-                if (!(rho.v > 0.0f)) atomicOr(err, ERR_RHO);
-                // Eq. 4: rho u = sum e f + F/2
-                const V1 inv = div2(V1{1.0f}, rho);
-                const V1 ux = fma2(0.5f, Fx, jx) * inv, uy = fma2(0.5f, Fy, jy) * inv, uz = fma2(0.5f, Fz, jz) * inv;
+                auto psi_at = [&](int ex, int ey, int ez) { return S.psi[ps5(zc + ez)][pc + ex + ey * TPX]; };
                 if constexpr (MODE == 1) {
-                    if (in) out.node(zc * nxy + (y0 + ly) * nx + x0 + lx, rho.v, ux.v, uy.v, uz.v);
+                    const Node3 n = node3([&](int a) { return f[a].v; }, psi_at, SF && !(tc[tcl] & T_BULK), ax, ay, az,
+                                          ph, err);
+                    if (in) out.node(zc * nxy + (y0 + ly) * nx + x0 + lx, n.rho, n.ux, n.uy, n.uz);
                 } else {
-                    const V1 X = div2(fma2(Fmx, Fmx, fma2(Fmy, Fmy, Fmz * Fmz)), psi_c * psi_c);
-                    collide3p(f, drho, rho, ux, uy, uz, Fx, Fy, Fz, X, kr);
+                    march_collide<SF>(f, d2, psi_at, ax, ay, az, ph, kr, err);
                     const unsigned o = unsigned(zc * fxy + (y0 + ly) * fp + x0 + lx);
                     if (in) {
 #pragma unroll

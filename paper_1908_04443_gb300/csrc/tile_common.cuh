@@ -200,6 +200,61 @@ __device__ __forceinline__ C psi_checked(C rho, const Phys<C>& e, unsigned* err)
     return csqrt(arg);
 }
 
+// F_m (Eq. 5), F = F_m + F_body + F_ads (Eq. 8 with the solid-fluid interaction scheme: sf, (ax, ay, az) =
+// sum_a w_a s(x + e_a) e_a) and u (Eq. 4) of a D3Q19 node in FP32, shared by the scalar z-march and by the fields
+// pass of the TMA march so that both round alike (the additions to F_m explicitly: which of them are fused
+// depends on the code around them otherwise).  f(a): the distributions; psi(ex, ey, ez): psi at a neighbour.
+struct Node3 {
+    float rho, drho, psi, Fmx, Fmy, Fmz, Fx, Fy, Fz, ux, uy, uz;
+};
+template <class F, class P>
+__device__ __forceinline__ Node3 node3(F f, P psi, bool sf, float ax, float ay, float az, const Phys<float>& ph,
+                                       unsigned* err) {
+    using L = D3Q19;
+    Node3 n;
+    n.psi = psi(0, 0, 0);
+    float sx = 0.0f, sy = 0.0f, sz = 0.0f;
+#pragma unroll
+    for (int a = 1; a < L::Q; ++a) {
+        if (L::opp(a) < a) continue;
+        const int ex = L::ex(a), ey = L::ey(a), ez = L::ez(a);
+        const float wd = float(L::wf(a)) * (psi(ex, ey, ez) - psi(-ex, -ey, -ez));
+        if (ex) sx += float(ex) * wd;
+        if (ey) sy += float(ey) * wd;
+        if (ez) sz += float(ez) * wd;
+    }
+    const float gpsi = __fmul_rn(-ph.G, n.psi);
+    n.Fmx = __fmul_rn(gpsi, sx);
+    n.Fmy = __fmul_rn(gpsi, sy);
+    n.Fmz = __fmul_rn(gpsi, sz);
+    float jx = 0.0f, jy = 0.0f, jz = 0.0f;
+    n.drho = 0.0f;
+#pragma unroll
+    for (int a = 0; a < L::Q; ++a) {
+        n.drho += f(a);
+        if (L::ex(a)) jx += float(L::ex(a)) * f(a);
+        if (L::ey(a)) jy += float(L::ey(a)) * f(a);
+        if (L::ez(a)) jz += float(L::ez(a)) * f(a);
+    }
+    n.rho = ph.rho_ref + n.drho;
+    if (sf) {   // F_ads = -G_w rho (ax, ay, az)
+        const float gr = __fmul_rn(-ph.wall_param, n.rho);
+        n.Fx = __fadd_rn(__fmaf_rn(gr, ax, n.Fmx), ph.fx);
+        n.Fy = __fadd_rn(__fmaf_rn(gr, ay, n.Fmy), ph.fy);
+        n.Fz = __fadd_rn(__fmaf_rn(gr, az, n.Fmz), ph.fz);
+    } else {
+        n.Fx = __fmaf_rn(gpsi, sx, ph.fx);
+        n.Fy = __fmaf_rn(gpsi, sy, ph.fy);
+        n.Fz = __fmaf_rn(gpsi, sz, ph.fz);
+    }
+    if (!(n.rho > 0.0f)) atomicOr(err, ERR_RHO);
+    const float inv = cdiv(1.0f, n.rho);
+    n.ux = __fmul_rn(__fmaf_rn(0.5f, n.Fx, jx), inv);
+    n.uy = __fmul_rn(__fmaf_rn(0.5f, n.Fy, jy), inv);
+    n.uz = __fmul_rn(__fmaf_rn(0.5f, n.Fz, jz), inv);
+    return n;
+}
+
 // The k-th cell of the one-cell-thick shell of an AX x AY (x AZ) box, enumerated so that
 // consecutive k are neighbouring cells (warps stay coherent).
 template <int AX, int AY, int AZ, int D>
