@@ -95,9 +95,8 @@ typedef enum { LBM_BODY_NONE = 0, LBM_BODY_BALL = 1, LBM_BODY_PLANE = 2 } lbm_bo
  *   has chosen one.  A y-march handle that records a trajectory for the adjoint steps with TILE
  *   from lbm_record on.
  * D3Q19 (every kernel marches z-planes through 32-plane chunks of x-y columns):
- *   ZTMA (FP32 only): 32 x 8 columns cut along z into work items, one CTA per item (those of
- *   lbm_d3q19_work_list, except that columns cut by the grid's edge are moved inside it and that small
- *   grids are cut into shorter items); the lead plane's 19 pull boxes are staged in shared memory by
+ *   ZTMA (FP32 only): 32 x 8 columns cut along z into work items, one CTA per item (see
+ *   lbm_d3q19_launch_list); the lead plane's 19 pull boxes are staged in shared memory by
  *   TMA, two planes in flight; items on planes near a solid also stage node types and do the bounce-back
  *   and virtual-density work; grids below 40 x 16 x 4 nodes run the z-pair march.  PAIR (FP32 only): the
  *   z-pair march, 32 x 4 columns, two planes per thread.  TILE: the scalar z-march; in FP64 (the only
@@ -292,14 +291,34 @@ lbm_status lbm_grid_shape(const lbm_handle* h, int32_t* shape4);
 /* Number of kernel launches this handle has issued (step kernels and others), for accounting. */
 int64_t lbm_kernel_launches(const lbm_handle* h);
 
-/* The work list of the TMA-staged D3Q19 z-march (LBM_KERNEL_ZTMA) for a solid mask: host code only
- * (no device, no handle), the list lbm_init builds for an FP32 D3Q19 handle on that kernel where every
- * column is full and the grid fills the GPU (else see lbm_step_kernel).  One
- * time step (Eqs. 1-7 with the Eq. 16-17 walls) is split into items, one CTA each: item i is the 5
+/* The work items of one launch of the TMA-staged D3Q19 z-march (LBM_KERNEL_ZTMA) for a solid mask on a GPU
+ * that holds `slots` of its CTAs at a time (two per SM): host code only (no device, no handle), the list
+ * lbm_init builds for an FP32 D3Q19 handle on that kernel.  One time step (Eqs. 1-7 with the Eq. 16-17
+ * walls) is split into items, one CTA each, in the order of their launch: item i is the 5 int32 values
+ * items[5i .. 5i+4] = {bx, by, z0, z1, solid}: the nodes x in [32 bx, 32 bx + 32), y in [8 by, 8 by + 8)
+ * of the grid on planes z0 <= z < z1, and solid = 1 where the item takes the path for planes near a solid
+ * (node types, bounce-back, virtual densities).  Every (column, plane) lies in exactly one item.  A column
+ * cut by the grid's far edge is worked on as the 32 x 8 block whose first node is (x0, y0), moved inside
+ * the grid: x0 = nx - 32 rounded up to a multiple of 4, y0 = ny - 8 (cells beyond the grid are its periodic
+ * images); it writes its own nodes only.  Planes within 3 planes of one with a solid within 3 nodes of the
+ * block, periodic in every axis, are always on the solid path.
+ *   Grids that fill the GPU twice over with items of 32 planes: runs of planes on one path cut at the
+ *   multiples of 32 planes (pieces of at most 46 planes, as a first or last one of fewer than 8 joins its
+ *   neighbour; runs of fewer than 8 bulk planes join the solid path), in ascending z0, by, bx, the bulk
+ *   pieces of 8 planes or more that begin in the last layer of 32 planes cut in four and put at the end.
+ *   Smaller ones: near-equal pieces of lengths chosen for the number of slots, those on the solid path first
+ *   (runs of fewer than 4 bulk planes join it).
+ * Arguments and errors as for lbm_d3q19_work_list below, and LBM_ERR_ARG for slots < 1 and for grids below
+ * 40 x 16 x 4 nodes, which the z-pair march steps. */
+lbm_status lbm_d3q19_launch_list(const uint8_t* solid_mask, int32_t nx, int32_t ny, int32_t nz, int32_t slots,
+                                 int32_t* items, int64_t capacity, int64_t* count);
+
+/* A cut of a grid's columns into items of about 32 planes, whatever the GPU: host code only.  It names the planes
+ * that need the solid path; the items that a launch runs are those of lbm_d3q19_launch_list.  Item i is the 5
  * int32 values items[5i .. 5i+4] = {bx, by, z0, z1, solid}: the column of cells x in [32 bx,
  * 32 bx + 32), y in [8 by, 8 by + 8) (clipped to the grid), planes z0 <= z < z1, and solid = 1 where
- * the item takes the path for planes within 3 planes of a solid near the column (node types,
- * bounce-back, virtual densities) or, for a column cut by the grid's edge, the z-pair march.  Every
+ * the item holds planes within 3 planes of a solid near the column or, with planes cut at the multiples of 32,
+ * for a column cut by the grid's edge and for grids below 64 x 16 x 4 nodes.  Every
  * (column, plane) lies in exactly one item; items run in ascending z0, then by, then bx.
  *   solid_mask: host, nz*ny*nx bytes (x fastest), nonzero = solid; read only during the call.
  *   items: host array of 5 * capacity int32, owned by the caller, or NULL to ask for the count.

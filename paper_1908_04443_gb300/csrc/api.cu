@@ -1846,12 +1846,14 @@ lbm_status lbm_grid_shape(const lbm_handle* h, int32_t* shape4) {
     return LBM_OK;
 }
 
-lbm_status lbm_d3q19_work_list(const uint8_t* solid_mask, int32_t nx, int32_t ny, int32_t nz, int32_t* items,
-                               int64_t capacity, int64_t* count) {
+static lbm_status list_checks(const uint8_t* solid_mask, int32_t nx, int32_t ny, int32_t nz, const int64_t* count) {
     if (!solid_mask || !count) return fail(nullptr, LBM_ERR_ARG, "null argument");
     if (nx < 1 || ny < 1 || nz < 1) return fail(nullptr, LBM_ERR_ARG, "grid sizes must be >= 1");
     if ((long long)nx * ny * nz > (1LL << 31) / 19) return fail(nullptr, LBM_ERR_ARG, "grid too large");
-    const std::vector<ZItem> v = ztma_work_list(solid_mask, nx, ny, nz);
+    return LBM_OK;
+}
+
+static lbm_status list_out(const std::vector<ZItem>& v, int32_t* items, int64_t capacity, int64_t* count) {
     *count = (int64_t)v.size();
     if (!items) return LBM_OK;
     if (capacity < (int64_t)v.size()) return fail(nullptr, LBM_ERR_ARG, "capacity below the item count");
@@ -1864,6 +1866,22 @@ lbm_status lbm_d3q19_work_list(const uint8_t* solid_mask, int32_t nx, int32_t ny
         o[4] = v[i].solid;
     }
     return LBM_OK;
+}
+
+lbm_status lbm_d3q19_launch_list(const uint8_t* solid_mask, int32_t nx, int32_t ny, int32_t nz, int32_t slots,
+                                 int32_t* items, int64_t capacity, int64_t* count) {
+    const lbm_status st = list_checks(solid_mask, nx, ny, nz, count);
+    if (st != LBM_OK) return st;
+    if (slots < 1) return fail(nullptr, LBM_ERR_ARG, "slots must be >= 1");
+    if (!ztma_marches(nx, ny, nz)) return fail(nullptr, LBM_ERR_ARG, "the z-march takes grids from 40 x 16 x 4 nodes");
+    return list_out(ztma_items(solid_mask, nx, ny, nz, slots), items, capacity, count);
+}
+
+lbm_status lbm_d3q19_work_list(const uint8_t* solid_mask, int32_t nx, int32_t ny, int32_t nz, int32_t* items,
+                               int64_t capacity, int64_t* count) {
+    const lbm_status st = list_checks(solid_mask, nx, ny, nz, count);
+    if (st != LBM_OK) return st;
+    return list_out(ztma_work_list(solid_mask, nx, ny, nz), items, capacity, count);
 }
 
 lbm_handle* lbm_batch_handle(lbm_batch* b, int32_t i) {

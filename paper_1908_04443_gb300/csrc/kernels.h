@@ -173,18 +173,17 @@ void d3q19_fp64_brick(int nx, int ny, int nz, int sms, int* bw, int* bh, int* bz
 // D3Q19 FP32 step as a z-pair march (two planes per thread, packed FP32x2 arithmetic); chunk flags
 // g.tile_solid per FP32 z-march chunk.
 cudaError_t launch_zpair_step(const void* fin, void* fout, const Geo& g, const DevParams& p, cudaStream_t s);
-// D3Q19 FP32 step, TMA-staged z-march over 32 x 8 columns of 32-plane chunks (ragged columns and
-// small grids take the z-pair march); tmap: the tensor map of fin (dimensions x, y, 19 nz; box
-// bx x by x 1, see ztma_box_dims), 128 bytes.
+// D3Q19 FP32 step, TMA-staged z-march over the items p.zitems; tmap: the tensor maps of fin (dimensions x, y,
+// 19 nz; boxes bx x by x 1, see ztma_maps), 128 bytes each.
 cudaError_t launch_ztma_step(const void* fin, void* fout, const void* tmap, const Geo& g, const DevParams& p,
                              cudaStream_t s);
 // Box (columns, rows) of tensor map k of a buffer; returns the number of maps, which lie behind one another.
 int ztma_maps(int k, int* bx, int* by);
-// Work list of the TMA-staged z-march for a grid with solid mask `mask` (host, nx*ny*nz bytes):
+// The cut of lbm_d3q19_work_list for a grid with solid mask `mask` (host, nx*ny*nz bytes; no launch runs it):
 // every boxed 32 x 8 column cut along z into runs that need the solid path and runs that do not
 // (bulk runs shorter than 8 planes join the solid path), each run cut at the multiples of 32 planes
-// (a first or last piece shorter than 8 planes joins its neighbour); the other columns as the z-pair
-// march's 32-plane chunks; ordered by first plane, then column.
+// (a first or last piece shorter than 8 planes joins its neighbour); the other columns as 32-plane
+// chunks; ordered by first plane, then column.
 std::vector<ZItem> ztma_work_list(const uint8_t* mask, int nx, int ny, int nz);
 // The items a handle's launch runs, for `slots` resident CTAs: every column on the march (the last ones moved
 // inside the grid), and shorter pieces where the grid would not fill the chip.  Only for grids that the march

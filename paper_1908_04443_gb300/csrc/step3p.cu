@@ -1250,7 +1250,7 @@ std::vector<ZItem> column_runs(const uint8_t* mask, int nx, int ny, int nz, int 
 
 // Runs cut at the multiples of 32 planes, so that items of neighbouring columns start on the same planes and
 // share their halo reads in L2; a first or last piece shorter than LBMWET_ZWL_MIN_RUN joins its neighbour
-// (items of up to 39 planes).
+// (items of up to 46 planes, where both do).
 std::vector<ZItem> aligned_items(const std::vector<ZItem>& runs, std::vector<ZItem> items) {
     constexpr int MIN_RUN = LBMWET_ZWL_MIN_RUN;
     for (const ZItem& r : runs) {
