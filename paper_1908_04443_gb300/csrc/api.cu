@@ -540,14 +540,14 @@ std::vector<uint8_t> merged_flags(const lbm_handle* h, int w, int th) {
     return out;
 }
 
-// The mask scan for a validated configuration: the step kernels' tile shape and, for D2Q9 in FP32,
-// the pair kernel's.
+// The mask scan for a validated configuration: for D2Q9 with the flags of the step kernels' tiles and, in FP32,
+// the pair kernel's (D3Q19: init_impl scans for those of the kernel that the grid takes).
 void scan_for(const lbm_config& c, const uint8_t* solid_mask, int threads, MaskScan* out) {
     int t[3], tp[2];
     step_tile_shape(c.lattice, c.precision, &t[0], &t[1], &t[2]);
-    const bool pair = c.lattice == LBM_D2Q9 && c.precision == LBM_FP32_DEV;
+    const bool d2 = c.lattice == LBM_D2Q9, pair = d2 && c.precision == LBM_FP32_DEV;
     if (pair) pair_tile_shape(&tp[0], &tp[1]);
-    scan_mask(solid_mask, c.nx, c.ny, c.nz, c.lattice == LBM_D2Q9 ? 2 : 3, t, pair ? tp : nullptr, threads, out);
+    scan_mask(solid_mask, c.nx, c.ny, c.nz, d2 ? 2 : 3, d2 ? t : nullptr, pair ? tp : nullptr, threads, out);
 }
 
 // lbm_init with the mask scan done by the caller (`pre`, consumed) or here, and with or without the
@@ -660,26 +660,28 @@ lbm_status init_impl(const lbm_config* cfg, const uint8_t* solid_mask, const dou
         }
     }
     CKI(dmalloc(&h->d_type, N, h->stream), "cudaMalloc type");
-    // (FP64: followed by the flags of the grid's FP64 tiles)
-    std::vector<uint8_t> flags = h->tile_solid;
+    // solid flags: D2Q9 those of the step kernels' tiles, in FP64 followed by the grid's FP64 tiles'; D3Q19 those
+    // of the kernel that steps the grid (FP64 bricks; chunks of the z-pair and scalar marches; the TMA march has
+    // its work list instead)
     int fw = 0, fh = 0, fz = 1;
-    if (h->prec == LBM_FP64) {
-        std::vector<uint8_t> own;
-        if (h->D == 2) {
-            d2q9_fp64_tile(&nx, &ny, 1, device_sms(), &fw, &fh);
-            own = merged_flags(h, fw, fh);
-        } else {
-            // (a brick is much smaller than the 32-plane chunks of tile_solid, and a flagged one costs more
-            // halo planes: its own scan)
-            d3q19_fp64_brick(nx, ny, nz, device_sms(), &fw, &fh, &fz);
-            const int t[3] = {fw, fh, fz};
-            own = tile_solid_flags(solid_mask, nx, ny, nz, t, 3, scan_threads(N));
-        }
-        flags.insert(flags.end(), own.begin(), own.end());
+    std::vector<uint8_t> own;
+    if (h->prec == LBM_FP64 && h->D == 2) {
+        d2q9_fp64_tile(&nx, &ny, 1, device_sms(), &fw, &fh);
+        own = merged_flags(h, fw, fh);
+    } else if (h->prec == LBM_FP64) {
+        d3q19_fp64_brick(nx, ny, nz, device_sms(), &fw, &fh, &fz);
+        const int t[3] = {fw, fh, fz};
+        own = tile_solid_flags(solid_mask, nx, ny, nz, t, 3, scan_threads(N));
+    } else if (h->D == 3 && zmaps.empty()) {
+        h->tile_solid = tile_solid_flags(solid_mask, nx, ny, nz, h->int_tile, 3, scan_threads(N));
     }
-    CKI(dmalloc(&h->d_tile_solid, flags.size(), h->stream), "cudaMalloc tile flags");
-    CKI(cudaMemcpyAsync(h->d_tile_solid, flags.data(), flags.size(), cudaMemcpyHostToDevice, h->stream),
-        "copy tile flags");
+    std::vector<uint8_t> flags = h->tile_solid;
+    flags.insert(flags.end(), own.begin(), own.end());
+    if (!flags.empty()) {
+        CKI(dmalloc(&h->d_tile_solid, flags.size(), h->stream), "cudaMalloc tile flags");
+        CKI(cudaMemcpyAsync(h->d_tile_solid, flags.data(), flags.size(), cudaMemcpyHostToDevice, h->stream),
+            "copy tile flags");
+    }
     CKI(dmalloc(&h->d_wall_id, sizeof(int) * N, h->stream), "cudaMalloc wall_id");
     CKI(dmalloc(&h->d_err, sizeof(unsigned), h->stream), "cudaMalloc err");
     const size_t nw = h->wall_nodes.size();

@@ -164,7 +164,7 @@ int ymarch_ctas_per_sm(int prec);
 struct Geo;
 cudaError_t launch_step3d(int prec, int mode, const void* fin, void* fout, const Geo& g, const DevParams& p,
                           double* rho, double* u, cudaStream_t s);
-void zmarch_tile_shape(int prec, int* tx, int* ty, int* tz);
+void zmarch_tile_shape(int* tx, int* ty, int* tz);
 // D3Q19 FP64: the step (mode 0) or the fields (mode 1) on bricks of p.tile_w x p.tile_h x p.tile_z nodes with
 // the flags p.pair_solid; and the brick for a grid on `sms` SMs.
 cudaError_t launch_d3q19_fp64(int mode, const void* fin, void* fout, const Geo& g, const DevParams& p, double* rho,

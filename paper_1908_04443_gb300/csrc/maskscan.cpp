@@ -142,7 +142,8 @@ void scan_mask(const uint8_t* mask, int nx, int ny, int nz, int D, const int t[3
     out->nfluid = N - ns;
     out->wall_nodes.resize(nw);
     parallel_for(nt, nt, [&](int k) { std::copy(part[k].begin(), part[k].end(), out->wall_nodes.begin() + off[k]); });
-    out->tile_solid = tile_solid_flags(mask, nx, ny, nz, t, D, nt);
+    if (t) out->tile_solid = tile_solid_flags(mask, nx, ny, nz, t, D, nt);
+    else out->tile_solid.clear();
     if (pair_t) {
         const int tp[3] = {pair_t[0], pair_t[1], 1};
         out->pair_solid = tile_solid_flags(mask, nx, ny, nz, tp, 2, nt);

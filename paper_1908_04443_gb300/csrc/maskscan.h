@@ -22,8 +22,8 @@ std::vector<uint8_t> tile_solid_flags(const uint8_t* mask, int nx, int ny, int n
                                       int threads = 1);
 
 // The full scan: fluid count, wall list (neighbourhood of the D2Q9 or D3Q19 velocity set,
-// periodic wrap), the step-kernel tile flags for tile shape t and, when pair_t is given, the pair
-// kernel's.  `threads` > 1 splits the rows over that many threads.
+// periodic wrap) and, when t and pair_t are given, the step-kernel tile flags for tile shape t and the
+// pair kernel's.  `threads` > 1 splits the rows over that many threads.
 void scan_mask(const uint8_t* mask, int nx, int ny, int nz, int D, const int t[3], const int* pair_t, int threads,
                MaskScan* out);
 

@@ -911,7 +911,7 @@ void step_tile_shape(int lat, int prec, int* tx, int* ty, int* tz) {
         if (prec == PREC_FP64) { *tx = TileShape<D2Q9, double>::X; *ty = TileShape<D2Q9, double>::Y; *tz = 1; }
         else { *tx = TileShape<D2Q9, float>::X; *ty = TileShape<D2Q9, float>::Y; *tz = 1; }
     } else {
-        zmarch_tile_shape(prec, tx, ty, tz);
+        zmarch_tile_shape(tx, ty, tz);   // (FP64: d3q19_fp64_brick)
     }
 }
 

@@ -46,7 +46,6 @@ struct ZShape;
 template <> struct ZShape<float> {
     static constexpr int X = LBMWET_Z3F_X, Y = LBMWET_Z3F_Y, Z = LBMWET_Z3F_Z, MINB = LBMWET_Z3F_MINB;
 };
-template <> struct ZShape<double> { static constexpr int X = 32, Y = 4, Z = 32; };   // flags only (FP64: step3d64.cu)
 
 template <class S, class C, int MODE>
 __global__ void __launch_bounds__(ZShape<S>::X* ZShape<S>::Y, ZShape<S>::MINB)
@@ -278,16 +277,10 @@ cudaError_t launch_z(const void* fin, void* fout, const Geo& g, const DevParams&
 
 }  // namespace
 
-void zmarch_tile_shape(int prec, int* tx, int* ty, int* tz) {
-    if (prec == PREC_FP64) {
-        *tx = ZShape<double>::X;
-        *ty = ZShape<double>::Y;
-        *tz = ZShape<double>::Z;
-    } else {
-        *tx = ZShape<float>::X;
-        *ty = ZShape<float>::Y;
-        *tz = ZShape<float>::Z;
-    }
+void zmarch_tile_shape(int* tx, int* ty, int* tz) {
+    *tx = ZShape<float>::X;
+    *ty = ZShape<float>::Y;
+    *tz = ZShape<float>::Z;
 }
 
 cudaError_t launch_step3d(int prec, int mode, const void* fin, void* fout, const Geo& g, const DevParams& p,

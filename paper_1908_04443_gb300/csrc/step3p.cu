@@ -1220,14 +1220,12 @@ std::vector<ZItem> column_runs(const uint8_t* mask, int nx, int ny, int nz, int 
             // planes within 3 planes (periodic) of a plane with a solid near the column's cells; a column moved
             // inside the grid also covers cells of its left and lower neighbours
             const int bx0 = bx * TTX + TTX > nx && bx > 0 ? bx - 1 : bx, by0 = by * TTY + TTY > ny && by > 0 ? by - 1 : by;
+            std::fill(need.begin(), need.end(), uint8_t(0));
             for (int z = 0; z < nz; ++z) {
                 uint8_t n = 0;
-                for (int d = -HALO; d <= HALO && !n; ++d) {
-                    const int zz = ((z + d) % nz + nz) % nz;
-                    for (int cy = by0; cy <= by; ++cy)
-                        for (int cx = bx0; cx <= bx; ++cx) n |= col[((size_t)zz * gy + cy) * gx + cx];
-                }
-                need[z] = n;
+                for (int cy = by0; cy <= by; ++cy)
+                    for (int cx = bx0; cx <= bx; ++cx) n |= col[((size_t)z * gy + cy) * gx + cx];
+                for (int d = -HALO; n && d <= HALO; ++d) need[((z + d) % nz + nz) % nz] = 1;
             }
             // runs of equal need; short bulk runs join the solid path
             std::vector<ZItem> runs;
