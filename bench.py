@@ -45,10 +45,10 @@ UNIT = "MLUPS"
 # of the kernel code: when the code changes the figure is stale and reported as null.
 NCU_TRAFFIC = {
     # pair_step_batched, 600 x 400 sweep of 24 grids: dram__bytes_read.sum + dram__bytes_write.sum of
-    # one launch (215.38 + 153.15 MB as ncu prints them)
-    ("c2", "fp32", "054e40c8e439c43c"): 368530000,
+    # one launch
+    ("c2", "fp32", "6a403a0e20dafb8c"): 374299904,
     # ztma_step, 256^3 sphere: one launch
-    ("c3", "fp32", "1645287eb60ebe95"): 2811863552,
+    ("c3", "fp32", "dacc8f5429e6fca9"): 2802910464,
 }
 
 
@@ -56,7 +56,7 @@ NCU_TRAFFIC = {
 # 600 x 400 sweep, from ncu: (2 x DFMA + DADD + DMUL thread instructions of one launch) / nodes =
 # (2 x 217,849,056 + 371,237,280 + 169,225,560) / 5,760,000; keyed by a hash of the kernel's code.
 FP64_FLOPS_PER_NODE = {
-    ("c2", "1f132e5983c80437"): 169.47,
+    ("c2", "bb787547f4ebd7ba"): 169.47,
 }
 # FP64 peak of a GB300 from its unit counts and clock: 1.25 TFLOP/s nominal is 4 FP64 flops (2 FMA) per
 # SM per clock at 2.07 GHz, so 152 SMs x 4 x 2.07 GHz = 1258.6 GFLOP/s.

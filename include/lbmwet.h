@@ -350,10 +350,11 @@ lbm_status lbm_record(lbm_handle* h, int64_t n_steps, int64_t ckpt_every);
 /* dL/dkappa for the trajectory of the last lbm_record, whose final state must still be the
  * handle's state (else LBM_ERR_STATE).  drho_final_dev: DEVICE array of N doubles, dL/drho_T at
  * every node (ignored at solid nodes).  dkappa_host: host array, one double per wall node in
- * lbm_wall_nodes() order.  Recomputes each checkpoint segment's states, then runs the reverse
- * sweep (each segment replayed as a CUDA graph); allocates ckpt_every + 2 distribution buffers and 19 N
- * scalars of scratch for the
- * call.  Synchronises the stream. */
+ * lbm_wall_nodes() order.  Recomputes each checkpoint segment's states beside the reverse sweep of the one
+ * after it; allocates ckpt_every + 2 distribution buffers for the call (2 ckpt_every + 2 with more than one
+ * segment) and, in FP64, 16 N doubles of scratch.  Up to 1 GiB in all they come from the memory pool, which
+ * keeps them (lbm_release_cached_memory returns them); larger ones go back to the driver when the call
+ * returns.  Synchronises the stream. */
 lbm_status lbm_adjoint(lbm_handle* h, const double* drho_final_dev, double* dkappa_host);
 
 /* ---- Batches (no counterpart in the paper: many independent grids of one physics) ----------

@@ -502,7 +502,7 @@ __global__ void __launch_bounds__(TileShape<L, S>::X* TileShape<L, S>::Y* TileSh
 
 // The fields pass of several grids (a batch's observables) in one launch.  A launch per grid leaves
 // most of the chip idle: a grid of 600 x 400 is 950 tiles, 1.6 waves of 4 CTAs per SM, and its tail and
-// start-up are most of its 8.6 us.  24 such grids: 206 us one by one, 59 us together.
+// start-up are most of its 8.6 us.  24 such grids: 206 us one by one, 113 us together.
 __global__ void __launch_bounds__(TileShape<D2Q9, float>::X* TileShape<D2Q9, float>::Y, TileShape<D2Q9, float>::MINB)
     fields_grids(const FieldGrid* __restrict__ tab, int n, Phys<float> ph) {
     using S = float;

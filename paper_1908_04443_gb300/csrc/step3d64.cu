@@ -7,8 +7,8 @@
 // Bound by the FP64 pipe (fp64.cuh), as in 2D: a plane of 16 x 8 nodes keeps it busy for 20,000 clocks, so
 // the second pull costs nothing beside it, and what counts is FP64 instructions and an equal share of
 // them for every SM, with several bricks on each to hide one another's latency.  d3q19_fp64_brick weighs
-// the halo's share (36 instructions a cell against 283 a node) against both.  A 64^3 step: 812 us in
-// 32 x 4 x 32 bricks on 64 of 152 SMs with the general functions, 230 us here.
+// the halo's share (36 instructions a cell against 283 a node) against both.  A 64^3 step: 789 us in
+// 32 x 4 x 32 bricks on 64 of 152 SMs with the general functions, 206 us here.
 #include "fp64.cuh"
 #include "kernels.h"
 #include "lattice.cuh"

@@ -1097,15 +1097,15 @@ __host__ __device__ __forceinline__ bool ztma_boxed(int x0, int y0, int nx, int 
     return x0 + TTX <= nx && y0 + TTY <= ny && nx >= 64 && ny >= 16 && nz >= 4;
 }
 
-// Bound by the instructions of a plane (256^3: issue slots 69 % busy at 26 warp instructions a node, DRAM at 79 %
-// of the copy rate): a table of the boxes in shared memory, the density's sum carried to the collision, and stores at a uniform
-// base plus one 32-bit offset took 256^3 from 541 to 502 us a step, 200 x 200 x 280 from 406 to 383, 97 x 83 x 75 from
-// 55.6 to 52.0.
+// Bound by DRAM with its over-read (256^3: 83 % of the copy rate) and by the instructions of a plane (issue slots
+// 63 % busy at 23 warp instructions a node; 69 % at 26 before a table of the boxes in shared memory, the density's
+// sum carried to the collision, and stores at a uniform base plus one 32-bit offset took 256^3 from 541 to 500 us
+// a step, 200 x 200 x 280 from 406 to 381, 97 x 83 x 75 from 55.6 to 51.4).
 // One CTA per item.  The last column of a grid whose width is not a multiple of 32 (8 in y) is moved inside
 // the grid, as far as the boxes' 16-byte boundary allows: up to 3 of its columns then lie beyond x = nx - 1
 // and hold periodic images, patched like the halo.  It writes only the nodes that no full column owns.  (Such
 // columns went to the z-pair march on narrow blocks before: the 200 x 200 x 280 grid, one column in seven,
-// took 561 us a step, 383 us now.)
+// took 561 us a step, 381 us now.)
 template <int MODE>
 __global__ void __launch_bounds__(TNT, 2)
     ztma_step(const float* __restrict__ fin, float* __restrict__ fout, const void* tmap, Geo g, Phys<float> ph,

@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(NT, 2) fields64_grids(const FieldGrid* __restr
 // the fullest SM decides; beyond that tiles are handed out as SMs get free and half a tile is the tail.
 // Fitted to 14 shapes on 4 grids (100 x 100 to
 // 1000 x 1000): it picks a shape within 5 % of the fastest on each, 8 x 10 (10.9 us a step) for 100 x 100,
-// 32 x 12 for 300 x 350 (34.6 us; 32 x 16 takes 44.9), 16 x 16 for 600 x 400 (67.8 us; 32 x 16 takes 78.9).
+// 32 x 12 for 300 x 350 (34.6 us; 32 x 16 takes 44.9), 16 x 14 for 600 x 400 (68 us; 32 x 16 takes 78.9).
 void d2q9_fp64_tile(const int* nx, const int* ny, int ngrids, int sms, int* tw, int* th) {
     auto warps = [](int n) { return double((n + 31) / 32 * 32); };
     double best = 1e300;

@@ -148,7 +148,7 @@ inline PairGrid pair_grid(const void* fin, const void* fout, const DevParams& p)
     return g;
 }
 
-// Division in compute precision: FP64 keeps IEEE division (parity with the FP64 oracle); the FP32
+// Division in compute precision: IEEE in FP64 (the adjoint; the FP64 steps have fp64.cuh); the FP32
 // path uses the fast hardware approximation (relative error of a few ulp, below the rounding of the
 // FP32 state).
 __device__ __forceinline__ float cdiv(float a, float b) { return __fdividef(a, b); }
